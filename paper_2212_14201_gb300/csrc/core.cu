@@ -112,6 +112,32 @@ size_t workspace_bytes(int n) {
   return std::max(sampler, std::max(reduce, hist)) + 4096;
 }
 
+int take_scratch(qs_state* s, size_t bytes, ScratchBuf* out, bool keep) {
+  constexpr size_t kKeep = (size_t)256 << 20;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  QS_CUDA(cudaStreamIsCapturing(s->stream, &cap));
+  if (!keep || bytes > kKeep || s->scratch_used || cap != cudaStreamCaptureStatusNone) {
+    QS_CUDA(dmalloc_async(&out->p, bytes, s->stream));
+    out->pooled = true;
+    out->pool = s->stream;
+    return QS_OK;
+  }
+  if (s->scratch_bytes < bytes) {
+    if (s->scratch) {
+      QS_CUDA(cudaStreamSynchronize(s->stream));
+      cudaFree(s->scratch);
+    }
+    s->scratch = nullptr;
+    s->scratch_bytes = 0;
+    QS_CUDA(dmalloc(&s->scratch, bytes));
+    s->scratch_bytes = bytes;
+  }
+  out->p = s->scratch;
+  out->kept = s;
+  s->scratch_used = true;
+  return QS_OK;
+}
+
 int ensure_pinned(qs_state* s, size_t bytes) {
   if (s->pinned_bytes >= bytes) return QS_OK;
   if (s->pinned) cudaFreeHost(s->pinned);
@@ -445,6 +471,7 @@ extern "C" int qs_free(qs_state* s) {
   if (!s) return QS_OK;
   cudaStreamSynchronize(s->stream);
   if (s->owns && s->amps) cudaFree(s->amps);
+  if (s->scratch) cudaFree(s->scratch);
   if (s->ws) cudaFree(s->ws);
   if (s->pinned) cudaFreeHost(s->pinned);
   if (s->tables) cudaFree(s->tables);

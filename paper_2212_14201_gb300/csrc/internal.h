@@ -40,6 +40,10 @@ struct qs_state {
   bool timing = false;
   std::vector<qs_pending_timing> pending;
   std::vector<cudaEvent_t> event_pool;
+  // Temporaries of one call (ScratchBuf), kept between calls.
+  void* scratch = nullptr;
+  size_t scratch_bytes = 0;
+  bool scratch_used = false;
   // Phase tables of tile passes: device copy, pinned staging, and the event of the
   // last upload (the staging buffer is rewritten only after that copy ran).
   void* tables = nullptr;
@@ -200,6 +204,22 @@ struct KTimer {
 
 // ---- workspace ------------------------------------------------------------------
 size_t workspace_bytes(int n);
+// Device memory for the length of one call on the state's stream.  Up to 256 MiB
+// comes from a buffer that the state keeps (the driver's pool gives freed memory
+// back at every synchronisation, so an allocation per call costs 80 us and more);
+// more than that, with keep = false (sizes a state should not hold on to), or under
+// stream capture, where a graph must own its memory, from the stream's pool.
+struct ScratchBuf {
+  void* p = nullptr;
+  qs_state* kept = nullptr;  // the state whose buffer it is (one at a time)
+  cudaStream_t pool = nullptr;
+  bool pooled = false;
+  ~ScratchBuf() {
+    if (pooled) cudaFreeAsync(p, pool);
+    if (kept) kept->scratch_used = false;
+  }
+};
+int take_scratch(qs_state* s, size_t bytes, ScratchBuf* out, bool keep = true);
 int ensure_pinned(qs_state* s, size_t bytes);
 
 }  // namespace qs

@@ -4,8 +4,8 @@
 // Section "Variational quantum circuit").
 //
 // Every reduction is deterministic: per-thread partials are combined by a fixed
-// warp-shuffle tree, CTA partials go to the workspace in CTA order and one
-// final CTA adds them in that order.  Results do not depend on timing.
+// warp-shuffle tree, CTA partials go to the workspace in CTA order and a finishing
+// kernel adds them in a fixed order.  Results do not depend on timing.
 #include <algorithm>
 #include <map>
 #include <mutex>
@@ -68,50 +68,98 @@ __global__ void k_probs_full(const T* __restrict__ a, double* __restrict__ p, ui
   for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < N; i += stride) p[i] = prob(ld_amp(a, i));
 }
 
-// ---- marginal over nq <= 12 qubits: per-CTA shared histogram ---------------------
 struct MargArgs {
   uint64_t N;
   int nq;
   int q[12];
 };
 
-__device__ __forceinline__ uint32_t extract_bits(uint64_t x, const MargArgs& g) {
-  uint32_t k = 0;
-  for (int j = 0; j < g.nq; ++j) k |= (uint32_t)((x >> g.q[j]) & 1) << j;
-  return k;
-}
+// ---- marginal over any listed qubits, FP64 ------------------------------------------
+// The index is read as (rest | listed high bits | lane): a lane is one of the 32
+// amplitudes of a row (qubits 0..4), a warp keeps the listed qubits >= 5 fixed at kh
+// and walks the rows of its chunk of the other qubits.  Every lane then adds to one
+// register sum per unrolled row, whatever nq is, and the row reads stay 512 bytes
+// long; the lanes that differ only in unlisted qubits are added once at the end.
+// (A shared histogram needs the 32 lanes added one after the other to be
+// deterministic: 64 shuffles and 32 dependent shared-memory additions per row.)
+// Bound by the FP64 pipe: two FMAs per amplitude, as k_norm2.
+struct MargRowArgs {
+  uint64_t units;              // warps of work: 2^hq * chunks
+  uint64_t rows;               // rows per unit, 2^(n - 5 - hq) / chunks
+  uint64_t H;                  // 2^nq outputs
+  uint64_t restmask;           // row bits (x >> 5) of the unlisted qubits >= 5
+  int n, hq, nrest;
+  int lowkey[5];               // output bit of lane bit b, or -1
+  int hbit[QS_MAX_QUBITS];     // listed qubits >= 5: row bit (ascending) ...
+  int hkey[QS_MAX_QUBITS];     // ... and output bit
+};
 
-// Each CTA owns a contiguous range of the state; a thread accumulates its own
-// elements into a shared histogram with shared-memory atomics would make the sum
-// order timing-dependent, so instead each warp owns a private histogram slice
-// and adds its lanes' values in lane order.
 template <class T>
-__global__ void __launch_bounds__(256) k_marginal_small(const T* __restrict__ a, double* __restrict__ part,
-                                                         const MargArgs g, uint64_t per_cta) {
-  extern __shared__ double hist[];  // [8 warps][2^nq]
-  const int H = 1 << g.nq;
-  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-  for (int i = threadIdx.x; i < 8 * H; i += blockDim.x) hist[i] = 0.0;
-  __syncthreads();
-  uint64_t begin = blockIdx.x * per_cta, end = min(g.N, begin + per_cta);
-  double* mine = hist + w * H;
-  for (uint64_t base = begin + (uint64_t)w * 32; base < end; base += 256) {
-    uint64_t x = base + l;
-    double p = x < end ? prob(ld_amp(a, x)) : 0.0;
-    uint32_t k = extract_bits(x, g);
-    // lanes add in lane order (deterministic)
-    for (int src = 0; src < 32; ++src) {
-      double ps = __shfl_sync(0xffffffffu, p, src);
-      uint32_t ks = __shfl_sync(0xffffffffu, k, src);
-      if (l == 0 && base + src < end) mine[ks] += ps;
+__global__ void __launch_bounds__(256) k_marginal_rows(const T* __restrict__ a, double* __restrict__ part,
+                                                       const MargRowArgs g) {
+  const uint64_t unit = blockIdx.x * (uint64_t)8 + (threadIdx.x >> 5);
+  if (unit >= g.units) return;
+  const uint32_t lane = threadIdx.x & 31;
+  const uint64_t kh = unit & ((1ull << g.hq) - 1), chunk = unit >> g.hq;
+  uint64_t fixed = 0, key = 0;
+  for (int j = 0; j < g.hq; ++j)
+    if ((kh >> j) & 1) {
+      fixed |= 1ull << g.hbit[j];
+      key |= 1ull << g.hkey[j];
+    }
+  // deposit the chunk's first rest index into the unlisted row bits
+  uint64_t r = 0, src = chunk * g.rows, m = g.restmask;
+  for (int j = 0; j < g.nrest; ++j) {
+    const uint64_t low = m & (0 - m);
+    if ((src >> j) & 1) r |= low;
+    m ^= low;
+  }
+  auto next = [&] { r = ((r | ~g.restmask) + 1) & g.restmask; };  // increment over the unlisted bits
+  const T* row = a + lane;
+  double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
+  uint64_t k = 0;
+  for (; k + 4 <= g.rows; k += 4) {  // four independent loads and sums in flight
+    const uint64_t x0 = (r | fixed) << 5;
+    next();
+    const uint64_t x1 = (r | fixed) << 5;
+    next();
+    const uint64_t x2 = (r | fixed) << 5;
+    next();
+    const uint64_t x3 = (r | fixed) << 5;
+    next();
+    const double2 v0 = ld_amp(row, x0), v1 = ld_amp(row, x1), v2 = ld_amp(row, x2), v3 = ld_amp(row, x3);
+    s0 = acc_prob(v0, s0);
+    s1 = acc_prob(v1, s1);
+    s2 = acc_prob(v2, s2);
+    s3 = acc_prob(v3, s3);
+  }
+  for (; k < g.rows; ++k) {
+    s0 = acc_prob(ld_amp(row, (r | fixed) << 5), s0);
+    next();
+  }
+  double v = (s0 + s1) + (s2 + s3);
+  bool writer = true;
+#pragma unroll
+  for (int b = 0; b < 5; ++b) {
+    if (g.lowkey[b] < 0) {
+      v += __shfl_xor_sync(0xffffffffu, v, 1 << b);
+      writer = writer && !((lane >> b) & 1);
+    } else if ((lane >> b) & 1) {
+      key |= 1ull << g.lowkey[b];
     }
   }
-  __syncthreads();
-  for (int i = threadIdx.x; i < H; i += blockDim.x) {
-    double s = 0.0;
-    for (int ww = 0; ww < 8; ++ww) s += hist[ww * H + i];
-    part[(size_t)blockIdx.x * H + i] = s;
-  }
+  if (writer) part[chunk * g.H + key] = v;
+}
+
+// out[k] = part[0][k] + part[1][k] + ... : one warp per output, then a fixed tree
+__global__ void __launch_bounds__(256) k_marginal_rows_finish(const double* __restrict__ part, uint64_t chunks,
+                                                              uint64_t H, double* __restrict__ out) {
+  const uint64_t k = blockIdx.x * (uint64_t)8 + (threadIdx.x >> 5);
+  if (k >= H) return;
+  double s = 0.0;
+  for (uint64_t c = threadIdx.x & 31; c < chunks; c += 32) s += part[c * H + k];
+  s = warp_sum(s);
+  if ((threadIdx.x & 31) == 0) out[k] = s;
 }
 
 // Marginal over nq <= 3 qubits (a measured qubit, a few bits): every thread keeps
@@ -216,22 +264,47 @@ __global__ void __launch_bounds__(256) k_marginal_exact(const T* __restrict__ a,
   }
 }
 
-__global__ void k_exact_finish(const uint64_t* __restrict__ part, int nblocks, int H, double* __restrict__ out) {
-  for (int i = threadIdx.x; i < H; i += blockDim.x) {
-    u128 t = 0;
-    for (int b = 0; b < nblocks; ++b)
-      t += ((u128)part[((size_t)b * H + i) * 2 + 1] << 64) | part[((size_t)b * H + i) * 2];
+// Sum over the 256 threads of a CTA, valid in thread 0 (sh: one slot per warp).
+__device__ __forceinline__ u128 block_sum_u128(u128 v, uint64_t (*sh)[2]) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += shfl_xor_u128(v, o);
+  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+  __syncthreads();
+  if (l == 0) {
+    sh[w][0] = (uint64_t)v;
+    sh[w][1] = (uint64_t)(v >> 64);
+  }
+  __syncthreads();
+  u128 t = 0;
+  if (threadIdx.x == 0)
+    for (int i = 0; i < 8; ++i) t += ((u128)sh[i][1] << 64) | sh[i][0];
+  return t;
+}
+
+__device__ __forceinline__ u128 ld_u128(const uint64_t* p) { return ((u128)p[1] << 64) | p[0]; }
+
+// The finishers take one CTA per output, its threads striding over the CTA partials:
+// one thread adding a thousand partials in turn waits for L2 on every one.
+__global__ void __launch_bounds__(256) k_exact_finish(const uint64_t* __restrict__ part, int nblocks, int H,
+                                                      double* __restrict__ out) {
+  __shared__ uint64_t sh[8][2];
+  u128 t = 0;
+  for (int b = threadIdx.x; b < nblocks; b += 256) t += ld_u128(part + ((size_t)b * H + blockIdx.x) * 2);
+  t = block_sum_u128(t, sh);
+  if (threadIdx.x == 0) {
     const double v = (double)(uint64_t)(t >> 64) * 18446744073709551616.0 + (double)(uint64_t)t;
-    out[i] = v * 0x1p-120;
+    out[blockIdx.x] = v * 0x1p-120;
   }
 }
 
-__global__ void k_marginal_finish(const double* __restrict__ part, int nblocks, int H, double* __restrict__ out) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < H; i += gridDim.x * blockDim.x) {
-    double s = 0.0;
-    for (int b = 0; b < nblocks; ++b) s += part[(size_t)b * H + i];
-    out[i] = s;
-  }
+// one CTA per output; each thread's partials in CTA order, then the fixed tree
+__global__ void __launch_bounds__(256) k_marginal_finish(const double* __restrict__ part, int nblocks, int H,
+                                                         double* __restrict__ out) {
+  __shared__ double sh[8];
+  double s = 0.0;
+  for (int b = threadIdx.x; b < nblocks; b += 256) s += part[(size_t)b * H + blockIdx.x];
+  s = block_sum256(s, sh);
+  if (threadIdx.x == 0) out[blockIdx.x] = s;
 }
 
 // ---- marginal over many qubits: one thread per output entry -----------------------
@@ -382,37 +455,44 @@ __global__ void __launch_bounds__(256, 3) k_expect_z_exact(const A* __restrict__
   }
 }
 
-// out[i] = T - 2 S_i from the exact CTA partials (bits >= r: CTA index bits).
-__global__ void k_expect_z_exact_finish(const uint64_t* __restrict__ part, int nblocks, int r, int n,
-                                        double* __restrict__ out) {
-  const int i = threadIdx.x;
-  if (i >= n) return;
+// out[i] = T - 2 S_i from the exact CTA partials (bits >= r: CTA index bits), CTA i
+// of this kernel for qubit i.
+__global__ void __launch_bounds__(256) k_expect_z_exact_finish(const uint64_t* __restrict__ part, int nblocks, int r,
+                                                               double* __restrict__ out) {
+  __shared__ uint64_t sh[8][2];
+  const int i = blockIdx.x;
   u128 T = 0, S = 0;
-  for (int c = 0; c < nblocks; ++c) {
+  for (int c = threadIdx.x; c < nblocks; c += 256) {
     const uint64_t* o = part + (size_t)c * (r + 1) * 2;
-    const u128 t = ((u128)o[1] << 64) | o[0];
+    const u128 t = ld_u128(o);
     T += t;
-    if (i < r) S += ((u128)o[2 * (1 + i) + 1] << 64) | o[2 * (1 + i)];
+    if (i < r) S += ld_u128(o + 2 * (1 + i));
     else if ((c >> (i - r)) & 1) S += t;
   }
+  T = block_sum_u128(T, sh);
+  S = block_sum_u128(S, sh);
+  if (threadIdx.x) return;
   const bool neg = T < 2 * S;  // T - 2S may be negative
   const u128 m = neg ? 2 * S - T : T - 2 * S;
   const double d = (double)(uint64_t)(m >> 64) * 18446744073709551616.0 + (double)(uint64_t)m;
   out[i] = (neg ? -d : d) * 0x1p-120;
 }
 
-__global__ void k_expect_z_finish(const double* __restrict__ part, int nblocks, int r, int n, double* __restrict__ out) {
-  // out[i] = T - 2 S_i; thread i handles qubit i; CTA partials added in CTA order.
-  int i = threadIdx.x;
-  if (i >= n) return;
+// The same from the FP64 partials: each thread's CTAs in order, then the fixed tree.
+__global__ void __launch_bounds__(256) k_expect_z_finish(const double* __restrict__ part, int nblocks, int r,
+                                                         double* __restrict__ out) {
+  __shared__ double sh[8];
+  const int i = blockIdx.x;
   double T = 0.0, S = 0.0;
-  for (int c = 0; c < nblocks; ++c) {
+  for (int c = threadIdx.x; c < nblocks; c += 256) {
     const double* o = part + (size_t)c * (r + 1);
     T += o[0];
     if (i < r) S += o[1 + i];
     else if ((c >> (i - r)) & 1) S += o[0];
   }
-  out[i] = T - 2.0 * S;
+  T = block_sum256(T, sh);
+  S = block_sum256(S, sh);
+  if (threadIdx.x == 0) out[i] = T - 2.0 * S;
 }
 
 // ---- Pauli terms ------------------------------------------------------------------------
@@ -638,15 +718,18 @@ __global__ void __launch_bounds__(256, 3) k_pauli_tile(const A* __restrict__ a, 
   }
 }
 
-// sums[slot0 + k] = the CTA partials of slot k added (modulo 2^128)
-__global__ void k_pauli_exact_finish(const uint64_t* __restrict__ part, int nblocks, int nt, uint64_t* __restrict__ sums) {
-  const int k = threadIdx.x;
-  if (k >= nt) return;
+// sums[k] = the CTA partials of slot k added (modulo 2^128), CTA k of this kernel
+__global__ void __launch_bounds__(256) k_pauli_exact_finish(const uint64_t* __restrict__ part, int nblocks,
+                                                            uint64_t* __restrict__ sums) {
+  __shared__ uint64_t sh[8][2];
+  const int k = blockIdx.x;
   u128 t = 0;
-  for (int b = 0; b < nblocks; ++b)
-    t += ((u128)part[((size_t)b * PS_MAX + k) * 2 + 1] << 64) | part[((size_t)b * PS_MAX + k) * 2];
-  sums[2 * k] = (uint64_t)t;
-  sums[2 * k + 1] = (uint64_t)(t >> 64);
+  for (int b = threadIdx.x; b < nblocks; b += 256) t += ld_u128(part + ((size_t)b * PS_MAX + k) * 2);
+  t = block_sum_u128(t, sh);
+  if (threadIdx.x == 0) {
+    sums[2 * k] = (uint64_t)t;
+    sums[2 * k + 1] = (uint64_t)(t >> 64);
+  }
 }
 
 }  // namespace qs
@@ -659,6 +742,50 @@ static int read_back(qs_state* s, const double* dev, size_t count, double* host)
   QS_CUDA(cudaStreamSynchronize(s->stream));
   memcpy(host, s->pinned, count * sizeof(double));
   return QS_OK;
+}
+
+// The chunks a warp's listed values are split into: enough warps to fill the GPU
+// (kWarps, twice what 152 SMs hold), at least 8 rows a warp, and partial sums that
+// fit the workspace.
+static int marginal_rows(qs_state* s, const int* qubits, int nq, double* dout) {
+  MargRowArgs g{};
+  g.n = s->n;
+  g.H = 1ull << nq;
+  for (int b = 0; b < 5; ++b) g.lowkey[b] = -1;
+  uint64_t used = 0;
+  int key_of[QS_MAX_QUBITS];
+  for (int j = 0; j < nq; ++j) {
+    used |= 1ull << qubits[j];
+    key_of[qubits[j]] = j;
+  }
+  for (int b = 0; b < s->n; ++b) {
+    if (!((used >> b) & 1)) {
+      if (b >= 5) g.restmask |= 1ull << (b - 5), ++g.nrest;
+    } else if (b < 5) {
+      g.lowkey[b] = key_of[b];
+    } else {
+      g.hbit[g.hq] = b - 5;
+      g.hkey[g.hq++] = key_of[b];
+    }
+  }
+  constexpr uint64_t kWarps = 2 * 152 * 64;
+  uint64_t chunks = 1;
+  while ((chunks << g.hq) < kWarps && (chunks << 4) <= (1ull << g.nrest) &&
+         2 * chunks * g.H * sizeof(double) <= s->ws_bytes)
+    chunks <<= 1;
+  g.units = chunks << g.hq;
+  g.rows = (1ull << g.nrest) / chunks;
+  double* part = chunks > 1 ? (double*)s->ws : dout;
+  with_amps(s, [&](auto* a) {
+    using T = std::remove_cv_t<std::remove_pointer_t<decltype(a)>>;
+    k_marginal_rows<T><<<(unsigned)((g.units + 7) / 8), 256, 0, s->stream>>>(a, part, g);
+    return QS_OK;
+  });
+  QS_TRY(launch_check("marginal_rows"));
+  if (chunks == 1) return QS_OK;
+  note_launch(1);
+  k_marginal_rows_finish<<<(unsigned)((g.H + 7) / 8), 256, 0, s->stream>>>(part, chunks, g.H, dout);
+  return launch_check("marginal_rows finish");
 }
 
 static int marginal_device(qs_state* s, const int* qubits, int nq, double* dout, bool allow_exact = true) {
@@ -694,7 +821,7 @@ static int marginal_device(qs_state* s, const int* qubits, int nq, double* dout,
       return QS_OK;
     });
     QS_TRY(launch_check("marginal_exact"));
-    k_exact_finish<<<1, 32, 0, s->stream>>>(part, nblocks, 1 << nq, dout);
+    k_exact_finish<<<1 << nq, 256, 0, s->stream>>>(part, nblocks, 1 << nq, dout);
     return launch_check("marginal_exact finish");
   }
   if (nq == 0) {  // squared norm: per-thread sums, a fixed shuffle tree, CTA partials in order
@@ -705,7 +832,7 @@ static int marginal_device(qs_state* s, const int* qubits, int nq, double* dout,
       return QS_OK;
     });
     QS_TRY(launch_check("norm2"));
-    k_marginal_finish<<<1, 32, 0, s->stream>>>(part, nblocks, 1, dout);
+    k_marginal_finish<<<1, 256, 0, s->stream>>>(part, nblocks, 1, dout);
     return launch_check("norm2 finish");
   }
   if (nq <= 3) {
@@ -727,32 +854,10 @@ static int marginal_device(qs_state* s, const int* qubits, int nq, double* dout,
     });
     QS_TRY(launch_check("marginal_tiny"));
     const int H = 1 << nq;
-    k_marginal_finish<<<1, 32, 0, s->stream>>>(part, nblocks, H, dout);
+    k_marginal_finish<<<H, 256, 0, s->stream>>>(part, nblocks, H, dout);
     return launch_check("marginal_finish");
   }
-  if (nq <= 10) {  // 8 warp-private histograms of 2^nq doubles fit in shared memory
-    MargArgs g;
-    g.N = N;
-    g.nq = nq;
-    for (int j = 0; j < nq; ++j) g.q[j] = qubits[j];
-    int nblocks = (int)std::min<uint64_t>(304, std::max<uint64_t>(1, N / 256));
-    uint64_t per = (N + nblocks - 1) / nblocks;
-    per = (per + 255) / 256 * 256;
-    nblocks = (int)((N + per - 1) / per);
-    size_t smem = (size_t)8 * (1 << nq) * sizeof(double);
-    double* part = (double*)s->ws;
-    QS_TRY(with_amps(s, [&](auto* a) {
-      using T = std::remove_cv_t<std::remove_pointer_t<decltype(a)>>;
-      if (smem > 48 * 1024)
-        QS_CUDA(cudaFuncSetAttribute(k_marginal_small<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-      k_marginal_small<<<nblocks, 256, smem, s->stream>>>((const T*)a, part, g, per);
-      return QS_OK;
-    }));
-    QS_TRY(launch_check("marginal_small"));
-    int H = 1 << nq;
-    k_marginal_finish<<<(H + 255) / 256, 256, 0, s->stream>>>(part, nblocks, H, dout);
-    return launch_check("marginal_finish");
-  }
+  if (n >= 5) return marginal_rows(s, qubits, nq, dout);
   MargBigArgs g;
   g.nq = nq;
   g.H = 1ull << nq;
@@ -789,17 +894,13 @@ namespace qs {
 // kernels (relative accuracy for tiny probabilities, where the exact integer form
 // is only accurate to 2^-45 absolute).
 int marginal_host(qs_state* s, const int* qubits, int nq, double* out, bool allow_exact) {
-  size_t H = (size_t)1 << nq;
-  double* tmp = nullptr;
-  QS_CUDA(dmalloc_async(&tmp, H * sizeof(double), s->stream));
-  int rc = marginal_device(s, qubits, nq, tmp, allow_exact);
-  if (rc == QS_OK) {
-    cudaError_t e = cudaMemcpyAsync(out, tmp, H * sizeof(double), cudaMemcpyDeviceToHost, s->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
-    if (e != cudaSuccess) rc = cuda_fail(e, "probs readback");
-  }
-  cudaFreeAsync(tmp, s->stream);
-  return rc;
+  const size_t bytes = sizeof(double) << nq;
+  ScratchBuf tmp;
+  QS_TRY(take_scratch(s, bytes, &tmp, nq < s->n));  // the whole distribution: half a state
+  QS_TRY(marginal_device(s, qubits, nq, (double*)tmp.p, allow_exact));
+  cudaError_t e = cudaMemcpyAsync(out, tmp.p, bytes, cudaMemcpyDeviceToHost, s->stream);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
+  return e == cudaSuccess ? QS_OK : cuda_fail(e, "probs readback");
 }
 }  // namespace qs
 
@@ -809,18 +910,8 @@ extern "C" int qs_probs(const qs_state* cs, const int* qubits, int nq, double* o
   QS_TRY(check_state(s));
   QS_TRY(check_qubit_list(s, qubits, nq));
   if (!out) return fail(QS_ERR_INVALID_ARG, "out is NULL");
-  size_t H = (size_t)1 << nq;
   if (on_device) return marginal_device(s, qubits, nq, out);
-  double* tmp = nullptr;
-  QS_CUDA(dmalloc_async(&tmp, H * sizeof(double), s->stream));
-  int rc = marginal_device(s, qubits, nq, tmp);
-  if (rc == QS_OK) {
-    cudaError_t e = cudaMemcpyAsync(out, tmp, H * sizeof(double), cudaMemcpyDeviceToHost, s->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
-    if (e != cudaSuccess) rc = cuda_fail(e, "probs readback");
-  }
-  cudaFreeAsync(tmp, s->stream);
-  return rc;
+  return marginal_host(s, qubits, nq, out, true);
 }
 
 extern "C" int qs_probs_dict(const qs_state* cs, const int* qubits, int nq, double threshold, uint64_t* idx,
@@ -889,7 +980,7 @@ extern "C" int qs_expect_z_all(const qs_state* cs, double* out) {
       return QS_OK;
     });
     QS_TRY(launch_check("expect_z"));
-    k_expect_z_exact_finish<<<1, 64, 0, s->stream>>>(ipart, nblocks, r, n, dres);
+    k_expect_z_exact_finish<<<n, 256, 0, s->stream>>>(ipart, nblocks, r, dres);
     QS_TRY(launch_check("expect_z_finish"));
     return read_back(s, dres, n, out);
   }
@@ -902,7 +993,7 @@ extern "C" int qs_expect_z_all(const qs_state* cs, double* out) {
     return QS_OK;
   });
   QS_TRY(launch_check("expect_z"));
-  k_expect_z_finish<<<1, 64, 0, s->stream>>>(part, nblocks, r, n, dres);
+  k_expect_z_finish<<<n, 256, 0, s->stream>>>(part, nblocks, r, dres);
   QS_TRY(launch_check("expect_z_finish"));
   return read_back(s, dres, n, out);
 }
@@ -981,7 +1072,7 @@ static int pauli_exact(qs_state* s, const qs_pauli* terms, size_t nterms, double
         return QS_OK;
       });
       QS_TRY(launch_check("pauli_tile"));
-      k_pauli_exact_finish<<<1, 32, 0, s->stream>>>(part, nblocks, g.nt, sums + 2 * (size_t)next);
+      k_pauli_exact_finish<<<g.nt, 256, 0, s->stream>>>(part, nblocks, sums + 2 * (size_t)next);
       QS_TRY(launch_check("pauli_exact_finish"));
       next += g.nt;
     }
@@ -1108,6 +1199,6 @@ extern "C" int qs_expect_z_all_noalloc(const double* device_amps, int n, double*
   // nothing left over from an earlier call is read
   k_expect_z<<<nblocks, 256, 0, st>>>((const double2*)device_amps, r, part);
   QS_TRY(launch_check("expect_z (no-alloc)"));
-  k_expect_z_finish<<<1, 64, 0, st>>>(part, nblocks, r, n, device_out);
+  k_expect_z_finish<<<n, 256, 0, st>>>(part, nblocks, r, device_out);
   return launch_check("expect_z_finish (no-alloc)");
 }

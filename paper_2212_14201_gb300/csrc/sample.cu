@@ -210,15 +210,10 @@ extern "C" int qs_sample(const qs_state* cs, uint64_t seed, uint64_t shots, uint
   long long* lsb = (long long*)(P + (nsb + 1));
   long long* lall = lsb + (nsb + 1);
   const int64_t K = L < 32 ? L : 32;  // amplitudes per running-sum checkpoint
-  struct StreamBuf {                   // freed on the stream when the call returns
-    void* p = nullptr;
-    cudaStream_t st;
-    ~StreamBuf() {
-      if (p) cudaFreeAsync(p, st);
-    }
-  } cpb{nullptr, s->stream};
-  QS_CUDA(dmalloc_async(&cpb.p, (size_t)(N / K) * sizeof(double), s->stream));  // 1/64 of the state's bytes
-  double* cp = (double*)cpb.p;
+  const size_t cp_count = (size_t)(N / K);  // 1/64 of the state's bytes
+  ScratchBuf buf;                           // the checkpoints, then the shots
+  QS_TRY(take_scratch(s, cp_count * sizeof(double) + (on_device ? 0 : shots * sizeof(uint64_t)), &buf));
+  double* cp = (double*)buf.p;
   int g1 = (int)std::min<int64_t>((nb + 127) / 128, 152 * 16);
   KTimer kt(s, QS_K_REDUCE, s->n, 3, 0, 0, (double)N, 4.0 * (double)N);
   note_launch(4);
@@ -234,11 +229,7 @@ extern "C" int qs_sample(const qs_state* cs, uint64_t seed, uint64_t shots, uint
   const int g2 = (int)std::max<int64_t>(1, std::min<int64_t>((nb + 255) / 256, 152 * 8));
   k_seg_offset<<<g2, 256, 0, s->stream>>>(E, nb, (int)G, P, lall, lastnz);
   QS_TRY(launch_check("superblock offset"));
-  uint64_t* dout = out;
-  if (!on_device) {
-    const cudaError_t e = dmalloc_async((void**)&dout, shots * sizeof(uint64_t), s->stream);
-    if (e != cudaSuccess) return cuda_fail(e, "cudaMallocAsync(samples)");
-  }
+  uint64_t* dout = on_device ? out : (uint64_t*)(cp + cp_count);
   int g3 = (int)std::min<uint64_t>((shots + 127) / 128, 152 * 16);
   with_amps(s, [&](auto* a) {
     k_sample<<<g3, 128, 0, s->stream>>>(a, E, lastnz, cp, nb, L, K, seed, shots, dout);
@@ -251,7 +242,6 @@ extern "C" int qs_sample(const qs_state* cs, uint64_t seed, uint64_t shots, uint
       if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
       if (e != cudaSuccess) rc = cuda_fail(e, "sample readback");
     }
-    cudaFreeAsync(dout, s->stream);
   }
   return rc;
 }
