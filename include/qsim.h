@@ -262,9 +262,8 @@ int qs_set_aggregate(int on);
  * over the tile (2^m phases in device memory, one complex product per
  * amplitude), leaving real rotations: 12 instead of 18 limb products per
  * amplitude.  A table is built where the general ops it makes real and the
- * diagonals it absorbs outweigh its own cost.  The tables are staged through
- * pinned memory per pass, so a qs_apply with a plan is not stream-capturable
- * while this is on.  Results agree with the switch off within rounding (table
+ * diagonals it absorbs outweigh its own cost.  The tables are built on the device
+ * before each pass.  Results agree with the switch off within rounding (table
  * entries formed in double).  Always QS_OK. */
 int qs_set_phase_tables(int on);
 

@@ -473,7 +473,7 @@ static int backward_fused(qs_state* s, double2* lam, const qs_gate* gates, size_
       const Mat2& rb = opm[rpheads[pi] + 2];
       for (int k = 0; k < 4; ++k)
         for (int c = 0; c < 4; ++c)
-          rpm.push_back(q60_split(q60_from_double(rb.m[2 * (k >> 1) + (c >> 1)].re * ra.m[2 * (k & 1) + (c & 1)].re)));
+          rpm.push_back(q60_split_coef(q60_from_double(rb.m[2 * (k >> 1) + (c >> 1)].re * ra.m[2 * (k & 1) + (c & 1)].re)));
     }
     bp.op_end = (int)ops.size();
     bp.nslots = slot;

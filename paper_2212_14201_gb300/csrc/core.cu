@@ -475,8 +475,6 @@ extern "C" int qs_free(qs_state* s) {
   if (s->ws) cudaFree(s->ws);
   if (s->pinned) cudaFreeHost(s->pinned);
   if (s->tables) cudaFree(s->tables);
-  if (s->tables_pinned) cudaFreeHost(s->tables_pinned);
-  if (s->tables_ev) cudaEventDestroy(s->tables_ev);
   for (auto& p : s->pending) {
     cudaEventDestroy(p.e0);
     cudaEventDestroy(p.e1);

@@ -165,6 +165,14 @@ QS_HD QL q60_split(int64_t V) {
   return {(int32_t)(V >> 30), (int32_t)(V & ((1ll << 30) - 1))};
 }
 
+// The same for a coefficient, with -2^29 <= l < 2^29 (h = round(V / 2^30)): a dropped
+// low x low product of a coefficient and an amplitude then has mean zero and half
+// the size, where two non-negative low limbs leave a bias of a quarter of 2^-60.
+QS_HD QL q60_split_coef(int64_t V) {
+  const int64_t h = (V + (1ll << 29)) >> 30;
+  return {(int32_t)h, (int32_t)(V - h * (1ll << 30))};
+}
+
 // c + a b.  A product and a 64-bit sum, which the assembler joins into one wide
 // multiply-add; written as one mad.wide it issues a multiply and a separate 64-bit
 // addition (ncu: 1.0 instead of 0.1 ALU instructions per product).  n=30 brickwork
@@ -228,9 +236,9 @@ struct QC {
 
 QS_HD QC qc_make(double re, double im) {
   QC c;
-  c.re = q60_split(q60_from_double(re));
-  c.im = q60_split(q60_from_double(im));
-  c.nim = q60_split(-q60_from_double(im));
+  c.re = q60_split_coef(q60_from_double(re));
+  c.im = q60_split_coef(q60_from_double(im));
+  c.nim = q60_split_coef(-q60_from_double(im));
   return c;
 }
 
@@ -241,9 +249,9 @@ QS_HD QC qc_make(double re, double im) {
 QS_HD QC qc_make_gauss(double re, double im) {
   const int64_t c = q60_from_double(re), d = q60_from_double(im);
   QC q;
-  q.re = q60_split(c);
-  q.im = q60_split(d - c);
-  q.nim = q60_split(c + d);
+  q.re = q60_split_coef(c);
+  q.im = q60_split_coef(d - c);
+  q.nim = q60_split_coef(c + d);
   return q;
 }
 

@@ -44,13 +44,9 @@ struct qs_state {
   void* scratch = nullptr;
   size_t scratch_bytes = 0;
   bool scratch_used = false;
-  // Phase tables of tile passes: device copy, pinned staging, and the event of the
-  // last upload (the staging buffer is rewritten only after that copy ran).
+  // Phase tables of the tile pass being run, where the workspace is too small (device).
   void* tables = nullptr;
   size_t tables_bytes = 0;
-  void* tables_pinned = nullptr;
-  size_t tables_pinned_bytes = 0;
-  cudaEvent_t tables_ev = nullptr;
 };
 
 namespace qs {

@@ -306,14 +306,41 @@ static Zyz zyz(const Mat2& U) {
   return z;
 }
 
-// A diagonal over the tile: entry j for tile index j (bit b of j = tile bit b),
-// times a sign per tile: (-1)^(x_q j_t) for each (q, t) in signs (a CZ between
-// the qubit q outside the tile and the tile bit t; x_q is the tile's own bit q).
+// A controlled diagonal gate among the tile's bits: where every bit of lmask is
+// set, diag(e0, e1) on tile bit tb.
+struct TableTerm {
+  uint32_t lmask;
+  int tb;
+  C2 e0, e1;
+};
+
+// A diagonal over the tile as a product: entry j (bit b of j = tile bit b) is the
+// product over the tile bits of d0 or d1 and over the terms, times a sign per
+// tile: (-1)^(x_q j_t) for each (q, t) in signs (a CZ between the qubit q outside
+// the tile and the tile bit t; x_q is the tile's own bit q).
 struct PhaseTable {
   int m = 0;
-  std::vector<C2> t;
+  std::vector<C2> d0, d1;
+  std::vector<TableTerm> terms;
   std::vector<std::pair<int, int>> signs;  // (global qubit outside the tile, tile bit)
 };
+
+// Its 2^m entries (the kernels get theirs from k_phase_tables).
+static std::vector<C2> table_entries(const PhaseTable& pt) {
+  std::vector<C2> t((size_t)1 << pt.m, C2{1.0, 0.0});
+  // product over tile bits, doubling the filled prefix once per bit
+  for (int b = 0; b < pt.m; ++b) {
+    const size_t h = (size_t)1 << b;
+    for (size_t j = 0; j < h; ++j) {
+      t[j + h] = cmul2(t[j], pt.d1[b]);
+      t[j] = cmul2(t[j], pt.d0[b]);
+    }
+  }
+  for (const TableTerm& tm : pt.terms)
+    for (size_t j = 0; j < t.size(); ++j)
+      if ((j & tm.lmask) == tm.lmask) t[j] = cmul2(t[j], ((j >> tm.tb) & 1) ? tm.e1 : tm.e0);
+  return t;
+}
 
 // A diagonal op that is a CZ between a tile bit and a qubit outside the tile:
 // diag(1, -1) on its target with exactly one control, one of the two qubits
@@ -517,18 +544,9 @@ static void extract_phases(const std::vector<Op1>& ops, const int* local, int n,
     }
     PhaseTable t;
     t.m = m;
-    t.t.assign((size_t)1 << m, C2{1.0, 0.0});
-    // product over tile bits, doubling the filled prefix once per bit
-    for (int b = 0; b < m; ++b) {
-      const size_t h = (size_t)1 << b;
-      for (size_t j = 0; j < h; ++j) {
-        t.t[j + h] = cmul2(t.t[j], d1[b]);
-        t.t[j] = cmul2(t.t[j], d0[b]);
-      }
-    }
-    for (const Term& tm : terms)
-      for (size_t j = 0; j < t.t.size(); ++j)
-        if ((j & tm.lmask) == tm.lmask) t.t[j] = cmul2(t.t[j], ((j >> tm.tb) & 1) ? tm.e1 : tm.e0);
+    t.d0.assign(d0, d0 + m);
+    t.d1.assign(d1, d1 + m);
+    for (const Term& tm : terms) t.terms.push_back(TableTerm{tm.lmask, tm.tb, tm.e0, tm.e1});
     terms.clear();
     // sign terms: a table of a pass may carry TILE_MAX_SIGNS of them, and only the
     // first TILE_MAX_SIGNED_TABLES tables of a pass carry any; the rest stay ops
@@ -1250,10 +1268,11 @@ extern "C" int qs_plan_pass_ops(const qs_plan* p, size_t pass, const qs_gate* ga
     }
   }
   for (size_t t = 0; t < pt.size() && t < table_cap; ++t) {
-    double* d = tables + t * 2 * pt[t].t.size();
-    for (size_t k = 0; k < pt[t].t.size(); ++k) {
-      d[2 * k] = pt[t].t[k].re;
-      d[2 * k + 1] = pt[t].t[k].im;
+    const std::vector<C2> e = table_entries(pt[t]);
+    double* d = tables + t * 2 * e.size();
+    for (size_t k = 0; k < e.size(); ++k) {
+      d[2 * k] = e[k].re;
+      d[2 * k + 1] = e[k].im;
     }
   }
   return QS_OK;
@@ -1280,29 +1299,20 @@ extern "C" int qs_set_aggregate(int on) {
 }
 
 
-// Copies a pass's phase tables to the device in the layout the tile kernel reads:
-// per table three arrays of 2^m limb pairs (the Gauss-form parts re, im, nim of
-// qc_make_gauss), so that a warp's loads of one part are consecutive.  Pinned
-// staging, one asynchronous copy on the state's stream, an event so that the
-// staging buffer is rewritten only after that copy has run (the host waits, the
-// stream does not); the device buffer is rewritten in stream order, after the
-// previous pass's kernel.
-static int upload_tables(qs_state* s, const std::vector<PhaseTable>& pt, const QL** dev, bool f32) {
-  size_t per = 0;
-  for (const PhaseTable& t : pt) per = std::max(per, t.t.size());
-  // FP32 engine: one float2 per entry (table t at t * 2^m)
-  // Q60 engine: per entry the limbs of c = Re T and d = Im T (16 bytes)
-  const size_t bytes = f32 ? pt.size() * per * sizeof(float2) : pt.size() * 2 * per * sizeof(QL);
-  if (!s->tables_ev) QS_CUDA(cudaEventCreateWithFlags(&s->tables_ev, cudaEventDisableTiming));
-  QS_CUDA(cudaEventSynchronize(s->tables_ev));
-  if (s->tables_pinned_bytes < bytes) {
-    if (s->tables_pinned) cudaFreeHost(s->tables_pinned);
-    s->tables_pinned = nullptr;
-    s->tables_pinned_bytes = 0;
-    QS_CUDA(hmalloc_pinned(&s->tables_pinned, bytes));
-    s->tables_pinned_bytes = bytes;
-  }
-  if (s->tables_bytes < bytes) {
+// Builds a pass's phase tables in the state's table buffer: their factors travel as
+// kernel parameters and k_phase_tables multiplies them out there (on the host the
+// 2^m entries of 25 tables took 0.6 ms of the 0.61 ms that 300 random gates on 20
+// qubits needed, and an upload had to wait for the pass before it).  They stay in
+// the workspace, which no other call uses while a pass runs (152 tables of 4096
+// entries fit); more than that, or wider ones, in a buffer of their own.  Either is
+// rewritten in stream order, after the previous pass's kernel.
+static size_t tables_bytes(const std::vector<PhaseTable>& pt, bool f32) {
+  return pt.empty() ? 0 : (pt.size() << pt[0].m) * (f32 ? sizeof(float2) : 2 * sizeof(QL));
+}
+static int build_tables(qs_state* s, const std::vector<PhaseTable>& pt, const QL** dev, bool f32) {
+  const int m = pt[0].m;
+  const size_t bytes = tables_bytes(pt, f32), per = bytes / pt.size();
+  if (s->ws_bytes < bytes && s->tables_bytes < bytes) {
     if (s->tables) {
       QS_CUDA(cudaStreamSynchronize(s->stream));
       cudaFree(s->tables);
@@ -1312,23 +1322,52 @@ static int upload_tables(qs_state* s, const std::vector<PhaseTable>& pt, const Q
     QS_CUDA(dmalloc(&s->tables, bytes));
     s->tables_bytes = bytes;
   }
-  if (f32) {
-    float2* hf = (float2*)s->tables_pinned;
-    for (size_t t = 0; t < pt.size(); ++t)
-      for (size_t j = 0; j < pt[t].t.size(); ++j)
-        hf[t * per + j] = make_float2((float)pt[t].t[j].re, (float)pt[t].t[j].im);
-  }
-  QL* host = (QL*)s->tables_pinned;
-  for (size_t t = 0; !f32 && t < pt.size(); ++t) {
-    QL* e = host + t * 2 * per;
-    for (size_t j = 0; j < pt[t].t.size(); ++j) {
-      e[2 * j] = q60_split(q60_from_double(pt[t].t[j].re));
-      e[2 * j + 1] = q60_split(q60_from_double(pt[t].t[j].im));
+  char* buf = (char*)(s->ws_bytes < bytes ? s->tables : s->ws);
+  std::unique_ptr<TableArgs> g(new (std::nothrow) TableArgs);
+  if (!g) return fail(QS_ERR_OOM, "host allocation failed");
+  for (size_t t = 0; t < pt.size();) {
+    g->m = m;
+    g->f32 = f32;
+    g->ntab = 0;
+    int used = 0;
+    const size_t first = t;
+    for (; t < pt.size() && g->ntab < TABLE_ARGS_MAX; ++t) {
+      const PhaseTable& p = pt[t];
+      // a CZ is a sign where both bits are set; the others multiply
+      auto is_cz = [](const TableTerm& x) {
+        return unit_code(x.e0) == U_ONE && unit_code(x.e1) == U_MINUS_ONE;
+      };
+      int ns = 0;
+      for (const TableTerm& x : p.terms) ns += is_cz(x);
+      const int nt = (int)p.terms.size() - ns, need = 4 * m + ns + 5 * nt;
+      if (used + need > TABLE_ARGS_WORDS) break;
+      const int k = g->ntab++;
+      g->off[k] = (uint16_t)used;
+      g->ns[k] = (uint16_t)ns;
+      g->nt[k] = (uint16_t)nt;
+      double* w = g->w + used;
+      for (int b = 0; b < m; ++b) {
+        *w++ = p.d0[b].re;
+        *w++ = p.d0[b].im;
+        *w++ = p.d1[b].re;
+        *w++ = p.d1[b].im;
+      }
+      for (const TableTerm& x : p.terms)
+        if (is_cz(x)) *w++ = (double)(x.lmask | (1u << x.tb));
+      for (const TableTerm& x : p.terms)
+        if (!is_cz(x)) {
+          *w++ = (double)((uint64_t)x.lmask * 32 + (uint64_t)x.tb);
+          *w++ = x.e0.re;
+          *w++ = x.e0.im;
+          *w++ = x.e1.re;
+          *w++ = x.e1.im;
+        }
+      used += need;
     }
+    if (t == first) return fail(QS_ERR_UNSUPPORTED, "phase table of %zu terms", pt[t].terms.size());
+    QS_TRY(launch_tables(s, *g, buf + first * per));
   }
-  QS_CUDA(cudaMemcpyAsync(s->tables, host, bytes, cudaMemcpyHostToDevice, s->stream));
-  QS_CUDA(cudaEventRecord(s->tables_ev, s->stream));
-  *dev = (const QL*)s->tables;
+  *dev = (const QL*)buf;
   return QS_OK;
 }
 
@@ -1665,7 +1704,7 @@ static int build_tile_args(int n, int prec, const PlanPass& ps, const qs_gate* g
   }
   for (int k = 0; rc == QS_OK && k < g->nops; ++k) {
     const TileOp& o = g->ops[k];
-    if (o.kind == TOP_DTABLE && (o.lcmask >= ptables.size() || o.tb != m || ptables[o.lcmask].t.size() != ((size_t)1 << m)))
+    if (o.kind == TOP_DTABLE && (o.lcmask >= ptables.size() || o.tb != m || ptables[o.lcmask].m != m))
       rc = fail(QS_ERR_INVALID_ARG, "internal: malformed phase-table op");
     if ((o.kind == TOP_REAL2 || o.kind == TOP_REAL3) && (k + 1 >= g->nops || g->ops[k + 1].kind != TOP_CONT ||
                                 (o.code1 >= 0 && (size_t)o.code1 >= ptables.size())))
@@ -1700,7 +1739,7 @@ static int run_tile_pass(qs_state* s, const PlanPass& ps, const qs_gate* gates, 
   std::vector<PhaseTable> ptables;
   double flops = 0.0, int_ops = 0.0;
   int rc = build_tile_args(s->n, s->prec, ps, gates, params, fixed, io, g, ptables, &flops, &int_ops);
-  if (rc == QS_OK && !ptables.empty()) rc = upload_tables(s, ptables, &g->tables, s->prec == 64);
+  if (rc == QS_OK && !ptables.empty()) rc = build_tables(s, ptables, &g->tables, s->prec == 64);
   if (rc == QS_OK && (g->nops > 0 || (g->io >> 8) != 0)) {
     rc = launch_tile(s, *g, fixed ? 0.0 : flops, fixed ? int_ops : 0.0, (int)ps.gates.size(), fixed);
     *launched = rc == QS_OK;

@@ -301,8 +301,8 @@ inline void q60_triple_coef(const double* ra, const double* rb, const double* rc
     const double sbk = (k & 2) ? -sb : sb, sck = (k & 1) ? -sc : sc;
     const double abr = ca * cb - sa * sbk, abi = sa * cb + ca * sbk;
     const double re = 0.25 * (abr * cc - abi * sck), im = 0.25 * (abi * cc + abr * sck);
-    out[2 * k] = q60_split(q60_from_double(re));
-    out[2 * k + 1] = q60_split(q60_from_double(im));
+    out[2 * k] = q60_split_coef(q60_from_double(re));
+    out[2 * k + 1] = q60_split_coef(q60_from_double(im));
   }
 }
 
@@ -323,7 +323,7 @@ inline void q60_quad4_coef(const double* ra, const double* rb, const double* rc,
       wr = tr;
       wi = ti;
     }
-    const QL re = q60_split(q60_from_double(0.125 * wr)), im = q60_split(q60_from_double(0.125 * wi));
+    const QL re = q60_split_coef(q60_from_double(0.125 * wr)), im = q60_split_coef(q60_from_double(0.125 * wi));
     P[3 * k] = q3_of(re);
     P[3 * k + 1] = q3_of(im);
     P[3 * k + 2] = q3_neg(P[3 * k + 1]);
@@ -339,7 +339,7 @@ inline void q60_pair_coef(const double* ra, const double* rb, QL out[6], int* fl
   const double pr = 0.5 * (ca * cb - sa * sb), pi = 0.5 * (sa * cb + ca * sb);
   const double qr = 0.5 * (ca * cb + sa * sb), qi = 0.5 * (sa * cb - ca * sb);
   const double v[6] = {pr, pi, -pi, qr, qi, -qi};
-  for (int k = 0; k < 6; ++k) out[k] = q60_split(q60_from_double(v[k]));
+  for (int k = 0; k < 6; ++k) out[k] = q60_split_coef(q60_from_double(v[k]));
 }
 
 }  // namespace qs

@@ -733,6 +733,66 @@ __global__ void __launch_bounds__(THREADS, THREADS == 256 ? E::kMinBlocks : 1) k
   }
 }
 
+// Phase tables from their factors: a CTA takes a run of entries of one table, forms
+// the products over the tile's low six bits and over the rest once (at most 64 + 128
+// products), and an entry is their product times its terms.  Bound by FP64 issue
+// (six FP64 instructions a complex product): 25 tables of 4096 entries a few
+// microseconds.
+constexpr uint32_t TABLE_RUN = 1024;
+__global__ void __launch_bounds__(256) k_phase_tables(const __grid_constant__ TableArgs g, void* out) {
+  __shared__ double2 lo[64], hi[1 << (TILE_MAX_M - 6)];
+  const uint32_t TS = 1u << g.m, run = min(TS, TABLE_RUN), per = TS / run;
+  const int t = blockIdx.x / per;
+  const uint32_t j0 = (blockIdx.x % per) * run;
+  const double* d = g.w + g.off[t];
+  const int lb = min(g.m, 6), hb = g.m - lb;
+  auto mul = [](double2 x, double2 y) {
+    return make_double2(fma(x.x, y.x, -x.y * y.y), fma(x.x, y.y, x.y * y.x));
+  };
+  auto prod = [&](uint32_t bits, int b0, int nb) {
+    double2 v = make_double2(1.0, 0.0);
+    for (int b = 0; b < nb; ++b) {
+      const double* e = d + 4 * (b0 + b);
+      const bool one = (bits >> b) & 1;
+      v = mul(v, make_double2(one ? e[2] : e[0], one ? e[3] : e[1]));
+    }
+    return v;
+  };
+  if (threadIdx.x < (1u << lb)) lo[threadIdx.x] = prod(threadIdx.x, 0, lb);
+  const uint32_t h = threadIdx.x - 64;  // the next threads: the high products
+  if (threadIdx.x >= 64 && h < (1u << hb)) hi[h] = prod(h, lb, hb);
+  __syncthreads();
+  const double* sg = d + 4 * g.m;
+  const double* tm = sg + g.ns[t];
+  for (uint32_t j = j0 + threadIdx.x; j < j0 + run; j += 256) {
+    double2 v = mul(lo[j & ((1u << lb) - 1)], hi[j >> lb]);
+    uint32_t neg = 0;
+    for (int k = 0; k < g.ns[t]; ++k) {
+      const uint32_t mask = (uint32_t)sg[k];
+      neg ^= (j & mask) == mask;
+    }
+    for (int k = 0; k < g.nt[t]; ++k) {
+      const uint32_t code = (uint32_t)tm[5 * k], mask = code >> 5;
+      const int e = (j >> (code & 31)) & 1 ? 3 : 1;
+      if ((j & mask) == mask) v = mul(v, make_double2(tm[5 * k + e], tm[5 * k + e + 1]));
+    }
+    if (neg) v = make_double2(-v.x, -v.y);
+    if (g.f32) {
+      reinterpret_cast<float2*>(out)[(size_t)t * TS + j] = make_float2((float)v.x, (float)v.y);
+    } else {
+      const QL c = q60_split_coef(q60_from_double(v.x)), s = q60_split_coef(q60_from_double(v.y));
+      reinterpret_cast<int4*>(out)[(size_t)t * TS + j] = make_int4(c.h, c.l, s.h, s.l);
+    }
+  }
+}
+
+int launch_tables(qs_state* s, const TableArgs& g, void* out) {
+  const uint32_t TS = 1u << g.m;
+  note_launch(1);
+  k_phase_tables<<<g.ntab * (TS / std::min(TS, TABLE_RUN)), 256, 0, s->stream>>>(g, out);
+  return launch_check("phase tables");
+}
+
 // In-place Q60 integer pairs -> complex128 (the same rounding as a tile pass's store).
 __global__ void k_q60_release(double2* __restrict__ a, size_t N) {
   longlong2* v = reinterpret_cast<longlong2*>(a);

@@ -83,6 +83,20 @@ struct TileArgs {
 };
 static_assert(sizeof(TileArgs) < 32000, "tile arguments must fit the kernel parameter space");
 
+// Factors of up to TABLE_ARGS_MAX phase tables of one pass: per table 4 m words (d0,
+// d1 of every tile bit), ns masks of two or more bits whose conjunction negates the
+// entry, and nt terms of five words (control mask * 32 + target bit, e0, e1).  A
+// pass has at most TILE_MAX_OPS gates, so any one table fits.
+constexpr int TABLE_ARGS_MAX = 16, TABLE_ARGS_WORDS = 1408;
+struct TableArgs {
+  int m, ntab, f32;
+  uint16_t off[TABLE_ARGS_MAX], ns[TABLE_ARGS_MAX], nt[TABLE_ARGS_MAX];
+  double w[TABLE_ARGS_WORDS];
+};
+static_assert(4 * TILE_MAX_M + 5 * TILE_MAX_OPS <= TABLE_ARGS_WORDS, "one table must fit a launch");
+// Multiplies the tables out at `out` (Q60 limb pairs of Re and Im, or float2).
+int launch_tables(qs_state* s, const TableArgs& args, void* out);
+
 int launch_tile(qs_state* s, const TileArgs& args, double flops, double int_ops, int ngates, bool fixed);
 // Converts a buffer of Q60 integer pairs (left by a tile pass with io bit 1) back
 // to complex128 in place.
