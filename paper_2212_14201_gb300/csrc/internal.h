@@ -165,6 +165,9 @@ int choose_fixed(qs_state* s, bool* fixed);
 int launch_op1(qs_state* s, const Op1& op, bool fixed);  // complex64 states: FP32 arithmetic
 int launch_dense(qs_state* s, const int* targets, int k, uint64_t cmask, const C2* mat);
 
+// Whether records of this type are diagonal whatever their parameters.
+bool structurally_diagonal(int type);
+
 // ---- planning ------------------------------------------------------------------
 // One greedy fusion pass over `remaining` (indices in program order): `pass`
 // receives the gates that run in a tile of at most m qubits containing `low`,

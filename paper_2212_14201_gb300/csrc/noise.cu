@@ -15,10 +15,14 @@
 // A trajectory, gate by gate: a rotation's theta gets e (2u - 1) (one draw);
 // the gate; then for each matching rule and each qubit the gate touches
 // (ascending) one draw u picks the smallest j with u W < w_1 + ... + w_j, and
-// psi <- K_j psi / sqrt(w_j).  Weights w_j = ||K_j psi||^2 = tr(K_j^dag K_j G),
-// G the 2x2 Gram matrix of the qubit's amplitude pairs (one reduction pass);
+// psi <- K_j psi / sqrt(w_j).  Weights w_j = ||K_j psi||^2;
 // for a set of scaled unitaries w_j is the squared scale (no pass), and the
 // chosen Pauli joins the gate stream, so such stretches stay fusable.
+// Every K_j above is real with a diagonal K_j^dag K_j: the weights need only the
+// populations of the qubit, and a diagonal K_j (the usual no-decay operator) scales
+// them.  So the joint populations of up to JOINT_MAX qubits that channels touch next
+// are read in one pass, the draws of a whole gate layer are decided from that table
+// on the host, and the chosen diagonal operators are applied together.
 #include <math.h>
 
 #include <string.h>
@@ -32,103 +36,52 @@
 
 namespace qs {
 
-// ---- Gram matrix of one qubit: g00 = sum |a0|^2, g11 = sum |a1|^2,
-// g01 = sum a0 conj(a1), over the pairs (x, x | 2^q) -------------------------------
+// ---- product of real diagonal factors on a few qubits ----------------------------------
+// a_x *= f[key], key = the listed qubits' bits of x.  Moves the state once for all of
+// them; two FP64 products per amplitude (2^22 amplitudes: 17 us at GB300's FP64 rate,
+// about what their bytes take from L2).
+constexpr int JOINT_MAX = 11;
+struct ScaleArgs {
+  uint64_t N;
+  int nq;
+  int q[JOINT_MAX];
+  double f[1 << JOINT_MAX];
+};
+
+__device__ __forceinline__ void scale_amp(double2* p, double f) {
+  const double2 v = *p;
+  *p = make_double2(v.x * f, v.y * f);
+}
+__device__ __forceinline__ void scale_amp(float2* p, double f) {
+  const float2 v = *p;
+  *p = make_float2((float)(v.x * f), (float)(v.y * f));
+}
+
 template <class A>
-__global__ void __launch_bounds__(256) k_gram(const A* __restrict__ a, uint64_t pairs, int q,
-                                               double* __restrict__ part) {
-  __shared__ double sh[4][8];
-  double g00 = 0.0, g11 = 0.0, gr = 0.0, gi = 0.0;
-  const uint64_t b = 1ull << q;
-  for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < pairs; i += (uint64_t)gridDim.x * blockDim.x) {
-    const uint64_t x0 = ((i >> q) << (q + 1)) | (i & (b - 1));
-    const double2 a0 = ld_amp(a, x0), a1 = ld_amp(a, x0 | b);
-    g00 = fma(a0.y, a0.y, fma(a0.x, a0.x, g00));
-    g11 = fma(a1.y, a1.y, fma(a1.x, a1.x, g11));
-    gr = fma(a0.y, a1.y, fma(a0.x, a1.x, gr));   // Re(a0 conj(a1))
-    gi = fma(a0.y, a1.x, fma(-a0.x, a1.y, gi));  // Im(a0 conj(a1))
-  }
-  double v[4] = {g00, g11, gr, gi};
-  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
-    if (l == 0) sh[k][w] = v[k];
-  }
+__global__ void __launch_bounds__(256) k_scale(A* __restrict__ a, const __grid_constant__ ScaleArgs g) {
+  __shared__ double f[1 << JOINT_MAX];
+  for (int i = threadIdx.x; i < (1 << g.nq); i += 256) f[i] = g.f[i];
   __syncthreads();
-  if (threadIdx.x < 4) {
-    double t = 0.0;
-    for (int i = 0; i < 8; ++i) t += sh[threadIdx.x][i];
-    part[(size_t)blockIdx.x * 4 + threadIdx.x] = t;
-  }
-}
-
-// The same four sums exactly, for a state within the Q60 bound: components rounded
-// once to Q60 and the products summed as 128-bit integers (units of 2^-120; every
-// sum is at most the squared norm <= 1.5625 in magnitude).  Integer pipes instead
-// of GB300's 1/74-rate FP64 pipe.
-using i128 = __int128;
-
-__device__ __forceinline__ i128 shfl_xor_i128(i128 v, int o) {
-  const unsigned long long lo = __shfl_xor_sync(0xffffffffu, (unsigned long long)(uint64_t)v, o);
-  const unsigned long long hi = __shfl_xor_sync(0xffffffffu, (unsigned long long)(uint64_t)((unsigned __int128)v >> 64), o);
-  return (i128)(((unsigned __int128)hi << 64) | lo);
-}
-
-template <class A>
-__global__ void __launch_bounds__(256) k_gram_exact(const A* __restrict__ a, uint64_t pairs, int q,
-                                                     uint64_t* __restrict__ part) {
-  __shared__ uint64_t sh[4][8][2];
-  i128 v[4] = {0, 0, 0, 0};
-  const uint64_t b = 1ull << q;
-  for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < pairs; i += (uint64_t)gridDim.x * blockDim.x) {
-    const uint64_t x0 = ((i >> q) << (q + 1)) | (i & (b - 1));
-    const double2 a0 = ld_amp(a, x0), a1 = ld_amp(a, x0 | b);
-    const int64_t r0 = q60_from_double(a0.x), i0 = q60_from_double(a0.y);
-    const int64_t r1 = q60_from_double(a1.x), i1 = q60_from_double(a1.y);
-    v[0] += (i128)r0 * r0 + (i128)i0 * i0;
-    v[1] += (i128)r1 * r1 + (i128)i1 * i1;
-    v[2] += (i128)r0 * r1 + (i128)i0 * i1;  // Re(a0 conj(a1))
-    v[3] += (i128)i0 * r1 - (i128)r0 * i1;  // Im(a0 conj(a1))
-  }
-  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+  const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
+  auto factor = [&](uint64_t x) {
+    uint32_t key = 0;
 #pragma unroll
-  for (int k = 0; k < 4; ++k) {
+    for (int j = 0; j < JOINT_MAX; ++j)
+      if (j < g.nq) key |= (uint32_t)((x >> g.q[j]) & 1) << j;
+    return f[key];
+  };
+  uint64_t x = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
+  for (; x + 3 * stride < g.N; x += 4 * stride) {  // four loads in flight
+    A v[4];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v[k] += shfl_xor_i128(v[k], o);
-    if (l == 0) {
-      sh[k][w][0] = (uint64_t)v[k];
-      sh[k][w][1] = (uint64_t)((unsigned __int128)v[k] >> 64);
+    for (int k = 0; k < 4; ++k) v[k] = a[x + k * stride];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      scale_amp(&v[k], factor(x + k * stride));
+      a[x + k * stride] = v[k];
     }
   }
-  __syncthreads();
-  if (threadIdx.x < 4) {
-    i128 t = 0;
-    for (int i = 0; i < 8; ++i) t += (i128)(((unsigned __int128)sh[threadIdx.x][i][1] << 64) | sh[threadIdx.x][i][0]);
-    part[((size_t)blockIdx.x * 4 + threadIdx.x) * 2] = (uint64_t)t;
-    part[((size_t)blockIdx.x * 4 + threadIdx.x) * 2 + 1] = (uint64_t)((unsigned __int128)t >> 64);
-  }
-}
-
-__global__ void k_gram_exact_finish(const uint64_t* __restrict__ part, int nblocks, double* __restrict__ out) {
-  const int k = threadIdx.x;
-  if (k >= 4) return;
-  i128 t = 0;
-  for (int c = 0; c < nblocks; ++c)
-    t += (i128)(((unsigned __int128)part[((size_t)c * 4 + k) * 2 + 1] << 64) | part[((size_t)c * 4 + k) * 2]);
-  const bool neg = t < 0;
-  const unsigned __int128 m = neg ? (unsigned __int128)(-t) : (unsigned __int128)t;
-  const double d = (double)(uint64_t)(m >> 64) * 18446744073709551616.0 + (double)(uint64_t)m;
-  out[k] = (neg ? -d : d) * 0x1p-120;
-}
-
-__global__ void k_gram_finish(const double* __restrict__ part, int nblocks, double* __restrict__ out) {
-  const int k = threadIdx.x;
-  if (k >= 4) return;
-  double t = 0.0;
-  for (int c = 0; c < nblocks; ++c) t += part[(size_t)c * 4 + k];
-  out[k] = t;
+  for (; x < g.N; x += stride) scale_amp(a + x, factor(x));
 }
 
 // ---- readout error on sampled indices ----------------------------------------------
@@ -247,6 +200,72 @@ struct Trajectory {
 
   double draw() { return u01_of(splitmix64(seed, k++)); }
 
+  // Diagonal operators chosen but not yet applied (real factors, at most one entry a
+  // qubit).  Every pending gate commutes with them: it is diagonal or its target is
+  // another qubit, so they may be applied before it.
+  struct Scale {
+    int q;
+    double f0, f1;
+  };
+  std::vector<Scale> scales;
+  // Joint populations of `jq` in the state with every pending gate and factor
+  // applied (entry bit i: qubit jq[i]); no pending non-diagonal gate has its target
+  // among them, so gates on other qubits leave them as they are.
+  std::vector<int> jq;
+  std::vector<double> joint;
+
+  int joint_bit(int q) const {
+    for (size_t i = 0; i < jq.size(); ++i)
+      if (jq[i] == q) return (int)i;
+    return -1;
+  }
+
+  // Appends a gate; target: its target qubit, diagonal: whether it is diagonal.
+  int push(const qs_gate& g, int target, bool diagonal) {
+    if (!diagonal) {
+      for (const Scale& c : scales)
+        if (c.q == target) {
+          QS_TRY(apply_scales());
+          break;
+        }
+      if (joint_bit(target) >= 0) jq.clear();
+    }
+    pending.push_back(g);
+    return QS_OK;
+  }
+
+  int apply_scales() {
+    if (scales.empty()) return QS_OK;
+    ScaleArgs g;
+    g.N = 1ull << s->n;
+    g.nq = (int)scales.size();
+    for (int j = 0; j < g.nq; ++j) g.q[j] = scales[j].q;
+    for (int k = 0; k < (1 << g.nq); ++k) {
+      double f = 1.0;
+      for (int j = 0; j < g.nq; ++j) f *= (k >> j) & 1 ? scales[j].f1 : scales[j].f0;
+      g.f[k] = f;
+    }
+    scales.clear();
+    const int nblocks = (int)std::min<uint64_t>(152 * 8, (g.N + 255) / 256);
+    KTimer kt(s, QS_K_DIAG, 1, g.nq, 0, 0, (double)g.N, 2.0 * (double)g.N);
+    with_amps(s, [&](auto* a) {
+      k_scale<<<nblocks, 256, 0, s->stream>>>(a, g);
+      return QS_OK;
+    });
+    return launch_check("scale");
+  }
+
+  // Joint populations of q and the other qubits in `ahead` (distinct, q first).
+  int read_joint(const std::vector<int>& ahead) {
+    QS_TRY(apply_scales());
+    QS_TRY(flush());
+    jq = ahead;
+    joint.resize((size_t)1 << jq.size());
+    const int rc = marginal_host(s, jq.data(), (int)jq.size(), joint.data(), false);
+    if (rc != QS_OK) jq.clear();
+    return rc;
+  }
+
   int flush() {
     if (pending.empty()) return QS_OK;
     int rc = QS_OK;
@@ -262,58 +281,21 @@ struct Trajectory {
     return rc;
   }
 
-  int gram(int q, double G[4]) {
-    const uint64_t pairs = 1ull << (s->n - 1);
-    const int nblocks = (int)std::min<uint64_t>(608, std::max<uint64_t>(1, pairs / 512));
-    double* part = (double*)s->ws;
-    double* dres = part + (size_t)nblocks * 4;
-    KTimer kt(s, QS_K_REDUCE, 1, 1, 1ull << q, 0, (double)(pairs * 2), 8.0 * (double)pairs);
-    if (s->bound == 1) {  // components known to lie within the Q60 bound: exact integer sums
-      uint64_t* ipart = (uint64_t*)s->ws;
-      dres = (double*)(ipart + (size_t)nblocks * 8);
-      with_amps(s, [&](auto* a) {
-        using T = std::remove_cv_t<std::remove_pointer_t<decltype(a)>>;
-        k_gram_exact<<<nblocks, 256, 0, s->stream>>>((const T*)a, pairs, q, ipart);
-        return QS_OK;
-      });
-      QS_TRY(launch_check("gram"));
-      k_gram_exact_finish<<<1, 32, 0, s->stream>>>(ipart, nblocks, dres);
-      QS_TRY(launch_check("gram finish"));
-    } else {
-      with_amps(s, [&](auto* a) {
-        using T = std::remove_cv_t<std::remove_pointer_t<decltype(a)>>;
-        k_gram<<<nblocks, 256, 0, s->stream>>>((const T*)a, pairs, q, part);
-        return QS_OK;
-      });
-      QS_TRY(launch_check("gram"));
-      k_gram_finish<<<1, 32, 0, s->stream>>>(part, nblocks, dres);
-      QS_TRY(launch_check("gram finish"));
-    }
-    QS_TRY(ensure_pinned(s, 4 * sizeof(double)));
-    QS_CUDA(cudaMemcpyAsync(s->pinned, dres, 4 * sizeof(double), cudaMemcpyDeviceToHost, s->stream));
-    QS_CUDA(cudaStreamSynchronize(s->stream));
-    memcpy(G, s->pinned, 4 * sizeof(double));
-    return QS_OK;
-  }
-
-  int channel(const KrausSet& ks, int q) {
+  // ahead(): q and the qubits of the channels that follow, as far as one table serves them.
+  template <class F>
+  int channel(const KrausSet& ks, int q, F&& ahead) {
     double w[4] = {0, 0, 0, 0};
     if (ks.unital) {
       for (int j = 0; j < ks.m; ++j) w[j] = ks.w[j];
     } else {
-      QS_TRY(flush());
-      double G[4];
-      QS_TRY(gram(q, G));
-      // w_j = tr(K^dag K G), G = [[g00, g01], [conj(g01), g11]]
+      if (joint_bit(q) < 0) QS_TRY(read_joint(ahead()));
+      const int b = joint_bit(q);
+      double p[2] = {0.0, 0.0};
+      for (size_t k = 0; k < joint.size(); ++k) p[(k >> b) & 1] += joint[k];
       for (int j = 0; j < ks.m; ++j) {
         const Mat2& K = ks.K[j];
-        const double a00 = K.m[0].re * K.m[0].re + K.m[0].im * K.m[0].im + K.m[2].re * K.m[2].re + K.m[2].im * K.m[2].im;
-        const double a11 = K.m[1].re * K.m[1].re + K.m[1].im * K.m[1].im + K.m[3].re * K.m[3].re + K.m[3].im * K.m[3].im;
-        // (K^dag K)_{01} = conj(K00) K01 + conj(K10) K11
-        const double br = K.m[0].re * K.m[1].re + K.m[0].im * K.m[1].im + K.m[2].re * K.m[3].re + K.m[2].im * K.m[3].im;
-        const double bi = K.m[0].re * K.m[1].im - K.m[0].im * K.m[1].re + K.m[2].re * K.m[3].im - K.m[2].im * K.m[3].re;
-        // tr(B G) = B00 g00 + B11 g11 + 2 Re(B01 conj(g01))
-        w[j] = a00 * G[0] + a11 * G[1] + 2.0 * (br * G[2] + bi * G[3]);
+        w[j] = (K.m[0].re * K.m[0].re + K.m[2].re * K.m[2].re) * p[0] +
+               (K.m[1].re * K.m[1].re + K.m[3].re * K.m[3].re) * p[1];
       }
     }
     double W = 0.0;
@@ -337,13 +319,29 @@ struct Trajectory {
         g.q0 = q;
         g.q1 = -1;
         g.param_idx = -1;
-        pending.push_back(g);
+        return push(g, q, ks.pauli[pick] == 3);
       }
       return QS_OK;
     }
     Mat2 M = ks.K[pick];
     const double sc = 1.0 / sqrt(w[pick]);
     for (int e = 0; e < 4; ++e) M.m[e] = {M.m[e].re * sc, M.m[e].im * sc};
+    if (M.m[1].re == 0.0 && M.m[2].re == 0.0) {
+      const double f0 = M.m[0].re, f1 = M.m[3].re;
+      const int b = joint_bit(q);
+      for (size_t k = 0; k < joint.size(); ++k) joint[k] *= (k >> b) & 1 ? f1 * f1 : f0 * f0;
+      for (Scale& c : scales)
+        if (c.q == q) {
+          c.f0 *= f0;
+          c.f1 *= f1;
+          return QS_OK;
+        }
+      scales.push_back({q, f0, f1});
+      return scales.size() == JOINT_MAX ? apply_scales() : QS_OK;
+    }
+    QS_TRY(apply_scales());
+    QS_TRY(flush());
+    jq.clear();
     // A renormalised Kraus operator is not unitary, but the state it produces is
     // normalised: the Q60 kernel applies it when every entry has |re| + |im| < 1.9
     // (its Gauss-form sums then stay below 2, the limb range), e.g. the usual
@@ -379,6 +377,31 @@ extern "C" int qs_run_noisy(qs_state* s, const qs_gate* gates, size_t ng, const 
   tr.s = s;
   tr.fuse = fuse != 0;
   tr.seed = seed;
+  auto matches = [&](const qs_noise_rule& R, const qs_gate& g) {
+    return (R.gate_type < 0 || R.gate_type == g.type) && (R.q0 < 0 || R.q0 == g.q0) &&
+           (R.q1 < 0 || R.q1 == (two_qubit(g.type) ? g.q1 : -1));
+  };
+  // q, then the qubits that channels with weights touch from gate k on, until
+  // the table is full or a gate changes the populations of one of them
+  auto ahead = [&](size_t k, int q) {
+    std::vector<int> list{q};
+    uint64_t in = 1ull << q;
+    for (size_t j = k; j < ng; ++j) {
+      int t;
+      uint64_t cm;
+      if (gate_qubits(gates[j], s->n, &t, &cm) != QS_OK) break;
+      if (j > k && !structurally_diagonal(gates[j].type) && ((in >> t) & 1)) break;
+      for (size_t r = 0; r < nrules; ++r) {
+        if (sets[r].unital || !matches(rules[r], gates[j])) continue;
+        for (uint64_t b = (cm | (1ull << t)) & ~in; b; b &= b - 1) {
+          if (list.size() == JOINT_MAX) return list;
+          list.push_back(__builtin_ctzll(b));
+          in |= b & (0 - b);
+        }
+      }
+    }
+    return list;
+  };
   int rc = QS_OK;
   for (size_t k = 0; k < ng && rc == QS_OK; ++k) {
     qs_gate g = gates[k];
@@ -387,20 +410,19 @@ extern "C" int qs_run_noisy(qs_state* s, const qs_gate* gates, size_t ng, const 
       g.param_idx = -1;
     }
     if (rotation_error > 0.0 && is_rotation(g.type)) g.p[0] += rotation_error * (2.0 * tr.draw() - 1.0);
-    tr.pending.push_back(g);
     int t;
     uint64_t cm;
     if ((rc = gate_qubits(g, s->n, &t, &cm)) != QS_OK) break;
-    const int first = g.q0, second = two_qubit(g.type) ? g.q1 : -1;
-    const uint64_t touched = cm | (1ull << t);
+    if ((rc = tr.push(g, t, structurally_diagonal(g.type))) != QS_OK) break;
     for (size_t r = 0; r < nrules && rc == QS_OK; ++r) {
-      const qs_noise_rule& R = rules[r];
-      if (R.gate_type >= 0 && R.gate_type != g.type) continue;
-      if (R.q0 >= 0 && R.q0 != first) continue;
-      if (R.q1 >= 0 && R.q1 != second) continue;
-      for (uint64_t b = touched; b && rc == QS_OK; b &= b - 1) rc = tr.channel(sets[r], __builtin_ctzll(b));
+      if (!matches(rules[r], g)) continue;
+      for (uint64_t b = cm | (1ull << t); b && rc == QS_OK; b &= b - 1) {
+        const int q = __builtin_ctzll(b);
+        rc = tr.channel(sets[r], q, [&] { return ahead(k, q); });
+      }
     }
   }
+  if (rc == QS_OK) rc = tr.apply_scales();
   if (rc == QS_OK) rc = tr.flush();
   if (ndraws) *ndraws = tr.k;
   if (rc == QS_OK) QS_CUDA(cudaStreamSynchronize(s->stream));

@@ -68,12 +68,6 @@ uint64_t fingerprint(const qs_gate* g, size_t ng) {
   return h;
 }
 
-// Whether a record is diagonal for every angle: Z, S, T, RZ, P, CZ, CR (and I).
-bool structurally_diagonal(int type) {
-  return type == QS_I || type == QS_Z || type == QS_S || type == QS_T || type == QS_RZ || type == QS_P ||
-         type == QS_CZ || type == QS_CR;
-}
-
 // Cost model of the greedy planner (seconds): a pass costs the larger of its HBM
 // time and its arithmetic time.  Rates of the Q60 engine measured at n=30: a
 // tile pass runs ~5.2e12 limb products per second, a per-gate kernel streams at
@@ -122,6 +116,16 @@ double op_touch_fraction(const qs_gate& g, uint64_t cmask) {
 }
 
 }  // namespace
+
+namespace qs {
+
+// Whether a record is diagonal for every angle: Z, S, T, RZ, P, CZ, CR (and I).
+bool structurally_diagonal(int type) {
+  return type == QS_I || type == QS_Z || type == QS_S || type == QS_T || type == QS_RZ || type == QS_P ||
+         type == QS_CZ || type == QS_CR;
+}
+
+}  // namespace qs
 
 namespace qs {
 
