@@ -11,14 +11,15 @@
 //             E_b + (left-to-right partial sum of block b up to x) > u_s;
 //             if no block qualifies, the largest x with p_x > 0.
 // Kernels: block totals (one thread per block, sequential; the running sum is
-// also kept after every K = min(32, L) amplitudes), the superblock prefixes (one
+// also kept after every K amplitudes), the superblock prefixes (one
 // CTA per superblock, its sequential sum staged through shared memory), the
 // prefix of the superblock totals (one CTA), the offset of every superblock's
 // prefixes, and one thread per shot (binary search over E, then over the block's
-// running-sum checkpoints, then a sequential scan of at most K amplitudes that
+// running-sum checkpoints, then a sequential scan of at most K (8 or 32) amplitudes that
 // continues the block's left-to-right sum from the checkpoint before them: the
 // same additions in the same order as a scan from the block's start).
 #include <algorithm>
+#include <type_traits>
 
 #include "ieee_sq.h"
 #include "internal.h"
@@ -73,6 +74,72 @@ __global__ void k_block_totals(const A* __restrict__ a, int64_t nb, int64_t L, i
     cp[b * M + M - 1] = S;
     lastnz[b] = last;
   }
+}
+
+// The same for states of at least 32 blocks of 1024: a CTA takes 32 blocks, 32
+// amplitudes of each at a time.  Eight warps read whole rows (512 contiguous bytes)
+// and leave p in shared memory, a ninth adds: its lane keeps one block's running sum
+// and its checkpoints.  (One thread a block reads 16 bytes every
+// 16 KB and has all of a block's arithmetic between two of its additions.)
+// Bound by the FP64 pipe (1.5 additions an amplitude) and the integer pipes together.
+constexpr int TOT_B = 32, TOT_K = 32, TOT_L = 1024, TOT_PROD = 8;
+template <class A, int K>
+__global__ void __launch_bounds__(32 * (TOT_PROD + 1)) k_block_totals_rows(const A* __restrict__ a,
+                                                                           double* __restrict__ T,
+                                                                           long long* __restrict__ lastnz,
+                                                                           double* __restrict__ cp) {
+  constexpr int R = TOT_B / TOT_PROD;  // rows of a chunk per producer warp
+  constexpr int M = TOT_L / TOT_K;     // chunks
+  __shared__ double buf[2][TOT_B][TOT_K + 1];
+  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+  const int64_t b0 = (int64_t)blockIdx.x * TOT_B;
+  if (w < TOT_PROD) {
+    const A* row = a + (b0 + w * R) * TOT_L + l;
+    double2 v[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) v[r] = ld_amp(row, (uint64_t)r * TOT_L);
+    for (int c = 0; c < M; ++c) {
+      double2 nx[R];
+      const int cn = c + 1 < M ? c + 1 : c;  // the next chunk's loads are in flight meanwhile
+#pragma unroll
+      for (int r = 0; r < R; ++r) nx[r] = ld_amp(row, (uint64_t)r * TOT_L + cn * TOT_K);
+      double p[R];
+      bool ok = true;
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        bool o1, o2, o3 = true;
+        const double sr = sq_rn_int(v[r].x, &o1), si = sq_rn_int(v[r].y, &o2);
+        p[r] = (r & 1) ? __dadd_rn(sr, si) : add_rn_pos_int(sr, si, &o3);
+        ok = ok && o1 && o2 && o3;
+      }
+      if (!__all_sync(0xffffffffu, ok)) {
+#pragma unroll
+        for (int r = 0; r < R; ++r) p[r] = p_exact(v[r]);
+      }
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        buf[c & 1][w * R + r][l] = p[r];
+        v[r] = nx[r];
+      }
+      __syncthreads();
+    }
+    return;
+  }
+  double S = 0.0;
+  long long last = -1;
+  const int64_t b = b0 + l;
+  for (int c = 0; c < M; ++c) {
+    __syncthreads();  // chunk c is in its buffer; the producers fill the other one next
+#pragma unroll
+    for (int i = 0; i < TOT_K; ++i) {
+      const double q = buf[c & 1][l][i];
+      S = __dadd_rn(S, q);
+      if (__double_as_longlong(q) != 0) last = b * TOT_L + c * TOT_K + i;
+      if ((i + 1) % K == 0) cp[b * (TOT_L / K) + (c * TOT_K + i) / K] = S;
+    }
+  }
+  T[b] = S;
+  lastnz[b] = last;
 }
 
 // One CTA per segment c of G entries of T (a superblock of blocks, or the
@@ -175,11 +242,21 @@ __global__ void k_sample(const A* __restrict__ a, const double* __restrict__ E, 
     if (lo2 < M) {
       const A* p = a + b * L;
       double S = lo2 ? c[lo2 - 1] : 0.0;
-      for (int64_t j = lo2 * K; j < lo2 * K + K; ++j) {
-        S = __dadd_rn(S, p_exact(ld_amp(p, j)));
-        if (__dadd_rn(eb, S) > u) {
-          pick = b * L + j;
-          break;
+      // eight amplitudes (one 128-byte line) in flight at a time
+      const int64_t end = lo2 * K + K;
+      bool found = false;
+      for (int64_t j = lo2 * K; j < end && !found; j += 8) {
+        double2 v[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) v[k] = ld_amp(p, j + k < end ? j + k : j);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+          if (found || j + k >= end) break;
+          S = __dadd_rn(S, p_exact(v[k]));
+          if (__dadd_rn(eb, S) > u) {
+            pick = b * L + j + k;
+            found = true;
+          }
         }
       }
     }
@@ -209,8 +286,13 @@ extern "C" int qs_sample(const qs_state* cs, uint64_t seed, uint64_t shots, uint
   double* P = Ssb + (nsb + 1);                 // superblock prefixes
   long long* lsb = (long long*)(P + (nsb + 1));
   long long* lall = lsb + (nsb + 1);
-  const int64_t K = L < 32 ? L : 32;  // amplitudes per running-sum checkpoint
-  const size_t cp_count = (size_t)(N / K);  // 1/64 of the state's bytes
+  // amplitudes per running-sum checkpoint: 8 where they stay within 128 MiB (a shot then
+  // reads and adds one 128-byte line; with 32, 16 amplitudes on average at two FP64
+  // additions and a square each, 10^6 shots of 2^26 amplitudes take 442 us), else 32
+  // (1/64 of the state's bytes)
+  const bool rows = nb >= TOT_B;
+  const int64_t K = rows && s->n <= 27 ? 8 : (L < 32 ? L : 32);
+  const size_t cp_count = (size_t)(N / K);
   ScratchBuf buf;                           // the checkpoints, then the shots
   QS_TRY(take_scratch(s, cp_count * sizeof(double) + (on_device ? 0 : shots * sizeof(uint64_t)), &buf));
   double* cp = (double*)buf.p;
@@ -218,7 +300,12 @@ extern "C" int qs_sample(const qs_state* cs, uint64_t seed, uint64_t shots, uint
   KTimer kt(s, QS_K_REDUCE, s->n, 3, 0, 0, (double)N, 4.0 * (double)N);
   note_launch(4);
   with_amps(s, [&](auto* a) {
-    k_block_totals<<<g1, 128, 0, s->stream>>>(a, nb, L, K, T, lastnz, cp);
+    using A = std::remove_cv_t<std::remove_pointer_t<decltype(a)>>;
+    const unsigned gr = (unsigned)(nb / TOT_B);
+    if (rows && K == 8) k_block_totals_rows<A, 8><<<gr, 32 * (TOT_PROD + 1), 0, s->stream>>>(a, T, lastnz, cp);
+    else if (rows) k_block_totals_rows<A, 32><<<gr, 32 * (TOT_PROD + 1), 0, s->stream>>>(a, T, lastnz, cp);
+    else
+      k_block_totals<<<g1, 128, 0, s->stream>>>(a, nb, L, K, T, lastnz, cp);
     return QS_OK;
   });
   QS_TRY(launch_check("block_totals"));
