@@ -718,17 +718,198 @@ __global__ void __launch_bounds__(256, 3) k_pauli_tile(const A* __restrict__ a, 
   }
 }
 
-// sums[k] = the CTA partials of slot k added (modulo 2^128), CTA k of this kernel
-__global__ void __launch_bounds__(256) k_pauli_exact_finish(const uint64_t* __restrict__ part, int nblocks,
-                                                            uint64_t* __restrict__ sums) {
+// Slots whose X mask is one coordinate of the tile's basis and that carry no Z (the
+// field terms of a transverse-field chain; Re w over all pairs), all twelve of a tile
+// in one visit.  A thread holds 16 amplitudes that span four coordinates in registers
+// and forms the 8 pairs of each from there; two exchanges through shared memory bring
+// the other eight coordinates.  Limbs of 30 bits (v = h 2^30 + l, |l| <= 2^29) let the
+// 16 products of a coordinate add up in three int64 columns
+//   sum h h' <= 1.5625 2^60,  sum h l' + l h' < 2^62.9,  sum l l' <= 2^62
+// and join the 128-bit sum once per coordinate and tile: 8 multiply-adds a pair and
+// little else (k_pauli_tile combines and adds 128 bits for every pair, and reads it
+// from shared memory: 540 us for 12 slots at n = 25).
+struct PXArgs {
+  uint64_t ntiles;
+  int lead[PT_TMAX];
+  uint64_t bm[PT_TMAX];
+  uint32_t want;  // coordinates whose slots are asked for
+};
+
+__device__ __forceinline__ Sp split30(int64_t v) {
+  const int64_t h = (v + (1ll << 29)) >> 30;
+  return {(int32_t)h, (int32_t)(v - h * (1ll << 30))};
+}
+
+__device__ __forceinline__ uint32_t px_slot(uint32_t e) { return e ^ ((e >> 4) & 7u); }  // bank spread
+
+// The pair sums of the four coordinates that the 16 amplitudes span.
+template <int FIRST>
+__device__ __forceinline__ void px_stage(const int4 (&v)[16], uint32_t want, u128 (&acc)[PT_TMAX]) {
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    if (!((want >> (FIRST + j)) & 1)) continue;
+    int64_t A = 0, B = 0, C = 0;
+#pragma unroll
+    for (int k = 0; k < 16; ++k) {
+      if (k & (1 << j)) continue;
+      const int4 x = v[k], y = v[k | (1 << j)];
+      A = madw(x.z, y.z, madw(x.x, y.x, A));
+      B = madw(x.x, y.y, madw(x.y, y.x, B));
+      B = madw(x.z, y.w, madw(x.w, y.z, B));
+      C = madw(x.w, y.w, madw(x.y, y.y, C));
+    }
+    acc[FIRST + j] += ((u128)(__int128)A << 60) + ((u128)(__int128)B << 30) + (u128)(__int128)C;
+  }
+}
+
+template <class A>
+__global__ void __launch_bounds__(256, 2) k_pauli_x(const A* __restrict__ a, const PXArgs g,
+                                                    uint64_t* __restrict__ part) {
+  extern __shared__ int4 tile[];  // 4096 entries (r.h, r.l, i.h, i.l)
   __shared__ uint64_t sh[8][2];
-  const int k = blockIdx.x;
+  const uint32_t t = threadIdx.x;
+  u128 acc[PT_TMAX];
+#pragma unroll
+  for (int i = 0; i < PT_TMAX; ++i) acc[i] = 0;
+  uint64_t st = 0;
+#pragma unroll
+  for (int i = 0; i < 8; ++i)
+    if ((t >> i) & 1) st ^= g.bm[i];
+  for (uint64_t c = blockIdx.x; c < g.ntiles; c += gridDim.x) {
+    uint64_t base = c;
+#pragma unroll
+    for (int i = 0; i < PT_TMAX; ++i) base = insert0(base, g.lead[i]);
+    int4 v[16];
+#pragma unroll
+    for (int h = 0; h < 16; h += 8) {
+      double2 d[8];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        uint64_t x = base ^ st;
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          if (((h + k) >> j) & 1) x ^= g.bm[8 + j];
+        d[k] = ld_amp(a, x);
+      }
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        const Sp r = split30(q60_from_double_nb(d[k].x)), i = split30(q60_from_double_nb(d[k].y));
+        v[h + k] = make_int4(r.h, r.l, i.h, i.l);
+      }
+    }
+    __syncthreads();  // the last tile's readers are done
+#pragma unroll
+    for (int k = 0; k < 16; ++k) tile[px_slot(t | (k << 8))] = v[k];
+    px_stage<8>(v, g.want, acc);
+    __syncthreads();
+    if (g.want & 0xf0) {
+#pragma unroll
+      for (int k = 0; k < 16; ++k) v[k] = tile[px_slot((t & 15) | (k << 4) | ((t >> 4) << 8))];
+      px_stage<4>(v, g.want, acc);
+    }
+    if (g.want & 0xf) {
+#pragma unroll
+      for (int k = 0; k < 16; ++k) v[k] = tile[px_slot(k | (t << 4))];
+      px_stage<0>(v, g.want, acc);
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < PT_TMAX; ++i) {
+    const u128 s = block_sum_u128(acc[i], sh);
+    if (t == 0) {
+      part[((size_t)blockIdx.x * PT_TMAX + i) * 2] = (uint64_t)s;
+      part[((size_t)blockIdx.x * PT_TMAX + i) * 2 + 1] = (uint64_t)(s >> 64);
+    }
+  }
+}
+
+// |a|^2 slots: pos = (sum p + sum (-1)^popc(x & zm) p) / 2.  A thread forms p of eight
+// amplitudes (index bits 8..10), their eight signed sums (a Walsh-Hadamard transform
+// in registers), and adds to every slot the one that its zm selects, with the sign of
+// the bits above: a slot costs one 128-bit addition per eight amplitudes.  The sign of
+// bits 0..7 is the thread's own and comes last.
+constexpr int PZ_MAX = 13;  // slots per launch (their sums stay in registers)
+struct PZArgs {
+  uint64_t ntiles;  // 2^(n - 11)
+  int nt;
+  uint64_t zm[PZ_MAX];
+};
+
+template <class A>
+__global__ void __launch_bounds__(256, 2) k_pauli_z(const A* __restrict__ a, const PZArgs g,
+                                                    uint64_t* __restrict__ part) {
+  __shared__ uint4 w[8][256];
+  __shared__ uint64_t sh[8][2];
+  const uint32_t t = threadIdx.x;
+  u128 acc[PZ_MAX], tot = 0;
+#pragma unroll
+  for (int k = 0; k < PZ_MAX; ++k) acc[k] = 0;
+  for (uint64_t c = blockIdx.x; c < g.ntiles; c += gridDim.x) {
+    const uint64_t base = c << 11;
+    double2 d[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) d[k] = ld_amp(a, base + t + (k << 8));
+    u128 p[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const Sp r = split31(q60_from_double_nb(d[k].x)), i = split31(q60_from_double_nb(d[k].y));
+      p[k] = dot2_exact(r, r, i, i);
+    }
+#pragma unroll
+    for (int b = 1; b < 8; b <<= 1)
+#pragma unroll
+      for (int k = 0; k < 8; ++k)
+        if (!(k & b)) {
+          const u128 x = p[k], y = p[k | b];
+          p[k] = x + y;
+          p[k | b] = x - y;
+        }
+    tot += p[0];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {  // read back by this thread only
+      const uint64_t lo = (uint64_t)p[k], hi = (uint64_t)(p[k] >> 64);
+      w[k][t] = make_uint4((uint32_t)lo, (uint32_t)(lo >> 32), (uint32_t)hi, (uint32_t)(hi >> 32));
+    }
+#pragma unroll
+    for (int k = 0; k < PZ_MAX; ++k) {
+      if (k < g.nt) {
+        const uint4 q = w[(g.zm[k] >> 8) & 7][t];
+        const u128 v = ((u128)(((uint64_t)q.w << 32) | q.z) << 64) | (((uint64_t)q.y << 32) | q.x);
+        if (__popcll(base & g.zm[k]) & 1) acc[k] -= v;
+        else acc[k] += v;
+      }
+    }
+  }
+  const u128 T = block_sum_u128(tot, sh);
+#pragma unroll
+  for (int k = 0; k < PZ_MAX; ++k) {
+    if (k < g.nt) {
+      const bool neg = __popc(t & (uint32_t)g.zm[k] & 0xffu) & 1;
+      const u128 S = block_sum_u128(neg ? 0 - acc[k] : acc[k], sh);
+      if (t == 0) {
+        const u128 pos = (T + S) >> 1;  // T + S = 2 pos >= 0
+        part[((size_t)blockIdx.x * PZ_MAX + k) * 2] = (uint64_t)pos;
+        part[((size_t)blockIdx.x * PZ_MAX + k) * 2 + 1] = (uint64_t)(pos >> 64);
+      }
+    }
+  }
+}
+
+// sums[2 k] = the CTA partials of one slot added (modulo 2^128), CTA k of this kernel
+// for the slot at slot[k] of a CTA's `stride` partials.
+struct PFinish {
+  int8_t slot[PZ_MAX];
+};
+__global__ void __launch_bounds__(256) k_pauli_exact_finish(const uint64_t* __restrict__ part, int nblocks, int stride,
+                                                            const PFinish f, uint64_t* __restrict__ sums) {
+  __shared__ uint64_t sh[8][2];
+  const int k = f.slot[blockIdx.x];
   u128 t = 0;
-  for (int b = threadIdx.x; b < nblocks; b += 256) t += ld_u128(part + ((size_t)b * PS_MAX + k) * 2);
+  for (int b = threadIdx.x; b < nblocks; b += 256) t += ld_u128(part + ((size_t)b * stride + k) * 2);
   t = block_sum_u128(t, sh);
   if (threadIdx.x == 0) {
-    sums[2 * k] = (uint64_t)t;
-    sums[2 * k + 1] = (uint64_t)(t >> 64);
+    sums[2 * blockIdx.x] = (uint64_t)t;
+    sums[2 * blockIdx.x + 1] = (uint64_t)(t >> 64);
   }
 }
 
@@ -1024,7 +1205,7 @@ static int pauli_exact(qs_state* s, const qs_pauli* terms, size_t nterms, double
     const size_t nslots = slots.size();
     std::vector<int> gidx(nslots, -1);
     uint64_t* part = (uint64_t*)s->ws;
-    const size_t part_words = (size_t)1216 * PS_MAX * 2;
+    const size_t part_words = (size_t)1216 * PZ_MAX * 2;
     uint64_t* sums = part + part_words;
     if ((part_words + 2 * nslots) * sizeof(uint64_t) > s->ws_bytes)
       return fail(QS_ERR_UNSUPPORTED, "Pauli slot sums exceed the workspace");
@@ -1032,21 +1213,90 @@ static int pauli_exact(qs_state* s, const qs_pauli* terms, size_t nterms, double
     std::call_once(smem_once, [] {
       cudaFuncSetAttribute(k_pauli_tile<double2>, cudaFuncAttributeMaxDynamicSharedMemorySize, 16 << PT_TMAX);
       cudaFuncSetAttribute(k_pauli_tile<float2>, cudaFuncAttributeMaxDynamicSharedMemorySize, 16 << PT_TMAX);
+      cudaFuncSetAttribute(k_pauli_x<double2>, cudaFuncAttributeMaxDynamicSharedMemorySize, 16 << PT_TMAX);
+      cudaFuncSetAttribute(k_pauli_x<float2>, cudaFuncAttributeMaxDynamicSharedMemorySize, 16 << PT_TMAX);
     });
     int next = 0;
+    // adds the partials of `count` slots (at f.slot[] of a CTA's) into sums[next ..]
+    auto finish = [&](int nblocks, int stride, const PFinish& f, int count) {
+      k_pauli_exact_finish<<<count, 256, 0, s->stream>>>(part, nblocks, stride, f, sums + 2 * (size_t)next);
+      next += count;
+      return launch_check("pauli_exact_finish");
+    };
+    // From 16 qubits on, field slots and |a|^2 slots have kernels of their own (below
+    // that, a state has too few tiles to fill the GPU with them).
+    const bool own = n >= 16;
+    if (own) {
+      std::vector<int> zs;
+      for (const auto& P : passes)
+        for (int k : P.sl)
+          if (!slots[k].xm) zs.push_back(k);
+      for (size_t z0 = 0; z0 < zs.size(); z0 += PZ_MAX) {
+        PZArgs g{};
+        PFinish f{};
+        g.ntiles = 1ull << (n - 11);
+        g.nt = (int)std::min<size_t>(PZ_MAX, zs.size() - z0);
+        for (int k = 0; k < g.nt; ++k) {
+          g.zm[k] = slots[zs[z0 + k]].zm;
+          gidx[zs[z0 + k]] = next + k;
+          f.slot[k] = (int8_t)k;
+        }
+        const int nblocks = (int)std::min<uint64_t>(2 * 152, g.ntiles);
+        KTimer kt(s, QS_K_REDUCE, n, g.nt, 0, 0, (double)(1ull << n), 8.0 * g.nt * (double)(1ull << n));
+        note_launch(2);
+        with_amps(s, [&](auto* a) {
+          using T = std::remove_cv_t<std::remove_pointer_t<decltype(a)>>;
+          k_pauli_z<T><<<nblocks, 256, 0, s->stream>>>(a, g, part);
+          return QS_OK;
+        });
+        QS_TRY(launch_check("pauli_z"));
+        QS_TRY(finish(nblocks, PZ_MAX, f, g.nt));
+      }
+    }
     for (const auto& P : passes) {
+      PXArgs gx{};
+      PFinish fx{};
+      int nx = 0;
       PTile g{};
       g.T = (int)P.bm.size();
-      g.ntiles = 1ull << (n - g.T);
+      g.ntiles = gx.ntiles = 1ull << (n - g.T);
       for (int q = 0; q < g.T; ++q) {
-        g.bm[q] = P.bm[q];
-        g.lead[q] = pp_lead(P.bm[q]);
+        g.bm[q] = gx.bm[q] = P.bm[q];
+        g.lead[q] = gx.lead[q] = pp_lead(P.bm[q]);
       }
-      g.nt = (int)P.sl.size();
-      g.nz = 0;
+      PFinish f{};
+      std::vector<int> left;  // slots for k_pauli_tile
+      for (int k : P.sl) {
+        const PauliSlot& sl = slots[k];
+        if (own && !sl.xm) continue;
+        uint32_t xc = 0;
+        if (sl.xm) pp_reduce(P.bm, sl.xm, &xc);
+        if (own && !sl.zm && !sl.im && (xc & (xc - 1)) == 0) {
+          gidx[k] = next + nx;
+          fx.slot[nx++] = (int8_t)(31 - __builtin_clz(xc));
+          gx.want |= xc;
+        } else {
+          left.push_back(k);
+        }
+      }
+      if (nx) {
+        const int nblocks = (int)std::min<uint64_t>(2 * 152, gx.ntiles);
+        KTimer kt(s, QS_K_REDUCE, n, nx, 0, 0, (double)(1ull << n), 8.0 * nx * (double)(1ull << n));
+        note_launch(2);
+        with_amps(s, [&](auto* a) {
+          using T = std::remove_cv_t<std::remove_pointer_t<decltype(a)>>;
+          k_pauli_x<T><<<nblocks, 256, (size_t)16 << PT_TMAX, s->stream>>>(a, gx, part);
+          return QS_OK;
+        });
+        QS_TRY(launch_check("pauli_x"));
+        QS_TRY(finish(nblocks, PT_TMAX, fx, nx));
+      }
+      if (left.empty()) continue;
+      g.nt = (int)left.size();
       for (int q = 0; q < g.nt; ++q) {
-        const PauliSlot& sl = slots[P.sl[q]];
-        gidx[P.sl[q]] = next + q;
+        const PauliSlot& sl = slots[left[q]];
+        gidx[left[q]] = next + q;
+        f.slot[q] = (int8_t)q;
         g.zm[q] = sl.zm;
         g.im[q] = (uint8_t)sl.im;
         uint32_t zc = 0;
@@ -1072,9 +1322,7 @@ static int pauli_exact(qs_state* s, const qs_pauli* terms, size_t nterms, double
         return QS_OK;
       });
       QS_TRY(launch_check("pauli_tile"));
-      k_pauli_exact_finish<<<g.nt, 256, 0, s->stream>>>(part, nblocks, sums + 2 * (size_t)next);
-      QS_TRY(launch_check("pauli_exact_finish"));
-      next += g.nt;
+      QS_TRY(finish(nblocks, PS_MAX, f, g.nt));
     }
     std::vector<uint64_t> hs(2 * nslots);
     if (nslots) QS_TRY(read_back(s, (const double*)sums, 2 * nslots, (double*)hs.data()));
