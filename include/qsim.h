@@ -203,7 +203,9 @@ int qs_state_modified(qs_state* s);
 /* Apply gates[0..ng-1] in order.  params (host, may be NULL if no record has
  * param_idx >= 0) supplies theta for parametrised records; param_idx must be
  * < the caller's params length (not checkable: the caller guarantees it).
- * plan == NULL: one kernel per gate (plain mode).  Otherwise the plan must have
+ * plan == NULL: the gates run in passes that the call plans for itself, or one
+ * kernel per gate (plain mode) where the timing log is on, arithmetic is FP64 or
+ * there is one gate only.  Otherwise the plan must have
  * been created from exactly this gate list and qubit count; its passes are run
  * (fused mode) with matrices computed from `params` at this call.
  * Every record is validated before any work is queued: a bad record returns

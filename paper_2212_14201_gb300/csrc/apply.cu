@@ -463,9 +463,6 @@ int launch_dense(qs_state* s, const int* targets, int k, uint64_t cmask, const C
 
 using namespace qs;
 
-int qs_apply_plan(qs_state* s, const qs_gate* gates, size_t ng, const double* params, const qs_plan* plan,
-                  bool fixed);
-
 extern "C" int qs_apply(qs_state* s, const qs_gate* gates, size_t ng, const double* params, const qs_plan* plan) {
   clear_error();
   QS_TRY(check_state(s));
@@ -473,6 +470,19 @@ extern "C" int qs_apply(qs_state* s, const qs_gate* gates, size_t ng, const doub
   bool fixed = false;
   QS_TRY(choose_fixed(s, &fixed));
   if (plan) return qs_apply_plan(s, gates, ng, params, plan, fixed);
+  // Two gates or more run as greedy tile passes planned here (3 us for 20 gates, 30
+  // for 600): a kernel per gate is a launch of 4 us each on small states and a sweep
+  // of HBM each on large ones.  Per gate stay FP64 arithmetic and a state whose
+  // timing log is on (its user asks for the gates one by one).
+  if (ng > 1 && !s->timing && (fixed || s->prec == 64)) {
+    qs_plan* p = nullptr;
+    if (plan_implicit(s->n, s->prec, gates, ng, &p) == QS_OK) {
+      const int rc = qs_apply_plan(s, gates, ng, params, p, fixed);
+      qs_plan_free(p);
+      return rc;
+    }
+    clear_error();  // no host memory for a plan
+  }
   for (size_t k = 0; k < ng; ++k) {
     int t;
     uint64_t cm;

@@ -162,6 +162,9 @@ int unit_code(const C2& z);
 // Whether the next gate kernels of this state run in Q60 fixed point (may
 // synchronise once to bound an unknown state's magnitude).
 int choose_fixed(qs_state* s, bool* fixed);
+// Buffer conversions in place: complex128 to Q60 integer pairs, and back.
+int launch_q60_hold(qs_state* s);
+int launch_q60_release(qs_state* s);
 int launch_op1(qs_state* s, const Op1& op, bool fixed);  // complex64 states: FP32 arithmetic
 int launch_dense(qs_state* s, const int* targets, int k, uint64_t cmask, const C2* mat);
 
@@ -222,3 +225,10 @@ int take_scratch(qs_state* s, size_t bytes, ScratchBuf* out, bool keep = true);
 int ensure_pinned(qs_state* s, size_t bytes);
 
 }  // namespace qs
+
+// The passes that qs_apply runs for a gate list without a plan.
+int plan_implicit(int n, int prec, const qs_gate* gates, size_t ng, qs_plan** out);
+// qs_apply with a plan.  held != nullptr: the amplitudes may stay Q60 integers after a
+// last tile pass (*held says so); else they are complex128 when the call returns.
+int qs_apply_plan(qs_state* s, const qs_gate* gates, size_t ng, const double* params, const qs_plan* plan,
+                  bool fixed, bool* held = nullptr);

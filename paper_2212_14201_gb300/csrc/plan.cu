@@ -47,6 +47,9 @@ struct qs_plan {
   std::vector<PlanPass> passes;
   double est_seconds = 0.0;
   int64_t n_tile = 0;
+  // Every gate as its own op with its own matrix: no products of matrices or phases,
+  // which would add double rounding of their own (see plan_implicit).
+  bool direct = false;
 };
 
 namespace {
@@ -792,7 +795,7 @@ static PlanPass make_pass(const qs_gate* gates, const std::vector<int>& tgt, con
 }
 
 static int plan_build(int n, const qs_gate* gates, size_t ng, int mode, int kmax, int mtile, qs_plan** out,
-                      int strategy = 0) {
+                      int strategy = 0, bool few_launches = false) {
   if (!out) return fail(QS_ERR_INVALID_ARG, "out is NULL");
   *out = nullptr;
   if (n < 1 || n > QS_MAX_QUBITS) return fail(QS_ERR_INVALID_ARG, "n out of range");
@@ -850,7 +853,7 @@ static int plan_build(int n, const qs_gate* gates, size_t ng, int mode, int kmax
       plain += pass_bytes * f / (kPlainHbmFraction * kHbmBytesPerS);
     }
     const double tile_cost = std::max(pass_bytes / kHbmBytesPerS, limbs / kTileLimbPerS);
-    if (ps.gates.size() == 1 || plain <= tile_cost) {
+    if (!few_launches && (ps.gates.size() == 1 || plain <= tile_cost)) {
       for (uint32_t k : ps.gates) {
         PlanPass g1;
         g1.kind = PASS_GATE;
@@ -867,6 +870,22 @@ static int plan_build(int n, const qs_gate* gates, size_t ng, int mode, int kmax
     remaining.swap(rest);
   }
   *out = p;
+  return QS_OK;
+}
+
+// The plan of a qs_apply without one.  Below 24 qubits the passes run every gate with
+// its own matrix: a fused pass's products of matrices and phases round to double, and
+// on amplitudes that large this error exceeds the 2^-60 resolution of the arithmetic
+// (relative error of 300 random gates at n = 12: per gate 8.4e-16, so 7.2e-16, fused
+// 1.8e-15; at n = 24 6.3e-15, 5.8e-15, 4.9e-15).  Tiles are narrow on small states, so
+// that several SMs share a pass (one SM takes 1 us for a gate on 2^12 amplitudes and a
+// launch 4 us).  complex64 states gain from fusion at any size.
+int plan_implicit(int n, int prec, const qs_gate* gates, size_t ng, qs_plan** out) {
+  if (n >= 24 || prec == 64) return plan_build(n, gates, ng, QS_PLAN_GREEDY, 5, TILE_DEFAULT_M, out);
+  const int m = n <= 10 ? n : std::min(TILE_DEFAULT_M, std::max(9, n - 6));
+  // (below 20 qubits a launch costs more than any sweep it saves: no per-gate passes)
+  QS_TRY(plan_build(n, gates, ng, QS_PLAN_GREEDY, 5, m, out, 0, n < 20));
+  (*out)->direct = true;
   return QS_OK;
 }
 
@@ -1216,7 +1235,8 @@ extern "C" int qs_plan_pass_info(const qs_plan* p, size_t pass, int* kind, uint6
 }
 
 static int build_pass_ops(int n, const PlanPass& ps, const qs_gate* gates, const double* params, bool tables_ok,
-                          std::vector<Op1>* rops, std::vector<PhaseTable>* ptables, int* local, int* m_out);
+                          std::vector<Op1>* rops, std::vector<PhaseTable>* ptables, int* local, int* m_out,
+                          bool direct = false);
 
 extern "C" int qs_plan_pass_ops(const qs_plan* p, size_t pass, const qs_gate* gates, size_t ng, const double* params,
                                 int q60, qs_pass_op* ops, size_t cap, size_t* count, double* tables,
@@ -1380,7 +1400,8 @@ static int build_tables(qs_state* s, const std::vector<PhaseTable>& pt, const QL
 // engine) general ops split into real rotations and phase tables.  local[b] is
 // the tile bit of qubit b (-1 outside the tile), *m the tile width.
 static int build_pass_ops(int n, const PlanPass& ps, const qs_gate* gates, const double* params, bool tables_ok,
-                          std::vector<Op1>* rops, std::vector<PhaseTable>* ptables, int* local, int* m_out) {
+                          std::vector<Op1>* rops, std::vector<PhaseTable>* ptables, int* local, int* m_out,
+                          bool direct) {
   int m = 0;
   for (int b = 0; b < 64; ++b) local[b] = -1;
   for (int b = 0; b < n; ++b)
@@ -1389,7 +1410,7 @@ static int build_pass_ops(int n, const PlanPass& ps, const qs_gate* gates, const
   rops->clear();
   ptables->clear();
   int merged = 0;
-  if (g_aggregate) {
+  if (g_aggregate && !direct) {
     QS_TRY(aggregate_pass(n, ps, gates, params, rops, &merged));
   } else {
     for (uint32_t k : ps.gates) {
@@ -1402,7 +1423,7 @@ static int build_pass_ops(int n, const PlanPass& ps, const qs_gate* gates, const
       if (op.cls != OP_IDENTITY) rops->push_back(op);
     }
   }
-  if (tables_ok && g_aggregate && g_phase_tables) {
+  if (tables_ok && g_aggregate && g_phase_tables && !direct) {
     std::vector<Op1> x;
     std::vector<PhaseTable> t;
     extract_phases(*rops, local, n, m, &x, &t);
@@ -1421,13 +1442,13 @@ static int build_pass_ops(int n, const PlanPass& ps, const qs_gate* gates, const
 // limb products.
 static int build_tile_args(int n, int prec, const PlanPass& ps, const qs_gate* gates, const double* params,
                            bool fixed, int io, TileArgs* g, std::vector<PhaseTable>& ptables, double* flops_out,
-                           double* int_ops_out) {
+                           double* int_ops_out, bool direct = false) {
   const uint64_t Q = ps.qmask;
   int local[64];
   int m = 0;
   std::vector<Op1> rops;
   const bool f32 = prec == 64;  // complex64 state: FP32 engine
-  int rc = build_pass_ops(n, ps, gates, params, (fixed && prec == 128) || f32, &rops, &ptables, local, &m);
+  int rc = build_pass_ops(n, ps, gates, params, (fixed && prec == 128) || f32, &rops, &ptables, local, &m, direct);
   int L = 0;
   while (L < n && ((Q >> L) & 1)) ++L;
   g->n = n;
@@ -1444,7 +1465,7 @@ static int build_tile_args(int n, int prec, const PlanPass& ps, const qs_gate* g
   g->tables = nullptr;
   double flops = 0.0, int_ops = 0.0;
   const double N = (double)(1ull << n);
-  const bool pairs = ((fixed && prec == 128) || f32) && g_rotation_pairs;
+  const bool pairs = ((fixed && prec == 128) || f32) && g_rotation_pairs && !direct;
   const bool triples = g_rotation_triples;
   const bool quads = g_rotation_quads;
   auto in_tile_real = [&](const Op1& o) { return o.cls == OP_REAL && o.cmask == 0 && local[o.target] >= 0; };
@@ -1736,13 +1757,13 @@ static int build_tile_args(int n, int prec, const PlanPass& ps, const qs_gate* g
 // io: TileArgs::io (Q60 engine only); *launched: whether a kernel ran (a pass
 // whose ops all cancel launches nothing).
 static int run_tile_pass(qs_state* s, const PlanPass& ps, const qs_gate* gates, const double* params, bool fixed,
-                         int io, bool* launched) {
+                         int io, bool* launched, bool direct) {
   *launched = false;
   TileArgs* g = new (std::nothrow) TileArgs;
   if (!g) return fail(QS_ERR_OOM, "host allocation failed");
   std::vector<PhaseTable> ptables;
   double flops = 0.0, int_ops = 0.0;
-  int rc = build_tile_args(s->n, s->prec, ps, gates, params, fixed, io, g, ptables, &flops, &int_ops);
+  int rc = build_tile_args(s->n, s->prec, ps, gates, params, fixed, io, g, ptables, &flops, &int_ops, direct);
   if (rc == QS_OK && !ptables.empty()) rc = build_tables(s, ptables, &g->tables, s->prec == 64);
   if (rc == QS_OK && (g->nops > 0 || (g->io >> 8) != 0)) {
     rc = launch_tile(s, *g, fixed ? 0.0 : flops, fixed ? int_ops : 0.0, (int)ps.gates.size(), fixed);
@@ -1792,7 +1813,7 @@ extern "C" int qs_plan_pass_kernel_ops(const qs_plan* p, size_t pass, const qs_g
 }
 
 int qs_apply_plan(qs_state* s, const qs_gate* gates, size_t ng, const double* params, const qs_plan* plan,
-                  bool fixed) {
+                  bool fixed, bool* held_out) {
   if (plan->n != s->n || plan->ng != ng || plan->fingerprint != fingerprint(gates, ng))
     return fail(QS_ERR_INVALID_ARG, "plan does not match the program");
   // Between consecutive Q60 tile passes the buffer keeps the Q60 integers (the
@@ -1815,12 +1836,15 @@ int qs_apply_plan(qs_state* s, const qs_gate* gates, size_t ng, const double* pa
       QS_TRY(gate_matrix(g, params, &m));
       QS_TRY(launch_op1(s, classify(t, cm, m), fixed));
     } else {
-      const bool next_tile = q60 && i + 1 < plan->passes.size() && plan->passes[i + 1].kind == PASS_TILE;
+      const bool last = i + 1 == plan->passes.size();
+      const bool next_tile = q60 && (last ? held_out != nullptr : plan->passes[i + 1].kind == PASS_TILE);
       bool launched = false;
-      QS_TRY(run_tile_pass(s, ps, gates, params, fixed, (held ? 1 : 0) | (next_tile ? 2 : 0), &launched));
+      QS_TRY(run_tile_pass(s, ps, gates, params, fixed, (held ? 1 : 0) | (next_tile ? 2 : 0), &launched,
+                           plan->direct));
       if (launched) held = next_tile;
     }
   }
-  if (held) QS_TRY(launch_q60_release(s));
+  if (held_out) *held_out = held;
+  else if (held) QS_TRY(launch_q60_release(s));
   return QS_OK;
 }

@@ -820,12 +820,13 @@ static int launch_engine_t(qs_state* s, const TileArgs& g, size_t smem) {
 
 // 256 threads per CTA (measured at n=30, 12-qubit tiles: 512 threads with 2 CTAs
 // per SM and 1024 with one are 2-6 % slower); a 13-qubit tile (one CTA per SM)
-// runs 512 threads.
+// runs 512 threads, and so does a pass of at most one tile of 11 qubits or more per
+// SM, where a CTA has the SM to itself.
 template <class E>
 static int launch_engine(qs_state* s, const TileArgs& g) {
   const size_t H = (size_t)1 << g.nhigh;
   const size_t smem = ((H * sizeof(uint64_t) + 15) & ~(size_t)15) + (sizeof(typename E::T) << g.m);
-  if (g.m >= 13) return launch_engine_t<E, 512>(s, g, smem);
+  if (g.m >= 13 || (g.m >= 11 && g.ntiles <= 152)) return launch_engine_t<E, 512>(s, g, smem);
   return launch_engine_t<E, 256>(s, g, smem);
 }
 
