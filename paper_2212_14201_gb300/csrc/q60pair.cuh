@@ -89,16 +89,6 @@ __device__ __forceinline__ void q60_pair_quad_t(longlong2& q0, longlong2& q1, lo
   q3 = make_longlong2(r3, i3);
 }
 
-// The quad (q0, q1, q2, q3) = indices bit(a) + 2 bit(b); flags as above.
-__device__ __forceinline__ void q60_pair_quad(longlong2& q0, longlong2& q1, longlong2& q2, longlong2& q3,
-                                              const QL* __restrict__ c, int flags) {
-  switch (flags) {
-    case 0: q60_pair_quad_t<0>(q0, q1, q2, q3, c); break;
-    case 1: q60_pair_quad_t<1>(q0, q1, q2, q3, c); break;
-    case 2: q60_pair_quad_t<2>(q0, q1, q2, q3, c); break;
-    default: q60_pair_quad_t<3>(q0, q1, q2, q3, c); break;
-  }
-}
 #endif
 
 // Three real rotations on tile bits a, b, c, applied to an amplitude octet

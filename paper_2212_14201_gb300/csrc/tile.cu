@@ -164,6 +164,43 @@ struct EngQ60 {
   }
 };
 
+// Two FP32 operations in one instruction (Blackwell's packed FP32): a complex64
+// amplitude is the pair.  The same roundings as fmaf and a product on each half.
+using F2 = unsigned long long;
+__device__ __forceinline__ F2 f2_pack(float x, float y) {
+  F2 d;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(x), "f"(y));
+  return d;
+}
+__device__ __forceinline__ float2 f2_unpack(F2 a) {
+  float2 v;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(v.x), "=f"(v.y) : "l"(a));
+  return v;
+}
+__device__ __forceinline__ F2 f2_mul(F2 a, F2 b) {
+  F2 d;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ F2 f2_fma(F2 a, F2 b, F2 c) {
+  F2 d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+// u * v for complex u, v: fma(u.x, v, (-u.y, u.y) (v.y, v.x)) in both halves
+__device__ __forceinline__ F2 f2_cmul(float2 u, F2 v) {
+  const float2 w = f2_unpack(v);
+  return f2_fma(f2_pack(u.x, u.x), v, f2_mul(f2_pack(-u.y, u.y), f2_pack(w.y, w.x)));
+}
+
+// A table entry negated where `odd` is: sign terms make an entry's sign the parity of
+// j & S.  Callers take that parity once per group of amplitudes and skip the signs of
+// a tile without any (n = 26 brickwork of 16 layers 15.81 -> 15.34 ms).
+__device__ __forceinline__ float2 entry_sign(float2 e, uint32_t odd) {
+  const uint32_t m = odd << 31;
+  return make_float2(__uint_as_float(__float_as_uint(e.x) ^ m), __uint_as_float(__float_as_uint(e.y) ^ m));
+}
+
 // ---- FP32 engine (complex64 states) -------------------------------------------------
 // The op's matrix arrives rounded to float by the host (no conversion on the FP64 pipe).
 struct EngF32 {
@@ -201,14 +238,15 @@ struct EngF32 {
 };
 
 // All pairs (j, j | tb) of one op in the tile, the op class fixed at compile time;
-// unrolled so that a thread has several independent pairs in flight.
+// unrolled twice so that a thread has independent pairs in flight (four times: the
+// kernel outgrows the instruction cache, n = 26 random circuit 26.4 -> 26.7 ms).
 template <class E, int KIND, int THREADS>
 __device__ __forceinline__ void pair_loop(typename E::T* tile, uint32_t cnt, uint32_t fixed, uint32_t lcm, uint32_t tb,
                                           const TileOp& op) {
   using T = typename E::T;
   const uint32_t tbp = tsw(tb);
   const uint32_t csw = tsw_bits(lcm ? tile_expand(threadIdx.x, fixed, lcm) : threadIdx.x + (threadIdx.x & ~(tb - 1)));
-#pragma unroll 4
+#pragma unroll 2
   for (uint32_t i = threadIdx.x; i < cnt; i += THREADS) {
     // without in-tile controls the insertion of one zero bit is a mask and an add
     const uint32_t j0 = (lcm ? tile_expand(i, fixed, lcm) : i + (i & ~(tb - 1))) ^ csw, j1 = j0 ^ tbp;
@@ -260,7 +298,12 @@ __device__ __forceinline__ void quad_real(longlong2* tile, uint32_t TS, uint32_t
       v[c] = tile[pp[c]];
       if (tab) v[c] = table_mul(__ldg(tab + jj[c]), v[c], __popc(jj[c] & S) & 1);
     }
-    q60_pair_quad(v[0], v[1], v[2], v[3], m0, flags);
+    if (flags) {  // reflections: the sign flip of their bit-1 half first
+#pragma unroll
+      for (int c = 1; c < 4; ++c)
+        if (__popc(c & flags) & 1) v[c] = make_longlong2(-v[c].x, -v[c].y);
+    }
+    q60_pair_quad_t<0>(v[0], v[1], v[2], v[3], m0);
 #pragma unroll
     for (int c = 0; c < 4; ++c) tile[pp[c]] = v[c];
   }
@@ -371,27 +414,32 @@ __device__ __forceinline__ void quad_real_f32(float2* tile, uint32_t TS, uint32_
     const uint32_t jj[4] = {j, j | ta, j | tbb, j | ta | tbb};
     const uint32_t pj = j ^ csw;
     const uint32_t pp[4] = {pj, pj ^ pa, pj ^ pb, pj ^ pa ^ pb};
-    float2 v[4];
+    F2 v[4];
+    F2* t2 = reinterpret_cast<F2*>(tile);
 #pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      v[c] = tile[pp[c]];
-      if (tab) {
-        float2 u = __ldg(tab + jj[c]);
-        if (__popc(jj[c] & S) & 1) u = make_float2(-u.x, -u.y);
-        v[c] = make_float2(fmaf(u.x, v[c].x, -u.y * v[c].y), fmaf(u.x, v[c].y, u.y * v[c].x));
+    for (int c = 0; c < 4; ++c) v[c] = t2[pp[c]];
+    if (tab) {
+      float2 e[4];
+#pragma unroll
+      for (int c = 0; c < 4; ++c) e[c] = __ldg(tab + jj[c]);
+      if (S) {
+        const uint32_t odd = __popc(j & S), oa = (S & ta) != 0, ob = (S & tbb) != 0;
+#pragma unroll
+        for (int c = 0; c < 4; ++c) e[c] = entry_sign(e[c], odd ^ ((c & 1) ? oa : 0u) ^ ((c & 2) ? ob : 0u));
       }
+#pragma unroll
+      for (int c = 0; c < 4; ++c) v[c] = f2_cmul(e[c], v[c]);
     }
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-      float xr = 0.0f, xi = 0.0f;
+      F2 x = 0;
 #pragma unroll
       for (int c = 0; c < 4; ++c) {
         const int e = 4 * k + c;
         const float u = e < 8 ? m0[e] : m1[e - 8];
-        xr = fmaf(u, v[c].x, xr);
-        xi = fmaf(u, v[c].y, xi);
+        x = f2_fma(f2_pack(u, u), v[c], x);
       }
-      tile[pp[k]] = make_float2(xr, xi);
+      t2[pp[k]] = x;
     }
   }
 }
@@ -426,30 +474,42 @@ __device__ __forceinline__ void quad4_f32(float2* tile, uint32_t TS, uint32_t ta
     auto slot = [&](int k) {
       return pj ^ ((k & 1) ? pa : 0u) ^ ((k & 2) ? pb : 0u) ^ ((k & 4) ? pc : 0u) ^ ((k & 8) ? pd : 0u);
     };
-    float2 v[16];
+    F2 v[16];
+    F2* t2 = reinterpret_cast<F2*>(tile);
 #pragma unroll
-    for (int k = 0; k < 16; ++k) {
-      v[k] = tile[slot(k)];
-      if (tab) {
-        const uint32_t jk = j | ((k & 1) ? ta : 0u) | ((k & 2) ? tb : 0u) | ((k & 4) ? tc : 0u) | ((k & 8) ? td : 0u);
-        float2 u = __ldg(tab + jk);
-        if (__popc(jk & S) & 1) u = make_float2(-u.x, -u.y);
-        v[k] = make_float2(fmaf(u.x, v[k].x, -u.y * v[k].y), fmaf(u.x, v[k].y, u.y * v[k].x));
+    for (int k = 0; k < 16; ++k) v[k] = t2[slot(k)];
+    if (tab) {
+      const uint32_t odd = __popc(j & S), oa = (S & ta) != 0, ob = (S & tb) != 0, oc = (S & tc) != 0,
+                     od = (S & td) != 0;
+#pragma unroll
+      for (int h = 0; h < 16; h += 8) {  // eight entries in flight
+        float2 e[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+          e[k] = __ldg(tab + (j | ((k & 1) ? ta : 0u) | ((k & 2) ? tb : 0u) | ((k & 4) ? tc : 0u) | (h ? td : 0u)));
+        if (S) {
+#pragma unroll
+          for (int k = 0; k < 8; ++k)
+            e[k] = entry_sign(e[k], odd ^ ((k & 1) ? oa : 0u) ^ ((k & 2) ? ob : 0u) ^ ((k & 4) ? oc : 0u) ^ (h ? od : 0u));
+        }
+#pragma unroll
+        for (int k = 0; k < 8; ++k) v[h + k] = f2_cmul(e[k], v[h + k]);
       }
     }
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-      const float m00 = r[4 * q], m01 = r[4 * q + 1], m10 = r[4 * q + 2], m11 = r[4 * q + 3];
+      const F2 m00 = f2_pack(r[4 * q], r[4 * q]), m01 = f2_pack(r[4 * q + 1], r[4 * q + 1]),
+               m10 = f2_pack(r[4 * q + 2], r[4 * q + 2]), m11 = f2_pack(r[4 * q + 3], r[4 * q + 3]);
 #pragma unroll
       for (int k = 0; k < 16; ++k)
         if (!(k & (1 << q))) {
-          const float2 x0 = v[k], x1 = v[k | (1 << q)];
-          v[k] = make_float2(fmaf(m01, x1.x, m00 * x0.x), fmaf(m01, x1.y, m00 * x0.y));
-          v[k | (1 << q)] = make_float2(fmaf(m11, x1.x, m10 * x0.x), fmaf(m11, x1.y, m10 * x0.y));
+          const F2 x0 = v[k], x1 = v[k | (1 << q)];
+          v[k] = f2_fma(m01, x1, f2_mul(m00, x0));
+          v[k | (1 << q)] = f2_fma(m11, x1, f2_mul(m10, x0));
         }
     }
 #pragma unroll
-    for (int k = 0; k < 16; ++k) tile[slot(k)] = v[k];
+    for (int k = 0; k < 16; ++k) t2[slot(k)] = v[k];
   }
 }
 
@@ -596,12 +656,13 @@ __global__ void __launch_bounds__(THREADS, THREADS == 256 ? E::kMinBlocks : 1) k
         if (op.kind == TOP_DTABLE) {
           const float2* tf = reinterpret_cast<const float2*>(g.tables) + (size_t)lcm * TS;
           const uint32_t S = table_sign_mask(g, (int)lcm, base);
+          const uint32_t odd = __popc(threadIdx.x & S);
 #pragma unroll 8
           for (uint32_t j = threadIdx.x; j < TS; j += THREADS) {
             float2 u = __ldg(tf + j);
-            const float2 v = tile[j ^ tsq];
-            if (__popc(j & S) & 1) u = make_float2(-u.x, -u.y);
-            tile[j ^ tsq] = make_float2(fmaf(u.x, v.x, -u.y * v.y), fmaf(u.x, v.y, u.y * v.x));
+            if (S) u = entry_sign(u, odd ^ __popc((j - threadIdx.x) & S));
+            F2* t2 = reinterpret_cast<F2*>(tile);
+            t2[j ^ tsq] = f2_cmul(u, t2[j ^ tsq]);
           }
           __syncthreads();
           continue;
@@ -802,6 +863,14 @@ __global__ void k_q60_release(double2* __restrict__ a, size_t N) {
   }
 }
 
+// The other way, as a tile pass's load.
+__global__ void k_q60_hold(double2* __restrict__ a, size_t N) {
+  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < N; i += (size_t)gridDim.x * blockDim.x) {
+    const double2 v = a[i];
+    reinterpret_cast<longlong2*>(a)[i] = make_longlong2(q60_from_double_nb(v.x), q60_from_double_nb(v.y));
+  }
+}
+
 template <class E, int THREADS>
 static int launch_engine_t(qs_state* s, const TileArgs& g, size_t smem) {
   static bool attr_set = false;
@@ -836,6 +905,13 @@ int launch_q60_release(qs_state* s) {
   KTimer kt(s, QS_K_OTHER, 0, 0, 0, 0, (double)N, 0.0);
   k_q60_release<<<blocks, 256, 0, s->stream>>>(s->amps, N);
   return launch_check("q60 release");
+}
+
+int launch_q60_hold(qs_state* s) {
+  const size_t N = (size_t)1 << s->n;
+  KTimer kt(s, QS_K_OTHER, 0, 0, 0, 0, (double)N, 0.0);
+  k_q60_hold<<<(int)std::min<size_t>((N + 255) / 256, 152 * 16), 256, 0, s->stream>>>(s->amps, N);
+  return launch_check("q60 hold");
 }
 
 int launch_tile(qs_state* s, const TileArgs& g, double flops, double int_ops, int ngates, bool fixed) {

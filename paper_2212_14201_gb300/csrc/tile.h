@@ -98,8 +98,5 @@ static_assert(4 * TILE_MAX_M + 5 * TILE_MAX_OPS <= TABLE_ARGS_WORDS, "one table 
 int launch_tables(qs_state* s, const TableArgs& args, void* out);
 
 int launch_tile(qs_state* s, const TileArgs& args, double flops, double int_ops, int ngates, bool fixed);
-// Converts a buffer of Q60 integer pairs (left by a tile pass with io bit 1) back
-// to complex128 in place.
-int launch_q60_release(qs_state* s);
 
 }  // namespace qs
