@@ -12,6 +12,8 @@
 #include <math.h>
 
 #include <algorithm>
+#include <memory>
+#include <new>
 #include <vector>
 
 #include "fixed.h"
@@ -182,79 +184,72 @@ __global__ void __launch_bounds__(256) k_adj_step(double2* __restrict__ psi, dou
   }
 }
 
-// lambda = (H / S) psi, as a gather over groups of terms sharing an X mask:
-//   lambda[y] = sum_g D_g(y) psi[y ^ xm_g],
-//   D_g(y) = sum_{k in g} c_k i^{ny_k} (-1)^{popcount((y ^ xm_g) & zm_k)}.
+// lambda = (H / S) psi (h_row in q60tile.cuh) as a gather.  FX: psi and lambda hold
+// Q60 integers, else complex128.
 constexpr int HMAX = 48;
 struct HArgs {
   uint64_t N;
-  int nterms, ngroups, accumulate;
-  uint64_t gxm[HMAX];
-  int gstart[HMAX + 1];
-  uint64_t zm[HMAX];
-  double c[HMAX];   // coef / S times the real unit of i^ny (+-1) ...
-  int64_t cq[HMAX]; // (the same in Q60)
-  int imag[HMAX];   // ... placed in the imaginary part when ny is odd
+  int nruns, ngroups, accumulate;
+  HRun runs[HMAX];
+  uint64_t xms[HMAX];
+  HGroup groups[HMAX];
+  HTerm terms[HMAX];
 };
 
+template <bool FX>
 __global__ void __launch_bounds__(256) k_apply_h(const double2* __restrict__ psi, double2* __restrict__ lam,
                                                  const __grid_constant__ HArgs h) {
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-  // Q60 integers (the FP64 pipe would bound this loop on GB300): the signed
-  // coefficient sums of a group are exact in int64 (sum |c_k| <= 1), each group's
-  // product with psi is rounded once, and the launch's total (|.| <= |psi|_inf)
-  // is converted once.
+  auto load = [](const double2* a, uint64_t x) {
+    if (FX) return reinterpret_cast<const longlong2*>(a)[x];
+    const double2 p = a[x];
+    return make_longlong2(q60_from_double_nb(p.x), q60_from_double_nb(p.y));
+  };
   for (uint64_t y = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; y < h.N; y += stride) {
-    int64_t ore = 0, oim = 0;
-    for (int gi = 0; gi < h.ngroups; ++gi) {
-      const uint64_t x = y ^ h.gxm[gi];
-      int64_t dre = 0, dim = 0;
-      for (int k = h.gstart[gi]; k < h.gstart[gi + 1]; ++k) {
-        const int64_t v = (__popcll(x & h.zm[k]) & 1) ? -h.cq[k] : h.cq[k];
-        if (h.imag[k]) dim += v;
-        else dre += v;
-      }
-      const double2 p = psi[x];
-      const QL px = q60_split(q60_from_double(p.x)), py = q60_split(q60_from_double(p.y));
-      const QL qr = q60_split(dre), qi = q60_split(dim), nqi = q60_split(-dim);
-      QAcc r = qacc_new(), i = qacc_new();
-      qacc_add(r, qr, px);  // re: dre px - dim py
-      qacc_add(r, nqi, py);
-      qacc_add(i, qr, py);  // im: dre py + dim px
-      qacc_add(i, qi, px);
-      ore += qacc_round(r);
-      oim += qacc_round(i);
+    longlong2 out = h_row(h.runs, h.nruns, h.xms, h.groups, h.ngroups, h.terms, y,
+                          [&](uint64_t x) { return load(psi, x); });
+    if (FX) {
+      longlong2* l = reinterpret_cast<longlong2*>(lam) + y;
+      if (h.accumulate) out = make_longlong2(out.x + l->x, out.y + l->y);
+      *l = out;
+    } else {
+      double2 v = make_double2(q60_to_double_nb(out.x), q60_to_double_nb(out.y));
+      if (h.accumulate) v = make_double2(v.x + lam[y].x, v.y + lam[y].y);
+      lam[y] = v;
     }
-    double2 out = make_double2(q60_to_double(ore), q60_to_double(oim));
-    if (h.accumulate) {
-      const double2 prev = lam[y];
-      out.x += prev.x;
-      out.y += prev.y;
-    }
-    lam[y] = out;
   }
 }
 
 // per-CTA partials of Re <psi|lambda>
+template <bool FX>
 __global__ void __launch_bounds__(256) k_dot_re(const double2* __restrict__ a, const double2* __restrict__ b, uint64_t N,
                                                 double* __restrict__ part) {
   __shared__ double sh[8];
   double acc = 0.0;
+  __int128 eq = 0;  // FX: exact products (units 2^-120)
   for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < N; i += (uint64_t)gridDim.x * blockDim.x) {
-    const double2 u = a[i], v = b[i];
-    acc += fma(u.x, v.x, u.y * v.y);
+    if (FX) {
+      const longlong2 u = reinterpret_cast<const longlong2*>(a)[i], v = reinterpret_cast<const longlong2*>(b)[i];
+      eq += (__int128)dot2_exact(split31(u.x), split31(v.x), split31(u.y), split31(v.y));
+    } else {
+      const double2 u = a[i], v = b[i];
+      acc += fma(u.x, v.x, u.y * v.y);
+    }
   }
+  if (FX) acc = q120_to_double(eq);
   double s = adj_block_sum(acc, sh);
   if (threadIdx.x == 0) part[blockIdx.x] = s;
 }
 
-// out[j] = sum over the CTA partials of slot j, in CTA order.
-__global__ void k_slot_sums(const double* __restrict__ part, int nslots, int nblocks, double* __restrict__ out) {
-  for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < nslots; j += gridDim.x * blockDim.x) {
-    double s = 0.0;
-    for (int b = 0; b < nblocks; ++b) s += part[(size_t)j * nblocks + b];
-    out[j] = s;
-  }
+// out[j] = sum over the CTA partials of slot j: one CTA a slot, its threads' partials in
+// CTA order, then a fixed tree (one thread a slot waited for memory 608 times).
+__global__ void __launch_bounds__(256) k_slot_sums(const double* __restrict__ part, int nblocks,
+                                                   double* __restrict__ out) {
+  __shared__ double sh[8];
+  double s = 0.0;
+  for (int b = threadIdx.x; b < nblocks; b += 256) s += part[(size_t)blockIdx.x * nblocks + b];
+  s = adj_block_sum(s, sh);
+  if (threadIdx.x == 0) out[blockIdx.x] = s;
 }
 
 // ---- fused backward sweep (Q60): tile passes over psi and lambda at once --------------
@@ -270,13 +265,15 @@ struct AdjPassArgs {
   const BOp* ops;   // ops of this pass (device), in execution order
   const QC* mats;   // 4 entries per op (device)
   const QC* dgm;    // 16 entries per diagonal group (device)
-  const QL* rpm;    // 16 entries per real pair (device)
+  const QL* rpm;    // 6 entries per real pair (device)
   double* part;     // [slot][ADJ_GRID_STRIDE]
   int slot_base;
 };
 
-__global__ void __launch_bounds__(BT_THREADS, 3) k_adj_pass(double2* __restrict__ psi, double2* __restrict__ lam,
-                                                         const AdjPassArgs a) {
+// psi and lambda hold Q60 integers from the last forward pass on: no conversion and no
+// rounding to double between passes.
+__global__ void __launch_bounds__(BT_THREADS, 3) k_adj_pass(longlong2* __restrict__ psi, longlong2* __restrict__ lam,
+                                                         const __grid_constant__ AdjPassArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
   const BPass& ps = a.ps;
   const int m = ps.m;
@@ -286,28 +283,23 @@ __global__ void __launch_bounds__(BT_THREADS, 3) k_adj_pass(double2* __restrict_
   longlong2* tP = reinterpret_cast<longlong2*>(smem);
   longlong2* tL = tP + TS;
   uint64_t* offs = reinterpret_cast<uint64_t*>(tL + TS);
-  double* wacc = reinterpret_cast<double*>(offs + H);  // [warps][nslots]
+  int64_t* wacc = reinterpret_cast<int64_t*>(offs + H);  // [warps][nslots]
   for (uint32_t h = threadIdx.x; h < H; h += BT_THREADS) {
     uint64_t o = 0;
     for (int b = 0; b < ps.nhigh; ++b) o |= (uint64_t)((h >> b) & 1u) << ps.qhigh[b];
     offs[h] = o;
   }
-  for (int s = threadIdx.x; s < ps.nslots * (BT_THREADS / 32); s += BT_THREADS) wacc[s] = 0.0;
-  const uint32_t lowmask = (1u << L) - 1;
+  for (int s = threadIdx.x; s < ps.nslots * (BT_THREADS / 32); s += BT_THREADS) wacc[s] = 0;
   const uint64_t ntiles = 1ull << ps.nout;
   for (uint64_t r = blockIdx.x; r < ntiles; r += gridDim.x) {
     uint64_t base = 0;
     for (int b = 0; b < ps.nout; ++b) base |= ((r >> b) & 1ull) << ps.outpos[b];
     __syncthreads();
-    for (uint32_t j = threadIdx.x; j < TS; j += BT_THREADS) {
-      const uint64_t x = base + offs[j >> L] + (j & lowmask);
-      const double2 u = psi[x], v = lam[x];
-      tP[j] = make_longlong2(q60_from_double(u.x), q60_from_double(u.y));
-      tL[j] = make_longlong2(q60_from_double(v.x), q60_from_double(v.y));
-    }
+    bt_load(tP, psi, base, offs, L, TS);
+    bt_load(tL, lam, base, offs, L, TS);
     __syncthreads();
     for (int k = ps.op_begin; k < ps.op_end; ++k) {
-      const BOp op = a.ops[k];
+      const BOp& op = a.ops[k];
       if (op.kb == BK_MEMBER || (base & op.ext) != op.ext) continue;
       // each thread reads and then rewrites only its own pairs (amplitudes) of this
       // op, so the generator partial and the update need no barrier between them
@@ -316,17 +308,22 @@ __global__ void __launch_bounds__(BT_THREADS, 3) k_adj_pass(double2* __restrict_
         const BOp* mem = a.ops + k + 1;
         bt_back_dgroup(tP, tL, TS, mem, op.nmem, a.dgm + 16 * op.gate, gp);
         for (int mm = 0; mm < op.nmem; ++mm)
-          if (mem[mm].slot >= 0) bt_warp_accumulate(gp[mm], wacc, ps.nslots, mem[mm].slot);
+          if (mem[mm].slot >= 0) bt_warp_accumulate(2 * gp[mm], wacc, ps.nslots, mem[mm].slot);
         __syncthreads();
         continue;
       }
       if (op.kb == BK_RPAIR) {
         const BOp* mem = a.ops + k + 1;
-        int64_t ga, gb;
-        bt_rpair_back(tP, tL, TS, 1u << mem[0].tb, 1u << mem[1].tb, mem[0].gen, mem[1].gen, a.rpm + 16 * op.gate,
-                      &ga, &gb);
-        if (mem[0].slot >= 0) bt_warp_accumulate(ga, wacc, ps.nslots, mem[0].slot);
-        if (mem[1].slot >= 0) bt_warp_accumulate(gb, wacc, ps.nslots, mem[1].slot);
+        int64_t gu, gv;
+        bt_rpair_back(tP, tL, TS, 1u << mem[0].tb, 1u << mem[1].tb, mem[0].slot >= 0 || mem[1].slot >= 0,
+                      a.rpm + 6 * op.gate, &gu, &gv);
+        if (mem[0].slot >= 0) bt_warp_accumulate(gu + gv, wacc, ps.nslots, mem[0].slot);
+        if (mem[1].slot >= 0) bt_warp_accumulate(gu - gv, wacc, ps.nslots, mem[1].slot);
+        __syncthreads();
+        continue;
+      }
+      if (op.kb == BK_PERM) {
+        bt_perm(tP, tL, TS, a.ops + k + 1, op.nmem, false, base);
         __syncthreads();
         continue;
       }
@@ -336,20 +333,17 @@ __global__ void __launch_bounds__(BT_THREADS, 3) k_adj_pass(double2* __restrict_
         continue;
       }
       if (op.slot >= 0 && op.kb == OP_REAL) {  // one pass over the pairs
-        bt_warp_accumulate(bt_back_real(tP, tL, TS, op, a.mats + 4 * k), wacc, ps.nslots, op.slot);
+        bt_warp_accumulate(2 * bt_back_real(tP, tL, TS, op, a.mats + 4 * k), wacc, ps.nslots, op.slot);
         __syncthreads();
         continue;
       }
-      if (op.slot >= 0) bt_warp_accumulate(bt_gen_partial(tP, tL, TS, op, base), wacc, ps.nslots, op.slot);
+      if (op.slot >= 0) bt_warp_accumulate(2 * bt_gen_partial(tP, tL, TS, op, base), wacc, ps.nslots, op.slot);
       bt_apply(tP, TS, op, op.kb, op.c0b, op.c1b, a.mats + 4 * k, base);
       bt_apply(tL, TS, op, op.kb, op.c0b, op.c1b, a.mats + 4 * k, base);
       __syncthreads();
     }
-    for (uint32_t j = threadIdx.x; j < TS; j += BT_THREADS) {
-      const uint64_t x = base + offs[j >> L] + (j & lowmask);
-      psi[x] = make_double2(q60_to_double(tP[j].x), q60_to_double(tP[j].y));
-      lam[x] = make_double2(q60_to_double(tL[j].x), q60_to_double(tL[j].y));
-    }
+    bt_store(tP, psi, base, offs, L, TS);
+    bt_store(tL, lam, base, offs, L, TS);
   }
   __syncthreads();
   for (int k = ps.op_begin + threadIdx.x; k < ps.op_end; k += BT_THREADS) {
@@ -384,7 +378,7 @@ static int backward_fused(qs_state* s, double2* lam, const qs_gate* gates, size_
   std::vector<QC> mats;
   std::vector<QC> dgm;    // 16 Gauss-form entries per diagonal group
   std::vector<int> dgheads, dgsrc, rpheads;
-  std::vector<QL> rpm;    // 16 limb pairs per real pair
+  std::vector<QL> rpm;    // 6 limb pairs per real pair
   std::vector<BPass> passes;
   int slot_base = 0;
   std::vector<int> slot_bases;
@@ -416,6 +410,9 @@ static int backward_fused(qs_state* s, double2* lam, const qs_gate* gates, size_
       op.kb = op.kf = (int8_t)o1.cls;
       op.c0b = (int8_t)o1.code0;
       op.c1b = (int8_t)o1.code1;
+      op.c0f = op.c0b;
+      op.c1f = op.c1b;
+      op.rot = o1.cls == OP_REAL && mt.m[0].re * mt.m[3].re - mt.m[1].re * mt.m[2].re > 0.0;
       uint32_t lcm = 0;
       uint64_t ext = 0;
       for (int b = 0; b < n; ++b)
@@ -468,12 +465,16 @@ static int backward_fused(qs_state* s, double2* lam, const qs_gate* gates, size_
         dgm.push_back(qc_make_gauss(re, im));
       }
     }
-    for (size_t pi = np0; pi < rpheads.size(); ++pi) {  // M = R_b (x) R_a, a = first member
-      const Mat2& ra = opm[rpheads[pi] + 1];
-      const Mat2& rb = opm[rpheads[pi] + 2];
-      for (int k = 0; k < 4; ++k)
-        for (int c = 0; c < 4; ++c)
-          rpm.push_back(q60_split_coef(q60_from_double(rb.m[2 * (k >> 1) + (c >> 1)].re * ra.m[2 * (k & 1) + (c & 1)].re)));
+    for (size_t pi = np0; pi < rpheads.size(); ++pi) {
+      double ra[4], rb[4];
+      for (int e = 0; e < 4; ++e) {
+        ra[e] = opm[rpheads[pi] + 1].m[e].re;
+        rb[e] = opm[rpheads[pi] + 2].m[e].re;
+      }
+      QL c[6];
+      int flags;  // rotations: 0
+      q60_pair_coef(ra, rb, c, &flags);
+      rpm.insert(rpm.end(), c, c + 6);
     }
     bp.op_end = (int)ops.size();
     bp.nslots = slot;
@@ -482,22 +483,28 @@ static int backward_fused(qs_state* s, double2* lam, const qs_gate* gates, size_
     slot_base += slot;
     remaining.swap(rest);
   }
-  BOp* d_ops = nullptr;
-  QC* d_mats = nullptr;
-  QC* d_dgm = nullptr;
-  QL* d_rpm = nullptr;
-  QS_CUDA(dmalloc_async((void**)&d_ops, sizeof(BOp) * std::max<size_t>(1, ops.size()), s->stream));
-  cudaError_t e = dmalloc_async((void**)&d_mats, sizeof(QC) * std::max<size_t>(4, mats.size()), s->stream);
-  if (e == cudaSuccess) e = dmalloc_async((void**)&d_dgm, sizeof(QC) * std::max<size_t>(16, dgm.size()), s->stream);
-  if (e == cudaSuccess) e = dmalloc_async((void**)&d_rpm, sizeof(QL) * std::max<size_t>(16, rpm.size()), s->stream);
-  if (e == cudaSuccess && !rpm.empty())
-    e = cudaMemcpyAsync(d_rpm, rpm.data(), sizeof(QL) * rpm.size(), cudaMemcpyHostToDevice, s->stream);
-  if (e == cudaSuccess && !ops.empty())
-    e = cudaMemcpyAsync(d_ops, ops.data(), sizeof(BOp) * ops.size(), cudaMemcpyHostToDevice, s->stream);
-  if (e == cudaSuccess && !mats.empty())
-    e = cudaMemcpyAsync(d_mats, mats.data(), sizeof(QC) * mats.size(), cudaMemcpyHostToDevice, s->stream);
-  if (e == cudaSuccess && !dgm.empty())
-    e = cudaMemcpyAsync(d_dgm, dgm.data(), sizeof(QC) * dgm.size(), cudaMemcpyHostToDevice, s->stream);
+  // one upload from pinned memory into the workspace (or, if that is too small, into
+  // memory of this call)
+  auto up16 = [](size_t b) { return (b + 15) & ~(size_t)15; };
+  const size_t ob = up16(sizeof(BOp) * ops.size()), mb = up16(sizeof(QC) * mats.size()),
+               db = up16(sizeof(QC) * dgm.size()), rb = up16(sizeof(QL) * rpm.size()), total = ob + mb + db + rb;
+  ScratchBuf big;
+  char* dev = (char*)s->ws;
+  if (total > s->ws_bytes) {
+    QS_TRY(take_scratch(s, total, &big));
+    dev = (char*)big.p;
+  }
+  QS_TRY(ensure_pinned(s, total + 16));
+  char* host = (char*)s->pinned;
+  if (!ops.empty()) memcpy(host, ops.data(), sizeof(BOp) * ops.size());
+  if (!mats.empty()) memcpy(host + ob, mats.data(), sizeof(QC) * mats.size());
+  if (!dgm.empty()) memcpy(host + ob + mb, dgm.data(), sizeof(QC) * dgm.size());
+  if (!rpm.empty()) memcpy(host + ob + mb + db, rpm.data(), sizeof(QL) * rpm.size());
+  cudaError_t e = total ? cudaMemcpyAsync(dev, host, total, cudaMemcpyHostToDevice, s->stream) : cudaSuccess;
+  const BOp* d_ops = (const BOp*)dev;
+  const QC* d_mats = (const QC*)(dev + ob);
+  const QC* d_dgm = (const QC*)(dev + ob + mb);
+  const QL* d_rpm = (const QL*)(dev + ob + mb + db);
   int rc = e == cudaSuccess ? QS_OK : cuda_fail(e, "adjoint op tables");
   static bool attr = false;
   if (rc == QS_OK && !attr) {
@@ -521,14 +528,11 @@ static int backward_fused(qs_state* s, double2* lam, const qs_gate* gates, size_
     const uint64_t grid = std::min<uint64_t>(1ull << a.ps.nout, (uint64_t)std::min(ADJ_GRID_STRIDE, 152 * per_sm));
     {
       KTimer kt(s, QS_K_ADJOINT, a.ps.m, a.ps.op_end - a.ps.op_begin, 0, 0, 2.0 * (double)(1ull << n), 0.0);
-      k_adj_pass<<<(unsigned)grid, BT_THREADS, smem, s->stream>>>(s->amps, lam, a);
+      k_adj_pass<<<(unsigned)grid, BT_THREADS, smem, s->stream>>>(reinterpret_cast<longlong2*>(s->amps),
+                                                                  reinterpret_cast<longlong2*>(lam), a);
     }
     rc = launch_check("adjoint pass");
   }
-  cudaFreeAsync(d_ops, s->stream);
-  cudaFreeAsync(d_mats, s->stream);
-  cudaFreeAsync(d_dgm, s->stream);
-  cudaFreeAsync(d_rpm, s->stream);
   return rc;
 }
 
@@ -551,60 +555,45 @@ static int gen_of(const qs_gate& g) {
 
 // Launch lambda = (H/S) psi for the whole Pauli sum (several launches if it is long).
 static int apply_hamiltonian(qs_state* s, const double2* psi, double2* lam, const qs_pauli* terms, size_t nterms,
-                             double S) {
-  // group by X mask, preserving first-appearance order
+                             double S, bool fx) {
+  std::vector<HRun> runs;
   std::vector<uint64_t> xms;
-  std::vector<std::vector<size_t>> members;
-  for (size_t k = 0; k < nterms; ++k) {
-    size_t gidx = 0;
-    while (gidx < xms.size() && xms[gidx] != terms[k].xmask) ++gidx;
-    if (gidx == xms.size()) {
-      xms.push_back(terms[k].xmask);
-      members.emplace_back();
-    }
-    members[gidx].push_back(k);
-  }
-  HArgs* h = new (std::nothrow) HArgs;
+  std::vector<HGroup> groups;
+  std::vector<HTerm> hterms;
+  h_plan(terms, nterms, S, &runs, &xms, &groups, &hterms);
+  std::unique_ptr<HArgs> h(new (std::nothrow) HArgs);
   if (!h) return fail(QS_ERR_OOM, "host allocation failed");
   h->N = 1ull << s->n;
-  h->accumulate = 0;
-  int rc = QS_OK;
-  size_t gi = 0;
   const int grid = (int)std::min<uint64_t>((h->N + 255) / 256, 152 * 16);
-  while (gi < xms.size() || (xms.empty() && !h->accumulate)) {
-    h->nterms = 0;
-    h->ngroups = 0;
-    while (gi < xms.size() && h->ngroups < HMAX && h->nterms + (int)members[gi].size() <= HMAX) {
-      h->gxm[h->ngroups] = xms[gi];
-      h->gstart[h->ngroups] = h->nterms;
-      for (size_t k : members[gi]) {
-        const qs_pauli& t = terms[k];
-        int ny = __builtin_popcountll(t.xmask & t.zmask) & 3;
-        double c = t.coef / S;
-        h->zm[h->nterms] = t.zmask;
-        h->c[h->nterms] = (ny >= 2) ? -c : c;
-        h->cq[h->nterms] = q60_from_double(h->c[h->nterms]);
-        h->imag[h->nterms] = ny & 1;
-        ++h->nterms;
-      }
-      ++h->ngroups;
+  size_t ri = 0, gi = 0;
+  h->accumulate = 0;
+  do {
+    h->nruns = h->ngroups = 0;
+    int nx = 0, nt = 0;
+    while (ri < runs.size() && nx + runs[ri].end - runs[ri].begin <= HMAX) {
+      HRun& r = h->runs[h->nruns++] = runs[ri];
+      r.begin = nx;
+      for (int k = runs[ri].begin; k < runs[ri].end; ++k) h->xms[nx++] = xms[k];
+      r.end = nx;
+      ++ri;
+    }
+    while (gi < groups.size() && nt + groups[gi].end - groups[gi].begin <= HMAX && h->ngroups < HMAX) {
+      HGroup& g = h->groups[h->ngroups++] = groups[gi];
+      g.begin = nt;
+      for (int k = groups[gi].begin; k < groups[gi].end; ++k) h->terms[nt++] = hterms[k];
+      g.end = nt;
       ++gi;
     }
-    if (h->ngroups == 0 && gi < xms.size()) {
-      rc = fail(QS_ERR_UNSUPPORTED, "more than %d terms share one X mask", HMAX);
-      break;
-    }
-    h->gstart[h->ngroups] = h->nterms;
+    if (gi < groups.size() && nt == 0) return fail(QS_ERR_UNSUPPORTED, "more than %d terms share one X mask", HMAX);
     {
-      KTimer kt(s, QS_K_ADJOINT, 0, h->nterms, 0, 0, (double)h->N * (1 + h->ngroups), 0.0);
-      k_apply_h<<<grid, 256, 0, s->stream>>>(psi, lam, *h);
+      KTimer kt(s, QS_K_ADJOINT, 0, nx + nt, 0, 0, (double)h->N * (1 + nx + h->ngroups), 0.0);
+      if (fx) k_apply_h<true><<<grid, 256, 0, s->stream>>>(psi, lam, *h);
+      else k_apply_h<false><<<grid, 256, 0, s->stream>>>(psi, lam, *h);
     }
-    if ((rc = launch_check("apply_h")) != QS_OK) break;
+    QS_TRY(launch_check("apply_h"));
     h->accumulate = 1;
-    if (xms.empty()) break;
-  }
-  delete h;
-  return rc;
+  } while (ri < runs.size() || gi < groups.size());
+  return QS_OK;
 }
 
 }  // namespace qs
@@ -637,41 +626,40 @@ extern "C" int qs_adjoint_grad(qs_state* s, const qs_gate* gates, size_t ng, con
   const uint64_t N = 1ull << n;
   const size_t bytes = N * sizeof(double2);
   // lambda lives next to the state for the duration of the call
-  double2* lam = nullptr;
-  QS_CUDA(dmalloc_async((void**)&lam, bytes, s->stream));
   const int nblocks = 608;
-  double* part = nullptr;
-  double* sums = nullptr;
+  ScratchBuf buf;
+  QS_TRY(take_scratch(s, bytes + sizeof(double) * (nslots + 1) * (nblocks + 1), &buf));
+  double2* lam = (double2*)buf.p;
+  double* part = (double*)(lam + N);
+  double* sums = part + (size_t)nblocks * (nslots + 1);
   int rc = QS_OK;
-  auto cleanup = [&]() {
-    if (lam) cudaFreeAsync(lam, s->stream);
-    if (part) cudaFreeAsync(part, s->stream);
-    if (sums) cudaFreeAsync(sums, s->stream);
-  };
-  cudaError_t e = dmalloc_async((void**)&part, sizeof(double) * nblocks * (nslots + 1), s->stream);
-  if (e == cudaSuccess) e = dmalloc_async((void**)&sums, sizeof(double) * (nslots + 1), s->stream);
-  if (e != cudaSuccess) {
-    cleanup();
-    return cuda_fail(e, "adjoint workspace");
-  }
+  cudaError_t e = cudaSuccess;
   // forward: psi = U_G ... U_1 |0>, fused
   const double S = csum > 0 ? exp2(ceil(log2(csum))) : 1.0;
   qs_plan* plan = nullptr;
-  if ((rc = qs_set_zero(s)) == QS_OK && (rc = qs_plan_create(n, gates, ng, QS_PLAN_GREEDY, 5, &plan)) == QS_OK)
-    rc = qs_apply(s, gates, ng, params, plan);
+  bool fixed = false, held = false;  // held: the amplitudes are Q60 integers
+  if ((rc = qs_set_zero(s)) == QS_OK && (rc = qs_plan_create(n, gates, ng, QS_PLAN_GREEDY, 5, &plan)) == QS_OK &&
+      (rc = choose_fixed(s, &fixed)) == QS_OK) {
+    const bool keep = fixed && g_adj_fused;
+    rc = qs_apply_plan(s, gates, ng, params, plan, fixed, keep ? &held : nullptr);
+    if (rc == QS_OK && keep && !held) {
+      rc = launch_q60_hold(s);
+      held = rc == QS_OK;
+    }
+  }
   if (plan) qs_plan_free(plan);
-  bool fixed = false;
-  if (rc == QS_OK) rc = choose_fixed(s, &fixed);
-  if (rc == QS_OK) rc = apply_hamiltonian(s, s->amps, lam, terms, nterms, S);
+  if (rc == QS_OK) rc = apply_hamiltonian(s, s->amps, lam, terms, nterms, S, held);
   if (rc == QS_OK) {
     KTimer kt(s, QS_K_ADJOINT, 0, 0, 0, 0, 2.0 * N, 2.0 * N);
-    k_dot_re<<<nblocks, 256, 0, s->stream>>>(s->amps, lam, N, part + (size_t)nslots * nblocks);
+    double* dot = part + (size_t)nslots * nblocks;
+    if (held) k_dot_re<true><<<nblocks, 256, 0, s->stream>>>(s->amps, lam, N, dot);
+    else k_dot_re<false><<<nblocks, 256, 0, s->stream>>>(s->amps, lam, N, dot);
     rc = launch_check("dot");
   }
   // backward
   std::vector<int> slot_param;
   size_t slot = 0;
-  const bool fused = fixed && g_adj_fused;
+  const bool fused = held;
   if (rc == QS_OK && fused) {
     e = cudaMemsetAsync(part, 0, sizeof(double) * nblocks * nslots, s->stream);
     rc = e == cudaSuccess ? backward_fused(s, lam, gates, ng, params, part, slot_param) : cuda_fail(e, "memset");
@@ -718,7 +706,7 @@ extern "C" int qs_adjoint_grad(qs_state* s, const qs_gate* gates, size_t ng, con
   }
   std::vector<double> host(nslots + 1);
   if (rc == QS_OK) {
-    k_slot_sums<<<(int)((nslots + 1 + 127) / 128), 128, 0, s->stream>>>(part, (int)nslots + 1, nblocks, sums);
+    k_slot_sums<<<(unsigned)(nslots + 1), 256, 0, s->stream>>>(part, nblocks, sums);
     rc = launch_check("slot sums");
   }
   if (rc == QS_OK) {
@@ -726,7 +714,10 @@ extern "C" int qs_adjoint_grad(qs_state* s, const qs_gate* gates, size_t ng, con
     if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
     if (e != cudaSuccess) rc = cuda_fail(e, "adjoint readback");
   }
-  cleanup();
+  if (held) {  // the state is complex128 again, also after an error
+    const int rc2 = launch_q60_release(s);
+    if (rc == QS_OK) rc = rc2;
+  }
   if (rc != QS_OK) return rc;
   *energy = host[nslots] * S;
   for (size_t j = 0; j < np; ++j) grad[j] = 0.0;

@@ -33,8 +33,9 @@ namespace cg = cooperative_groups;
 
 namespace qs {
 
-constexpr int BT_CLUSTER = 8;  // largest cluster (portable size); the launch uses 1, 2, 4 or 8
-static_assert(BT_CLUSTER <= BT_THREADS / 32, "cluster rows must fit the warp-row accumulator");
+constexpr int BT_CLUSTER = 16;  // largest cluster (above the portable size of 8); the launch uses 1, 2, 4, 8 or 16
+constexpr int BT_ACC_ROWS = BT_CLUSTER;  // accumulator rows: one per warp, then one per CTA of the cluster
+static_assert(BT_ACC_ROWS >= BT_THREADS / 32, "a row per warp");
 static_assert(BT_MAX_OPS <= BT_THREADS, "one thread per gradient slot");
 
 struct BItem {
@@ -45,8 +46,10 @@ struct BItem {
 
 
 struct BSet {
-  int n, pass_begin, npasses, gate_begin, ngates, group_begin, ngroups, param_begin, nparams;
+  int n, pass_begin, npasses, gate_begin, ngates, param_begin, nparams;
+  int run_begin, nruns, group_begin, ngroups;  // H / S (run, group and term indices are the batch's)
   int dg_begin, ndg;  // diagonal groups (BK_DGROUP heads) of the set's passes
+  int rp_begin, nrp;  // real pairs (BK_RPAIR heads)
   long long amp_off;
   double S;
 };
@@ -54,18 +57,6 @@ struct BSet {
 struct BGate {
   int type, param, dagger;
   double p[3];
-};
-
-struct BGroup {
-  uint64_t xm;
-  int tbegin, tend;
-};
-
-struct BTerm {
-  double c;       // coef / S, with the real sign of i^ny
-  int64_t cq;     // the same in Q60 (|c| <= 1)
-  uint64_t zm;
-  int imag;       // i^ny is imaginary
 };
 
 struct BatchArgs {
@@ -76,18 +67,23 @@ struct BatchArgs {
   const BPass* passes;
   const BOp* ops;
   const BGate* gates;
-  const BGroup* groups;
-  const BTerm* terms;
+  const HRun* runs;
+  const uint64_t* xms;
+  const HGroup* groups;
+  const HTerm* terms;
   const double* params;
   double* grads;
   double* energies;
-  double2* psi;
-  double2* lam;
+  longlong2* psi;  // Q60 integers for the whole run: no conversion between passes
+  longlong2* lam;
   QC* matf;   // 4 per gate (Gauss form)
   QC* matb;   // 4 per gate (Gauss form)
   const int* dghead;  // per diagonal group: global index of its head op
   QC* dgf;    // 16 per diagonal group (Gauss form), forward
   QC* dgb;    // 16 per diagonal group, adjoint
+  const int* rphead;  // per real pair: global index of its head op
+  QL* rpf;    // 6 limb pairs per real pair, forward
+  QL* rpb;    // 6 limb pairs per real pair, adjoint
   int* counter;
 };
 
@@ -152,54 +148,65 @@ __device__ __forceinline__ void bt_cluster_sync() {
 // Backward: for every op in reverse, the generator term then U^dag on psi and
 // lambda; gradient contributions are added in backward op order, per slot the
 // warps of a CTA in warp order, then the CTAs in rank order.
-__device__ void bt_run_pass(const BatchArgs& d, const BPass& ps, double2* psi, double2* lam, const QC* matf,
-                            const QC* matb, bool backward, longlong2* tP, longlong2* tL, uint64_t* offs, double* acc,
-                            int rank, int nr) {
+__device__ void bt_run_pass(const BatchArgs& d, const BPass& ps, longlong2* psi, longlong2* lam, const QC* matf,
+                            const QC* matb, bool backward, longlong2* tP, longlong2* tL, uint64_t* offs, int64_t* acc,
+                            BStage* stage, int rank, int nr) {
   const int m = ps.m;
   const int L = m - ps.nhigh;
   const uint32_t TS = 1u << m;
   const uint32_t H = 1u << ps.nhigh;
-  const uint32_t lowmask = (1u << L) - 1;
   const uint64_t ntiles = 1ull << ps.nout;
   for (uint32_t h = threadIdx.x; h < H; h += BT_THREADS) {
     uint64_t o = 0;
     for (int b = 0; b < ps.nhigh; ++b) o |= (uint64_t)((h >> b) & 1u) << ps.qhigh[b];
     offs[h] = o;
   }
-  for (int s = threadIdx.x; s < ps.nslots * (BT_THREADS / 32); s += BT_THREADS) acc[s] = 0.0;
+  for (int s = threadIdx.x; s < ps.nslots * (BT_THREADS / 32); s += BT_THREADS) acc[s] = 0;
+  // (the stage's last readers are past the barrier that ends every pass)
+  const BRecords rec = bt_records(stage, ps, d.ops, backward ? d.dgb : d.dgf, backward ? d.rpb : d.rpf);
   for (uint64_t r = rank; r < ntiles; r += nr) {
     uint64_t base = 0;
     for (int b = 0; b < ps.nout; ++b) base |= ((r >> b) & 1ull) << ps.outpos[b];
     __syncthreads();
-    for (uint32_t j = threadIdx.x; j < TS; j += BT_THREADS) {
-      const uint64_t x = base + offs[j >> L] + (j & lowmask);
-      const double2 a = psi[x];
-      tP[j] = make_longlong2(q60_from_double(a.x), q60_from_double(a.y));
-      if (backward) {
-        const double2 b = lam[x];
-        tL[j] = make_longlong2(q60_from_double(b.x), q60_from_double(b.y));
-      }
-    }
+    bt_load(tP, psi, base, offs, L, TS);
+    if (backward) bt_load(tL, lam, base, offs, L, TS);
     __syncthreads();
     if (!backward) {
       for (int k = ps.op_begin; k < ps.op_end; ++k) {
-        const BOp op = d.ops[k];
+        const BOp& op = rec.ops[k];
         if (op.kf == BK_MEMBER || (base & op.ext) != op.ext) continue;
-        if (op.kf == BK_DGROUP) bt_apply_dgroup(tP, TS, d.ops + k + 1, op.nmem, d.dgf + 16 * op.gate);
+        if (op.kf == BK_DGROUP) bt_apply_dgroup(tP, TS, rec.ops + k + 1, op.nmem, rec.dg + 16 * op.gate);
+        else if (op.kf == BK_RPAIR) bt_rpair(tP, TS, 1u << rec.ops[k + 1].tb, 1u << rec.ops[k + 2].tb, rec.rp + 6 * op.gate);
+        else if (op.kf == BK_PERM) bt_perm(tP, nullptr, TS, rec.ops + k + 1, op.nmem, false, base);
         else bt_apply(tP, TS, op, op.kf, op.c0f, op.c1f, matf + 4 * op.gate, base);
         __syncthreads();
       }
     } else {
       for (int k = ps.op_end - 1; k >= ps.op_begin; --k) {
-        const BOp op = d.ops[k];
+        const BOp& op = rec.ops[k];
         if (op.kb == BK_MEMBER || (base & op.ext) != op.ext) continue;
         // each thread reads and then rewrites only its own pairs (amplitudes) of this op
         if (op.kb == BK_DGROUP) {
           int64_t part[BT_DG_MAX];
-          const BOp* mem = d.ops + k + 1;
-          bt_back_dgroup(tP, tL, TS, mem, op.nmem, d.dgb + 16 * op.gate, part);
+          const BOp* mem = rec.ops + k + 1;
+          bt_back_dgroup(tP, tL, TS, mem, op.nmem, rec.dg + 16 * op.gate, part);
           for (int mm = 0; mm < op.nmem; ++mm)
-            if (mem[mm].slot >= 0) bt_warp_accumulate(part[mm], acc, ps.nslots, mem[mm].slot);
+            if (mem[mm].slot >= 0) bt_warp_accumulate(2 * part[mm], acc, ps.nslots, mem[mm].slot);
+          __syncthreads();
+          continue;
+        }
+        if (op.kb == BK_RPAIR) {
+          const BOp* mem = rec.ops + k + 1;
+          int64_t gu, gv;
+          bt_rpair_back(tP, tL, TS, 1u << mem[0].tb, 1u << mem[1].tb, mem[0].slot >= 0 || mem[1].slot >= 0,
+                        rec.rp + 6 * op.gate, &gu, &gv);
+          if (mem[0].slot >= 0) bt_warp_accumulate(gu + gv, acc, ps.nslots, mem[0].slot);
+          if (mem[1].slot >= 0) bt_warp_accumulate(gu - gv, acc, ps.nslots, mem[1].slot);
+          __syncthreads();
+          continue;
+        }
+        if (op.kb == BK_PERM) {
+          bt_perm(tP, tL, TS, rec.ops + k + 1, op.nmem, true, base);
           __syncthreads();
           continue;
         }
@@ -209,21 +216,18 @@ __device__ void bt_run_pass(const BatchArgs& d, const BPass& ps, double2* psi, d
           continue;
         }
         if (op.slot >= 0 && op.kb == OP_REAL) {  // one pass over the pairs
-          bt_warp_accumulate(bt_back_real(tP, tL, TS, op, matb + 4 * op.gate), acc, ps.nslots, op.slot);
+          bt_warp_accumulate(2 * bt_back_real(tP, tL, TS, op, matb + 4 * op.gate), acc, ps.nslots, op.slot);
           __syncthreads();
           continue;
         }
-        if (op.slot >= 0) bt_warp_accumulate(bt_gen_partial(tP, tL, TS, op, base), acc, ps.nslots, op.slot);
+        if (op.slot >= 0) bt_warp_accumulate(2 * bt_gen_partial(tP, tL, TS, op, base), acc, ps.nslots, op.slot);
         bt_apply(tP, TS, op, op.kb, op.c0b, op.c1b, matb + 4 * op.gate, base);
         bt_apply(tL, TS, op, op.kb, op.c0b, op.c1b, matb + 4 * op.gate, base);
         __syncthreads();
       }
     }
-    for (uint32_t j = threadIdx.x; j < TS; j += BT_THREADS) {
-      const uint64_t x = base + offs[j >> L] + (j & lowmask);
-      psi[x] = make_double2(q60_to_double(tP[j].x), q60_to_double(tP[j].y));
-      if (backward) lam[x] = make_double2(q60_to_double(tL[j].x), q60_to_double(tL[j].y));
-    }
+    bt_store(tP, psi, base, offs, L, TS);
+    if (backward) bt_store(tL, lam, base, offs, L, TS);
   }
   __syncthreads();
   if (nr == 1) {
@@ -244,14 +248,15 @@ __device__ void bt_run_pass(const BatchArgs& d, const BPass& ps, double2* psi, d
   // shared memory), then rank 0 adds them in rank order
   const double v = threadIdx.x < ps.nslots ? bt_warp_total(acc, ps.nslots, threadIdx.x) : 0.0;
   bt_cluster_sync();
-  if (threadIdx.x < ps.nslots) cg::this_cluster().map_shared_rank(acc, 0)[rank * ps.nslots + threadIdx.x] = v;
+  double* rows = reinterpret_cast<double*>(acc);
+  if (threadIdx.x < ps.nslots) cg::this_cluster().map_shared_rank(rows, 0)[rank * ps.nslots + threadIdx.x] = v;
   bt_cluster_sync();
   if (rank == 0 && threadIdx.x == 0) {
     for (int k = ps.op_end - 1; k >= ps.op_begin; --k) {
       const BOp& op = d.ops[k];
       if (op.slot < 0) continue;
       double t = 0.0;
-      for (int q = 0; q < nr; ++q) t += acc[q * ps.nslots + op.slot];
+      for (int q = 0; q < nr; ++q) t += rows[q * ps.nslots + op.slot];
       d.grads[op.param] += t * op.gsign;
     }
   }
@@ -260,11 +265,11 @@ __device__ void bt_run_pass(const BatchArgs& d, const BPass& ps, double2* psi, d
 
 // Energy and gradient of one set, by CTA `rank` of `nr` cooperating CTAs.
 __device__ void bt_eval_set(const BatchArgs& d, int set_id, int rank, int nr, longlong2* tP, longlong2* tL,
-                            uint64_t* offs, double* acc, double* red, double* epart) {
+                            uint64_t* offs, int64_t* acc, double* red, double* epart, BStage* stage) {
   const BSet st = d.sets[set_id];
   const uint64_t N = 1ull << st.n;
-  double2* psi = d.psi + st.amp_off;
-  double2* lam = d.lam + st.amp_off;
+  longlong2* psi = d.psi + st.amp_off;
+  longlong2* lam = d.lam + st.amp_off;
   QC* matf = d.matf + 4 * (size_t)st.gate_begin;
   QC* matb = d.matb + 4 * (size_t)st.gate_begin;
   const int t0 = rank * BT_THREADS + threadIdx.x, ts = nr * BT_THREADS;
@@ -305,47 +310,45 @@ __device__ void bt_eval_set(const BatchArgs& d, int set_id, int rank, int nr, lo
       eb[idx] = qc_make_gauss(b.x, b.y);
     }
   }
+  // real pairs: w_a w_b / 2 and w_a conj(w_b) / 2 with w = c + i s (s negated: adjoint)
+  for (int pi = t0; pi < st.nrp; pi += ts) {
+    const int head = d.rphead[st.rp_begin + pi];
+    double c[2], s[2];
+    for (int mm = 0; mm < 2; ++mm) {
+      double2 mt[4];
+      bt_gate_matrix(d.gates[st.gate_begin + d.ops[head + 1 + mm].gate], d.params, false, mt);
+      c[mm] = mt[0].x;
+      s[mm] = mt[2].x;
+    }
+    for (int adj = 0; adj < 2; ++adj) {
+      const double sa = adj ? -s[0] : s[0], sb = adj ? -s[1] : s[1];
+      const double v[4] = {0.5 * (c[0] * c[1] - sa * sb), 0.5 * (sa * c[1] + c[0] * sb),
+                           0.5 * (c[0] * c[1] + sa * sb), 0.5 * (sa * c[1] - c[0] * sb)};
+      QL* o = (adj ? d.rpb : d.rpf) + 6 * (size_t)(st.rp_begin + pi);
+      for (int h = 0; h < 2; ++h) {
+        o[3 * h] = q60_split_coef(q60_from_double(v[2 * h]));
+        o[3 * h + 1] = q60_split_coef(q60_from_double(v[2 * h + 1]));
+        o[3 * h + 2] = q60_split_coef(q60_from_double(-v[2 * h + 1]));
+      }
+    }
+  }
   for (int j = t0; j < st.nparams; j += ts) d.grads[st.param_begin + j] = 0.0;
   // 2. psi = |0>, forward passes
-  for (uint64_t x = t0; x < N; x += ts) psi[x] = make_double2(x == 0 ? 1.0 : 0.0, 0.0);
+  for (uint64_t x = t0; x < N; x += ts) psi[x] = make_longlong2(x == 0 ? 1ll << 60 : 0, 0);
   if (nr == 1) __syncthreads();
   else bt_cluster_sync();
   for (int p = st.pass_begin; p < st.pass_begin + st.npasses; ++p)
-    bt_run_pass(d, d.passes[p], psi, lam, matf, matb, false, tP, tL, offs, acc, rank, nr);
-  // 3. lambda = (H/S) psi, energy, in Q60 integers (GB300's FP64 pipe would bound
-  // this loop): per group of terms sharing an X mask the signed coefficient sums
-  // d = sum_t (-1)^popc(x & zm_t) c_t are exact in int64 (sum |c_t| <= 1), the
-  // group's product d * psi_x is rounded once, and lambda_y = sum over groups
-  // (|lambda_y| <= |psi|_inf <= 1.25: every partial fits).
-  double e = 0.0;
+    bt_run_pass(d, d.passes[p], psi, lam, matf, matb, false, tP, tL, offs, acc, stage, rank, nr);
+  // 3. lambda = (H/S) psi and the energy Re <psi|lambda>, a sum of exact products
+  __int128 eq = 0;
   for (uint64_t y = t0; y < N; y += ts) {
-    int64_t ore = 0, oim = 0;
-    for (int gi = st.group_begin; gi < st.group_begin + st.ngroups; ++gi) {
-      const BGroup grp = d.groups[gi];
-      const uint64_t x = y ^ grp.xm;
-      int64_t dre = 0, dim = 0;
-      for (int k = grp.tbegin; k < grp.tend; ++k) {
-        const BTerm& t = d.terms[k];
-        const int64_t v = (__popcll(x & t.zm) & 1) ? -t.cq : t.cq;
-        if (t.imag) dim += v;
-        else dre += v;
-      }
-      const double2 pv = psi[x];
-      const QL px = q60_split(q60_from_double(pv.x)), py = q60_split(q60_from_double(pv.y));
-      const QL qr = q60_split(dre), qi = q60_split(dim), nqi = q60_split(-dim);
-      QAcc r = qacc_new(), i = qacc_new();
-      qacc_add(r, qr, px);   // re: dre px - dim py
-      qacc_add(r, nqi, py);
-      qacc_add(i, qr, py);   // im: dre py + dim px
-      qacc_add(i, qi, px);
-      ore += qacc_round(r);
-      oim += qacc_round(i);
-    }
-    const double lr = q60_to_double(ore), li = q60_to_double(oim);
-    lam[y] = make_double2(lr, li);
-    const double2 pyv = psi[y];
-    e += pyv.x * lr + pyv.y * li;
+    const longlong2 l = h_row(d.runs + st.run_begin, st.nruns, d.xms, d.groups + st.group_begin, st.ngroups, d.terms,
+                              y, [&](uint64_t x) { return psi[x]; });
+    lam[y] = l;
+    const longlong2 p = psi[y];
+    eq += (__int128)dot2_exact(split31(p.x), split31(l.x), split31(p.y), split31(l.y));
   }
+  const double e = q120_to_double(eq);
   const double E = bt_block_sum(e, red);
   if (nr == 1) {
     if (threadIdx.x == 0) d.energies[set_id] = E * st.S;
@@ -361,7 +364,7 @@ __device__ void bt_eval_set(const BatchArgs& d, int set_id, int rank, int nr, lo
   }
   // 4. backward
   for (int p = st.pass_begin + st.npasses - 1; p >= st.pass_begin; --p)
-    bt_run_pass(d, d.passes[p], psi, lam, matf, matb, true, tP, tL, offs, acc, rank, nr);
+    bt_run_pass(d, d.passes[p], psi, lam, matf, matb, true, tP, tL, offs, acc, stage, rank, nr);
   if (rank == 0 && threadIdx.x == 0)
     for (int j = 0; j < st.nparams; ++j) d.grads[st.param_begin + j] *= st.S;
 }
@@ -370,13 +373,16 @@ __device__ void bt_eval_set(const BatchArgs& d, int set_id, int rank, int nr, lo
 // cluster takes the next work item from the device counter (items pre-sorted by
 // decreasing estimated cost); the item is either one large set shared by the whole
 // cluster or up to d.csize small sets, one per CTA.
-__global__ void __launch_bounds__(BT_THREADS, 3) k_batch(const BatchArgs d) {
+// Two CTAs per SM: a third would leave 80 registers a thread and next to no L1 for what
+// they spill (128 sets of 10..18 qubits: 40.6 ms with three, 29.6 with two).
+__global__ void __launch_bounds__(BT_THREADS, 2) k_batch(const BatchArgs d) {
   extern __shared__ __align__(16) unsigned char smem[];
   longlong2* tP = reinterpret_cast<longlong2*>(smem);
   longlong2* tL = tP + (1 << BT_M);
   uint64_t* offs = reinterpret_cast<uint64_t*>(tL + (1 << BT_M));
-  double* acc = reinterpret_cast<double*>(offs + BT_OFFS);  // [warps][slots]; [rank][slot] across the cluster
-  double* red = acc + BT_MAX_OPS * (BT_THREADS / 32);
+  int64_t* acc = reinterpret_cast<int64_t*>(offs + BT_OFFS);  // [warps][slots]; [rank][slot] across the cluster
+  double* red = reinterpret_cast<double*>(acc + BT_MAX_OPS * BT_ACC_ROWS);
+  BStage* stage = reinterpret_cast<BStage*>(red + 8);
   __shared__ int s_item;
   __shared__ double s_epart[BT_CLUSTER];
   cg::cluster_group cl = cg::this_cluster();
@@ -396,13 +402,13 @@ __global__ void __launch_bounds__(BT_THREADS, 3) k_batch(const BatchArgs d) {
     } else if (rank < item.nsets) {
       set_id = item.sets[rank];
     }
-    if (set_id >= 0) bt_eval_set(d, set_id, r, nr, tP, tL, offs, acc, red, s_epart);
+    if (set_id >= 0) bt_eval_set(d, set_id, r, nr, tP, tL, offs, acc, red, s_epart, stage);
   }
 }
 
 size_t batch_smem_bytes() {
   return 2 * sizeof(longlong2) * (1 << BT_M) + sizeof(uint64_t) * BT_OFFS +
-         sizeof(double) * (BT_MAX_OPS * (BT_THREADS / 32) + 8);
+         sizeof(double) * (BT_MAX_OPS * BT_ACC_ROWS + 8) + sizeof(BStage);
 }
 
 static int bt_gen(int type) {
@@ -563,9 +569,11 @@ extern "C" int qs_batch_create(size_t nsets, const int* n_per_set, const qs_gate
   std::vector<BPass> passes;
   std::vector<BOp> ops;
   std::vector<BGate> bgates;
-  std::vector<BGroup> groups;
-  std::vector<BTerm> bterms;
-  std::vector<int> dgheads, dgsrc;
+  std::vector<HRun> runs;
+  std::vector<uint64_t> xms;
+  std::vector<HGroup> groups;
+  std::vector<HTerm> hterms;
+  std::vector<int> dgheads, dgsrc, rpheads;
   long long amp_off = 0;
   for (size_t si = 0; si < nsets; ++si) {
     const int n = n_per_set[si];
@@ -611,30 +619,17 @@ extern "C" int qs_batch_create(size_t nsets, const int* n_per_set, const qs_gate
       csum += fabs(terms[k].coef);
     }
     st.S = csum > 0 ? exp2(ceil(log2(csum))) : 1.0;
+    st.run_begin = (int)runs.size();
     st.group_begin = (int)groups.size();
-    std::vector<uint64_t> xms;
-    for (size_t k = t0; k < t1; ++k)
-      if (std::find(xms.begin(), xms.end(), terms[k].xmask) == xms.end()) xms.push_back(terms[k].xmask);
-    for (uint64_t xm : xms) {
-      BGroup grp;
-      grp.xm = xm;
-      grp.tbegin = (int)bterms.size();
-      for (size_t k = t0; k < t1; ++k) {
-        if (terms[k].xmask != xm) continue;
-        const int ny = __builtin_popcountll(terms[k].xmask & terms[k].zmask) & 3;
-        BTerm bt;
-        bt.c = (ny >= 2 ? -terms[k].coef : terms[k].coef) / st.S;
-        bt.cq = q60_from_double(bt.c);
-        bt.zm = terms[k].zmask;
-        bt.imag = ny & 1;
-        bterms.push_back(bt);
-      }
-      grp.tend = (int)bterms.size();
-      groups.push_back(grp);
+    {
+      std::vector<HRun> r;
+      h_plan(terms + t0, t1 - t0, st.S, &r, &xms, &groups, &hterms);
+      runs.insert(runs.end(), r.begin(), r.end());
     }
-    st.ngroups = (int)xms.size();
+    st.nruns = (int)runs.size() - st.run_begin;
+    st.ngroups = (int)groups.size() - st.group_begin;
     // greedy tile passes
-    const int dg_first = (int)dgheads.size();
+    const int dg_first = (int)dgheads.size(), rp_first = (int)rpheads.size();
     const int m = std::min(n, BT_M);
     const uint64_t low = (1ull << std::min(n, 3)) - 1;
     std::vector<uint32_t> remaining(ng), pass, rest;
@@ -682,16 +677,19 @@ extern "C" int qs_batch_create(size_t nsets, const int* n_per_set, const qs_gate
           op.kf = BK_SCALAR;
           op.kb = BK_SCALAR;
         }
+        op.rot = g.type == QS_RY;
         op.gen = g.param_idx >= 0 ? (int8_t)bt_gen(g.type) : BG_NONE;
         op.gsign = g.dagger ? -1.0 : 1.0;
         op.slot = -1;
         if (op.gen != BG_NONE) op.slot = (int16_t)slot++;
         ops.push_back(op);
       }
-      // (no real pairs here: their quad code alone pushes the batch kernel past its
-      // 80-register budget for three CTAs per SM; measured 847 -> 879 ms)
-      group_diagonals(ops, bp.op_begin, &dgheads, &dgsrc, nullptr);
+      bp.dg_begin = (int)dgheads.size();
+      bp.rp_begin = (int)rpheads.size();
+      group_diagonals(ops, bp.op_begin, &dgheads, &dgsrc, &rpheads);
       bp.op_end = (int)ops.size();
+      bp.dg_end = (int)dgheads.size();
+      bp.rp_end = (int)rpheads.size();
       bp.nslots = slot;
       passes.push_back(bp);
       remaining.swap(rest);
@@ -699,6 +697,8 @@ extern "C" int qs_batch_create(size_t nsets, const int* n_per_set, const qs_gate
     st.npasses = (int)passes.size() - st.pass_begin;
     st.dg_begin = dg_first;
     st.ndg = (int)dgheads.size() - dg_first;
+    st.rp_begin = rp_first;
+    st.nrp = (int)rpheads.size() - rp_first;
   }
   qs_batch* b = new (std::nothrow) qs_batch;
   if (!b) return fail(QS_ERR_OOM, "host allocation failed");
@@ -719,18 +719,24 @@ extern "C" int qs_batch_create(size_t nsets, const int* n_per_set, const qs_gate
   if (rc == QS_OK) chk(upload(b, passes, &a.passes));
   if (rc == QS_OK) chk(upload(b, ops, &a.ops));
   if (rc == QS_OK) chk(upload(b, bgates, &a.gates));
+  if (rc == QS_OK) chk(upload(b, runs, &a.runs));
+  if (rc == QS_OK) chk(upload(b, xms, &a.xms));
   if (rc == QS_OK) chk(upload(b, groups, &a.groups));
-  if (rc == QS_OK) chk(upload(b, bterms, &a.terms));
+  if (rc == QS_OK) chk(upload(b, hterms, &a.terms));
   if (rc == QS_OK) chk(upload(b, dgheads, &a.dghead));
   if (rc == QS_OK && chk(dev_alloc(b, std::max<size_t>(1, dgheads.size()) * 16 * sizeof(QC), &p0dg))) a.dgf = (QC*)p0dg;
   if (rc == QS_OK && chk(dev_alloc(b, std::max<size_t>(1, dgheads.size()) * 16 * sizeof(QC), &p0dg))) a.dgb = (QC*)p0dg;
+  if (rc == QS_OK) chk(upload(b, rpheads, &a.rphead));
+  const size_t rp_bytes = std::max<size_t>(1, rpheads.size()) * 6 * sizeof(QL);
+  if (rc == QS_OK && chk(dev_alloc(b, rp_bytes, &p0dg))) a.rpf = (QL*)p0dg;
+  if (rc == QS_OK && chk(dev_alloc(b, rp_bytes, &p0dg))) a.rpb = (QL*)p0dg;
   void* p = nullptr;
   const size_t np = std::max<size_t>(1, b->total_params);
   if (rc == QS_OK && chk(dev_alloc(b, np * sizeof(double), &p))) { a.params = (const double*)p; b->d_params = (double*)p; }
   if (rc == QS_OK && chk(dev_alloc(b, np * sizeof(double), &p))) a.grads = (double*)p;
   if (rc == QS_OK && chk(dev_alloc(b, nsets * sizeof(double), &p))) a.energies = (double*)p;
-  if (rc == QS_OK && chk(dev_alloc(b, (size_t)amp_off * sizeof(double2), &p))) a.psi = (double2*)p;
-  if (rc == QS_OK && chk(dev_alloc(b, (size_t)amp_off * sizeof(double2), &p))) a.lam = (double2*)p;
+  if (rc == QS_OK && chk(dev_alloc(b, (size_t)amp_off * sizeof(longlong2), &p))) a.psi = (longlong2*)p;
+  if (rc == QS_OK && chk(dev_alloc(b, (size_t)amp_off * sizeof(longlong2), &p))) a.lam = (longlong2*)p;
   if (rc == QS_OK && chk(dev_alloc(b, std::max<size_t>(1, bgates.size()) * 4 * sizeof(QC), &p))) a.matf = (QC*)p;
   if (rc == QS_OK && chk(dev_alloc(b, std::max<size_t>(1, bgates.size()) * 4 * sizeof(QC), &p))) a.matb = (QC*)p;
   if (rc == QS_OK && chk(dev_alloc(b, sizeof(int), &p))) a.counter = (int*)p;
@@ -743,6 +749,7 @@ extern "C" int qs_batch_create(size_t nsets, const int* n_per_set, const qs_gate
   if (rc == QS_OK) {
     b->smem = batch_smem_bytes();
     e = cudaFuncSetAttribute(k_batch, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)b->smem);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_batch, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     int sms = 0;
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, 0);
     if (e != cudaSuccess) chk(cuda_fail(e, "batch kernel set-up"));
@@ -758,6 +765,10 @@ extern "C" int qs_batch_create(size_t nsets, const int* n_per_set, const qs_gate
       batch_config(b, c * std::max(1, sms), &cfg, attr);
       int nclusters = 0;
       e = cudaOccupancyMaxActiveClusters(&nclusters, k_batch, &cfg);
+      if (e == cudaErrorInvalidClusterSize && c > 8) {  // not on this device
+        cudaGetLastError();
+        continue;
+      }
       if (e != cudaSuccess) {
         chk(cuda_fail(e, "cudaOccupancyMaxActiveClusters"));
         break;

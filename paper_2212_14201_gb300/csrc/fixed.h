@@ -113,6 +113,14 @@ QS_HD unsigned __int128 dot2_exact(Sp x1, Sp y1, Sp x2, Sp y2) {
   return ((u128)A << 62) + ((u128)B << 31) + (u128)C;
 }
 
+// A sum of such products (units 2^-120) as a double.
+QS_HD double q120_to_double(__int128 v) {
+  const bool neg = v < 0;
+  const unsigned __int128 m = neg ? (unsigned __int128)0 - (unsigned __int128)v : (unsigned __int128)v;
+  const double d = (double)(uint64_t)(m >> 64) * 0x1p-56 + (double)(uint64_t)m * 0x1p-120;
+  return neg ? -d : d;
+}
+
 // Nearest double to V * 2^-60 (round half to even).  Integer operations only.
 QS_HD double q60_to_double(int64_t V) {
   if (V == 0) return 0.0;

@@ -5,10 +5,14 @@
 
 #include <string.h>
 
+#include <algorithm>
+#include <utility>
+
 #include <vector>
 
 #include "fixed.h"
 #include "internal.h"
+#include "q60pair.cuh"
 
 namespace qs {
 
@@ -23,17 +27,20 @@ constexpr int BT_OFFS = 1 << (BT_M - 3);  // high-bit offset table: tiles hold q
 // of j (member m at bit m), E = the product of the members' diagonals (16 entries
 // per group, Gauss form).  The members follow the head as BK_MEMBER records
 // (nothing to run on their own) and keep their generator slots.
-// BK_RPAIR: two uncontrolled real ops on distinct tile qubits a (first member)
-// and b, run as one real 4x4 M = R_b (x) R_a on the quads (j, j|a, j|b, j|a|b)
-// (entries row-major, quad index 2*bit(b) + bit(a); 16 limb pairs per pair,
-// gate = pair index); in the backward sweep the op also takes both members'
-// generator terms from the quads it has loaded.
-enum : int8_t { BK_SCALAR = 9, BK_DGROUP = 10, BK_MEMBER = 11, BK_RPAIR = 12 };
+// BK_RPAIR: two uncontrolled real rotations on distinct tile qubits a (first member)
+// and b, run as two complex products on one component of the quads (j, j|a, j|b,
+// j|a|b) at a time (q60pair.cuh; 6 limb pairs per pair, gate = pair index); in the
+// backward sweep the op also takes both members' generator terms from the basis
+// that the products run in.
+// BK_PERM: a run of X and CNOT gates without a gradient, run as one permutation of
+// the tile (nmem members follow).
+enum : int8_t { BK_SCALAR = 9, BK_DGROUP = 10, BK_MEMBER = 11, BK_RPAIR = 12, BK_PERM = 13 };
 constexpr int BT_DG_MAX = 4;  // members per group
 enum : int8_t { BG_NONE = 0, BG_X = 1, BG_Y = 2, BG_Z = 3, BG_P = 4 };
 
 struct BPass {
   int m, nhigh, nout, op_begin, op_end, nslots;
+  int dg_begin, dg_end, rp_begin, rp_end;  // its diagonal groups and real pairs
   int qhigh[16];
   int outpos[32];
 };
@@ -49,7 +56,8 @@ struct BOp {
   int8_t tb;        // local target bit (global target bit for SCALAR)
   int8_t gen;
   int8_t c0f, c1f, c0b, c1b;
-  int8_t nmem;      // BK_DGROUP head: members following it (gate = group index)
+  int8_t nmem;      // group heads: members following it (gate = group index)
+  int8_t rot;       // a real rotation (determinant +1) for every angle
 };
 
 // Diagonal group (see BK_DGROUP): a_j *= E[idx(j)].
@@ -68,14 +76,6 @@ static __device__ void bt_apply_dgroup(longlong2* tile, uint32_t TS, const BOp* 
     q60_gauss_mul(u, q60_split(a.x), q60_split(a.y), q60_split(a.x + a.y), &re, &im);
     tile[j] = make_longlong2(re, im);
   }
-}
-
-// One output component of the 4x4 real M (row k) on four split inputs.
-__device__ __forceinline__ int64_t bt_row4(const QL* M, int k, const QL* x) {
-  QAcc acc = qacc_new();
-#pragma unroll
-  for (int c = 0; c < 4; ++c) qacc_add(acc, M[4 * k + c], x[c]);
-  return qacc_round(acc);
 }
 
 // Generator term of one pair (amplitudes 0 and 1 of the pair) for generator `gen`,
@@ -102,62 +102,119 @@ __device__ __forceinline__ int64_t bt_pair_gen(int gen, QL l0x, QL l0y, QL l1x, 
   return qaccf_result(pos) - qaccf_result(neg);
 }
 
-// Real pair forward: the quads of the tile through M.
+// The pair's two complex products on basis values u, v (see q60_pair_comp), back to
+// the quad at x[0], x[o01], x[o10], x[o11].
+__device__ __forceinline__ void bt_pair_products(const QL* c, int64_t ur, int64_t ui, int64_t vr, int64_t vi,
+                                                 int64_t* x, uint32_t o01, uint32_t o10, uint32_t o11) {
+  const QL a = q60_split(ur), b = q60_split(ui), d = q60_split(vr), e = q60_split(vi);
+  QAcc A = qacc_new(), B = qacc_new(), D = qacc_new(), E = qacc_new();
+  qacc_add(A, c[0], a);
+  qacc_add(A, c[2], b);
+  qacc_add(B, c[1], a);
+  qacc_add(B, c[0], b);
+  qacc_add(D, c[3], d);
+  qacc_add(D, c[5], e);
+  qacc_add(E, c[4], d);
+  qacc_add(E, c[3], e);
+  const int64_t Ur = qacc_round(A), Ui = qacc_round(B), Vr = qacc_round(D), Vi = qacc_round(E);
+  x[0] = Ur + Vr;
+  x[o01] = Ui + Vi;
+  x[o10] = Ui - Vi;
+  x[o11] = Vr - Ur;
+}
+
+// Real pair forward on one component a thread (12 wide multiply-adds a quad and
+// component for both rotations; as the real 4x4 matrix it took 48, as two single
+// rotations 48 and two sweeps).
 static __device__ __noinline__ void bt_rpair(longlong2* tile, uint32_t TS, uint32_t ta, uint32_t tbb,
-                                             const QL* __restrict__ M) {
+                                             const QL* __restrict__ cg) {
   const uint32_t lo = min(ta, tbb), hi = max(ta, tbb);
-  for (uint32_t i = threadIdx.x; i < (TS >> 2); i += BT_THREADS) {
+  const QL c[6] = {cg[0], cg[1], cg[2], cg[3], cg[4], cg[5]};
+  int64_t* comp = reinterpret_cast<int64_t*>(tile) + (threadIdx.x & 1);
+  for (uint32_t i = threadIdx.x >> 1; i < (TS >> 2); i += BT_THREADS / 2) {
     uint32_t j = i + (i & ~(lo - 1));
     j = j + (j & ~(hi - 1));
-    const uint32_t jj[4] = {j, j | ta, j | tbb, j | ta | tbb};
-    QL r[4], im[4];
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      const longlong2 v = tile[jj[c]];
-      r[c] = q60_split(v.x);
-      im[c] = q60_split(v.y);
-    }
-#pragma unroll
-    for (int k = 0; k < 4; ++k) tile[jj[k]] = make_longlong2(bt_row4(M, k, r), bt_row4(M, k, im));
+    int64_t* x = comp + 2 * j;
+    const int64_t p0 = x[0], p1 = x[2 * ta], p2 = x[2 * tbb], p3 = x[2 * (ta | tbb)];
+    bt_pair_products(c, p0 - p3, p1 + p2, p0 + p3, p1 - p2, x, 2 * ta, 2 * tbb, 2 * (ta | tbb));
   }
 }
 
-// Real pair backward: both members' generator terms (member a on the pairs
-// (0,1), (2,3) of the quad, member b on (0,2), (1,3)), then M on both tiles.
+// Real pair backward: the products on psi and lambda, and with gens the generator
+// terms of both members.  On one component, with z_b = p_b0 + i p_b1, u = z_0 + i z_1,
+// v = z_0 - i z_1 on psi and U, V the same on lambda, the members' terms
+//   a: sum_b l_b1 p_b0 - l_b0 p_b1,   b: sum_a l_1a p_0a - l_0a p_1a
+// are (Im conj(u) U +- Im conj(v) V) / 2: four products instead of eight.  *out_u and
+// *out_v receive the two sums over the tile (kept to all four limb products: they are
+// summed over the state; |sum| <= 2 ||psi|| ||lambda|| <= 3.2, below 2^62).
 static __device__ __noinline__ void bt_rpair_back(longlong2* P, longlong2* Lt, uint32_t TS, uint32_t ta,
-                                                  uint32_t tbb, int gen_a, int gen_b, const QL* __restrict__ M,
-                                                  int64_t* out_a, int64_t* out_b) {
-  int64_t sa = 0, sb = 0;
+                                                  uint32_t tbb, bool gens, const QL* __restrict__ cg, int64_t* out_u,
+                                                  int64_t* out_v) {
+  int64_t su = 0, sv = 0;
   const uint32_t lo = min(ta, tbb), hi = max(ta, tbb);
-  for (uint32_t i = threadIdx.x; i < (TS >> 2); i += BT_THREADS) {
+  const QL c[6] = {cg[0], cg[1], cg[2], cg[3], cg[4], cg[5]};
+  const uint32_t o01 = 2 * ta, o10 = 2 * tbb, o11 = 2 * (ta | tbb);
+  int64_t* cp = reinterpret_cast<int64_t*>(P) + (threadIdx.x & 1);
+  int64_t* cl = reinterpret_cast<int64_t*>(Lt) + (threadIdx.x & 1);
+  auto im = [](int64_t ar, int64_t ai, int64_t br, int64_t bi) {  // Im conj(a) b
+    QAccF acc{0, 0, 0};
+    qaccf_add(acc, q60_split(ar), q60_split(bi));
+    qaccf_add(acc, q60_split(-ai), q60_split(br));
+    return qaccf_result(acc);
+  };
+  for (uint32_t i = threadIdx.x >> 1; i < (TS >> 2); i += BT_THREADS / 2) {
     uint32_t j = i + (i & ~(lo - 1));
     j = j + (j & ~(hi - 1));
-    const uint32_t jj[4] = {j, j | ta, j | tbb, j | ta | tbb};
-    QL pr[4], pi[4], lr[4], li[4];
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      const longlong2 v = P[jj[c]], w = Lt[jj[c]];
-      pr[c] = q60_split(v.x);
-      pi[c] = q60_split(v.y);
-      lr[c] = q60_split(w.x);
-      li[c] = q60_split(w.y);
+    int64_t *x = cp + 2 * j, *y = cl + 2 * j;
+    const int64_t p0 = x[0], p1 = x[o01], p2 = x[o10], p3 = x[o11];
+    const int64_t l0 = y[0], l1 = y[o01], l2 = y[o10], l3 = y[o11];
+    const int64_t ur = p0 - p3, ui = p1 + p2, vr = p0 + p3, vi = p1 - p2;
+    const int64_t Ur = l0 - l3, Ui = l1 + l2, Vr = l0 + l3, Vi = l1 - l2;
+    if (gens) {
+      su += im(ur, ui, Ur, Ui);
+      sv += im(vr, vi, Vr, Vi);
     }
-    if (gen_a != BG_NONE) {
-      sa += bt_pair_gen(gen_a, lr[0], li[0], lr[1], li[1], pr[0], pi[0], pr[1], pi[1]);
-      sa += bt_pair_gen(gen_a, lr[2], li[2], lr[3], li[3], pr[2], pi[2], pr[3], pi[3]);
-    }
-    if (gen_b != BG_NONE) {
-      sb += bt_pair_gen(gen_b, lr[0], li[0], lr[2], li[2], pr[0], pi[0], pr[2], pi[2]);
-      sb += bt_pair_gen(gen_b, lr[1], li[1], lr[3], li[3], pr[1], pi[1], pr[3], pi[3]);
-    }
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      P[jj[k]] = make_longlong2(bt_row4(M, k, pr), bt_row4(M, k, pi));
-      Lt[jj[k]] = make_longlong2(bt_row4(M, k, lr), bt_row4(M, k, li));
+    bt_pair_products(c, ur, ui, vr, vi, x, o01, o10, o11);
+    bt_pair_products(c, Ur, Ui, Vr, Vi, y, o01, o10, o11);
+  }
+  *out_u = su;
+  *out_v = sv;
+}
+
+// A run of X and CNOT gates (members in program order, or reversed) as one
+// permutation of the tile P, and of Lt if given: amplitude j moves to the index that
+// the gates take j to.  That map is affine over bits, so a thread follows its first
+// index and the strides of its loop through the gates once.  (A sweep and a barrier
+// per gate otherwise, 11 of them for the ring of an ansatz layer.)
+static __device__ __noinline__ void bt_perm(longlong2* P, longlong2* Lt, uint32_t TS, const BOp* mem, int nm,
+                                            bool reverse, uint64_t base) {
+  constexpr int E = (1 << BT_M) / BT_THREADS;  // amplitudes per thread
+  uint32_t d = threadIdx.x, s0 = BT_THREADS, s1 = 2 * BT_THREADS, s2 = 4 * BT_THREADS;
+  static_assert(E == 8, "three stride bits");
+  for (int k = 0; k < nm; ++k) {
+    const BOp& op = mem[reverse ? nm - 1 - k : k];
+    if ((base & op.ext) != op.ext) continue;
+    const uint32_t c = op.lcm, t = 1u << op.tb;
+    if ((d & c) == c) d ^= t;
+    if (c) {  // the linear part: no control, no change
+      if (s0 & c) s0 ^= t;
+      if (s1 & c) s1 ^= t;
+      if (s2 & c) s2 ^= t;
     }
   }
-  *out_a = sa;
-  *out_b = sb;
+  for (int a = 0; a < 2; ++a) {
+    longlong2* tile = a ? Lt : P;
+    if (!tile) break;
+    longlong2 v[E];
+#pragma unroll
+    for (int e = 0; e < E; ++e)
+      if (threadIdx.x + e * BT_THREADS < TS) v[e] = tile[threadIdx.x + e * BT_THREADS];
+    __syncthreads();
+#pragma unroll
+    for (int e = 0; e < E; ++e)
+      if (threadIdx.x + e * BT_THREADS < TS)
+        tile[d ^ ((e & 1) ? s0 : 0u) ^ ((e & 2) ? s1 : 0u) ^ ((e & 4) ? s2 : 0u)] = v[e];
+  }
 }
 
 // Backward step of a diagonal group in one sweep: per amplitude the members'
@@ -437,23 +494,84 @@ static __device__ void bt_anti_both(longlong2* P, longlong2* Lt, uint32_t TS, co
   }
 }
 
-// Adds this thread's partial (Q60 units) to its warp's accumulator of `slot`
-// without a CTA barrier: the warp sums exactly by integer shuffles (the bound of
-// bt_gen_partial holds for the warp's total too), lane 0 converts once and owns
-// the warp's row, so the order of the FP64 additions is fixed.  wacc holds
-// (BT_THREADS / 32) rows of nslots.
-__device__ __forceinline__ void bt_warp_accumulate(int64_t v, double* wacc, int nslots, int slot) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += (int64_t)__shfl_xor_sync(0xffffffffu, (long long)v, o);
-  if ((threadIdx.x & 31) == 0) wacc[(threadIdx.x >> 5) * nslots + slot] += q60_to_double(v);
+// Sum over the warp, exactly: three integer reductions of 24, 24 and 16 bits.
+__device__ __forceinline__ int64_t bt_warp_sum(int64_t v) {
+  const uint32_t a = __reduce_add_sync(0xffffffffu, (uint32_t)v & 0xffffffu);
+  const uint32_t b = __reduce_add_sync(0xffffffffu, (uint32_t)(v >> 24) & 0xffffffu);
+  const int32_t c = __reduce_add_sync(0xffffffffu, (int32_t)(v >> 48));
+  return (int64_t)a + ((int64_t)b << 24) + (int64_t)c * (1ll << 48);
 }
 
-// After a barrier: the CTA's total of `slot`, warps added in warp order.
-__device__ __forceinline__ double bt_warp_total(const double* wacc, int nslots, int slot) {
-  double t = 0.0;
+// Adds this thread's partial to its warp's accumulator of `slot` without a CTA
+// barrier.  Accumulators hold twice the Q60 value (v2 = 2 x the partial) and stay
+// exact: a slot's sum over the whole state is below 4 in magnitude (bt_gen_partial),
+// twice that below 8 = 2^63.  wacc holds (BT_THREADS / 32) rows of nslots.  (As doubles
+// they took two FP64 instructions a slot, warp and op, 37 cycles of the SM's FP64 pipe
+// each, and a conversion.)
+__device__ __forceinline__ void bt_warp_accumulate(int64_t v2, int64_t* wacc, int nslots, int slot) {
+  v2 = bt_warp_sum(v2);
+  if ((threadIdx.x & 31) == 0) wacc[(threadIdx.x >> 5) * nslots + slot] += v2;
+}
+
+// After a barrier: the CTA's total of `slot`.
+__device__ __forceinline__ double bt_warp_total(const int64_t* wacc, int nslots, int slot) {
+  int64_t t = 0;
 #pragma unroll
   for (int w = 0; w < BT_THREADS / 32; ++w) t += wacc[w * nslots + slot];
-  return t;
+  return 0.5 * q60_to_double(t);
+}
+
+// The records a pass works from (ops, group diagonals, pair coefficients), copied to
+// shared memory where they fit: with the tiles there, the SM's L1 is too small to hold
+// them, and every op began with a chain of loads from L2.
+constexpr int BT_ST_OPS = 192, BT_ST_DG = 20, BT_ST_RP = 48;
+struct BStage {
+  BOp ops[BT_ST_OPS];
+  QC dg[16 * BT_ST_DG];
+  QL rp[6 * BT_ST_RP];
+};
+struct BRecords {  // indexed as the global arrays
+  const BOp* ops;
+  const QC* dg;
+  const QL* rp;
+};
+template <class T>
+__device__ __forceinline__ const T* bt_stage(T* dst, const T* src, int begin, int end, int per, int cap) {
+  if (end - begin > cap) return src;
+  static_assert(sizeof(T) % 8 == 0, "copied in 8-byte words");
+  const int words = (int)((end - begin) * per * (sizeof(T) / 8));
+  const uint64_t* s8 = reinterpret_cast<const uint64_t*>(src + (size_t)begin * per);
+  uint64_t* d8 = reinterpret_cast<uint64_t*>(dst);
+  for (int i = threadIdx.x; i < words; i += BT_THREADS) d8[i] = s8[i];
+  return dst - (ptrdiff_t)begin * per;
+}
+// (A barrier must follow before the records are read, and one must precede when the
+// stage holds another pass's.)
+__device__ __forceinline__ BRecords bt_records(BStage* st, const BPass& ps, const BOp* ops, const QC* dg,
+                                               const QL* rp) {
+  BRecords r;
+  r.ops = bt_stage(st->ops, ops, ps.op_begin, ps.op_end, 1, BT_ST_OPS);
+  r.dg = bt_stage(st->dg, dg, ps.dg_begin, ps.dg_end, 16, BT_ST_DG);
+  r.rp = bt_stage(st->rp, rp, ps.rp_begin, ps.rp_end, 6, BT_ST_RP);
+  return r;
+}
+
+// Tile loads and stores.  (Eight loads in flight per thread were slower: their
+// registers spill.)
+__device__ __forceinline__ void bt_load(longlong2* tile, const longlong2* src, uint64_t base, const uint64_t* offs,
+                                        int L, uint32_t TS) {
+  const uint32_t lowmask = (1u << L) - 1;
+  for (uint32_t j = threadIdx.x; j < TS; j += BT_THREADS) tile[j] = src[base + offs[j >> L] + (j & lowmask)];
+}
+__device__ __forceinline__ void bt_store(const longlong2* tile, longlong2* dst, uint64_t base, const uint64_t* offs,
+                                         int L, uint32_t TS) {
+  constexpr int E = (1 << BT_M) / BT_THREADS;
+  const uint32_t lowmask = (1u << L) - 1;
+#pragma unroll
+  for (int e = 0; e < E; ++e) {
+    const uint32_t j = threadIdx.x + e * BT_THREADS;
+    if (j < TS) dst[base + offs[j >> L] + (j & lowmask)] = tile[j];
+  }
 }
 
 static __device__ double bt_block_sum(double v, double* red) {
@@ -469,26 +587,189 @@ static __device__ double bt_block_sum(double v, double* red) {
   return r;
 }
 
+// ---- lambda = (H / S) psi -------------------------------------------------------------
+// The terms of H / S as
+//   runs    X masks whose only term has no Z and the same real coefficient: their
+//           amplitudes are added first and multiplied once;
+//   groups  every other X mask, with its terms: the signed coefficient sums
+//           d = sum_t (-1)^popc(x & zm_t) c_t are exact in int64 (sum |c_t| <= 1).
+// |lambda_y| <= |psi|_inf <= 1.25 and every product is rounded once.
+constexpr int HRUN_MAX = 32;  // a run's amplitude sum stays below sqrt(32) * 1.25 < 8
+struct HRun {
+  int64_t c;  // coef / S, Q60
+  int begin, end;
+};
+struct HGroup {
+  uint64_t xm;
+  int begin, end, imag;  // imag: some term has an imaginary factor
+};
+struct HTerm {
+  int64_t c;  // coef / S with the real sign of i^ny, Q60
+  uint64_t zm;
+  int imag;   // i^ny is imaginary
+};
+
+// The runs, groups and terms of a Pauli sum; xms: the X masks of the runs in order.
+static inline void h_plan(const qs_pauli* terms, size_t nt, double S, std::vector<HRun>* runs,
+                          std::vector<uint64_t>* xms, std::vector<HGroup>* groups, std::vector<HTerm>* hterms) {
+  std::vector<uint64_t> order;
+  std::vector<std::vector<size_t>> of;
+  for (size_t k = 0; k < nt; ++k) {  // by X mask, in order of first appearance
+    size_t g = 0;
+    while (g < order.size() && order[g] != terms[k].xmask) ++g;
+    if (g == order.size()) {
+      order.push_back(terms[k].xmask);
+      of.emplace_back();
+    }
+    of[g].push_back(k);
+  }
+  std::vector<std::pair<int64_t, uint64_t>> plain;
+  for (size_t g = 0; g < order.size(); ++g) {
+    if (of[g].size() == 1 && terms[of[g][0]].zmask == 0) {
+      plain.push_back({q60_from_double(terms[of[g][0]].coef / S), order[g]});
+      continue;
+    }
+    HGroup gr{order[g], (int)hterms->size(), 0, 0};
+    for (size_t k : of[g]) {
+      const int ny = __builtin_popcountll(terms[k].xmask & terms[k].zmask) & 3;
+      const double c = terms[k].coef / S;
+      hterms->push_back(HTerm{q60_from_double(ny >= 2 ? -c : c), terms[k].zmask, ny & 1});
+      gr.imag |= ny & 1;
+    }
+    gr.end = (int)hterms->size();
+    groups->push_back(gr);
+  }
+  std::stable_sort(plain.begin(), plain.end(),
+                   [](const auto& a, const auto& b) { return a.first < b.first; });
+  for (size_t k = 0; k < plain.size(); ++k) {
+    if (k == 0 || runs->back().c != plain[k].first || runs->back().end - runs->back().begin == HRUN_MAX)
+      runs->push_back(HRun{plain[k].first, (int)xms->size(), (int)xms->size()});
+    xms->push_back(plain[k].second);
+    ++runs->back().end;
+  }
+}
+
+#ifdef __CUDACC__
+// c * s for a Q60 coefficient |c| <= 1 and a sum |s| < 8, rounded once: limbs of 32
+// bits with signed low limbs, c in units of 2^-62.
+__device__ __forceinline__ int64_t h_mul_sum(int64_t c, int64_t s) {
+  const int64_t C = c << 2;
+  const int32_t cl = (int32_t)C, sl = (int32_t)s;
+  const int32_t ch = (int32_t)(C >> 32) + (int32_t)((uint32_t)cl >> 31);
+  const int32_t sh = (int32_t)(s >> 32) + (int32_t)((uint32_t)sl >> 31);
+  const int64_t hi = madw(ch, sh, 0), mid = madw(cl, sh, madw(ch, sl, 1ll << 29));
+  return (hi << 2) + (mid >> 30);
+}
+
+__device__ __forceinline__ bool h_parity(uint64_t x, uint64_t zm) {
+  const uint32_t hi = (uint32_t)(x >> 32) & (uint32_t)(zm >> 32);
+  return __popc(((uint32_t)x & (uint32_t)zm) ^ hi) & 1;
+}
+
+// Row y of (H / S) psi; load(x) gives psi_x in Q60.
+template <class F>
+__device__ __forceinline__ longlong2 h_row(const HRun* runs, int nruns, const uint64_t* xms, const HGroup* groups,
+                                           int ngroups, const HTerm* terms, uint64_t y, F&& load) {
+  int64_t ore = 0, oim = 0;
+  for (int r = 0; r < nruns; ++r) {
+    const HRun run = runs[r];
+    int64_t sr = 0, si = 0;
+    int k = run.begin;
+    for (; k + 4 <= run.end; k += 4) {  // four gathers in flight
+      const longlong2 a = load(y ^ xms[k]), b = load(y ^ xms[k + 1]), c = load(y ^ xms[k + 2]),
+                      d = load(y ^ xms[k + 3]);
+      sr += (a.x + b.x) + (c.x + d.x);
+      si += (a.y + b.y) + (c.y + d.y);
+    }
+    for (; k < run.end; ++k) {
+      const longlong2 a = load(y ^ xms[k]);
+      sr += a.x;
+      si += a.y;
+    }
+    ore += h_mul_sum(run.c, sr);
+    oim += h_mul_sum(run.c, si);
+  }
+  for (int g = 0; g < ngroups; ++g) {
+    const HGroup gr = groups[g];
+    const uint64_t x = y ^ gr.xm;
+    const longlong2 p = load(x);
+    int64_t dre = 0, dim = 0;
+    if (!gr.imag) {
+      for (int k = gr.begin; k < gr.end; ++k) {
+        const int64_t c = terms[k].c;
+        dre += h_parity(x, terms[k].zm) ? -c : c;
+      }
+    } else {
+      for (int k = gr.begin; k < gr.end; ++k) {
+        const int64_t v = h_parity(x, terms[k].zm) ? -terms[k].c : terms[k].c;
+        if (terms[k].imag) dim += v;
+        else dre += v;
+      }
+    }
+    const QL px = q60_split(p.x), py = q60_split(p.y), qr = q60_split_coef(dre);
+    QAcc re = qacc_new(), im = qacc_new();
+    qacc_add(re, qr, px);  // re: dre px - dim py
+    qacc_add(im, qr, py);  // im: dre py + dim px
+    if (gr.imag) {
+      qacc_add(re, q60_split_coef(-dim), py);
+      qacc_add(im, q60_split_coef(dim), px);
+    }
+    ore += qacc_round(re);
+    oim += qacc_round(im);
+  }
+  return make_longlong2(ore, oim);
+}
+#endif
+
 // Runs of up to BT_DG_MAX consecutive uncontrolled diagonal ops (forward and
 // adjoint class) on distinct tile qubits, with a Z, P or no generator, of the
 // ops [begin, end) become diagonal groups: a BK_DGROUP head (gate = group index,
 // nmem members) is inserted before the members, which turn into BK_MEMBER
 // records.  Heads are appended to `heads` (their index in the new op list);
 // src[i - begin] receives the old index of new op i (-1 for a head).
-// Consecutive uncontrolled real ops on distinct tile qubits become real pairs
-// the same way (a BK_RPAIR head, gate = index into `pairs`, two BK_MEMBER records).
+// Consecutive uncontrolled real rotations on distinct tile qubits become real pairs
+// the same way (a BK_RPAIR head, gate = index into `pairs`, two BK_MEMBER records),
+// and runs of X and CNOT gates without a gradient permutations (a BK_PERM head).
 static inline void group_diagonals(std::vector<BOp>& ops, size_t begin, std::vector<int>* heads,
-                                   std::vector<int>* src, std::vector<int>* pairs = nullptr) {
+                                   std::vector<int>* src, std::vector<int>* pairs) {
   auto eligible = [](const BOp& o) {
     const bool df = o.kf == OP_DIAG || o.kf == OP_PHASE1, db = o.kb == OP_DIAG || o.kb == OP_PHASE1;
     return df && db && o.lcm == 0 && o.ext == 0 && (o.gen == BG_NONE || o.gen == BG_Z || o.gen == BG_P);
   };
-  auto real = [](const BOp& o) { return o.kf == OP_REAL && o.kb == OP_REAL && o.lcm == 0 && o.ext == 0; };
+  auto real = [](const BOp& o) {
+    return o.kf == OP_REAL && o.kb == OP_REAL && o.rot && o.lcm == 0 && o.ext == 0 &&
+           (o.gen == BG_NONE || o.gen == BG_Y);
+  };
+  auto swaps = [](const BOp& o) {
+    return o.kf == OP_ANTI && o.kb == OP_ANTI && o.c0f == U_ONE && o.c1f == U_ONE && o.c0b == U_ONE &&
+           o.c1b == U_ONE && __builtin_popcount(o.lcm) <= 1 && o.gen == BG_NONE;
+  };
   std::vector<BOp> out(ops.begin(), ops.begin() + begin);
   src->clear();
   size_t i = begin;
   while (i < ops.size()) {
-    if (pairs && i + 1 < ops.size() && real(ops[i]) && real(ops[i + 1]) && ops[i].tb != ops[i + 1].tb) {
+    size_t run = i;
+    while (run < ops.size() && run - i < 127 && swaps(ops[run])) ++run;
+    if (run - i >= 2) {
+      BOp h;
+      memset(&h, 0, sizeof h);
+      h.kf = h.kb = BK_PERM;
+      h.nmem = (int8_t)(run - i);
+      h.slot = -1;
+      h.param = -1;
+      h.gen = BG_NONE;
+      out.push_back(h);
+      src->push_back(-1);
+      for (size_t k = i; k < run; ++k) {
+        BOp mo = ops[k];
+        mo.kf = mo.kb = BK_MEMBER;
+        out.push_back(mo);
+        src->push_back((int)k);
+      }
+      i = run;
+      continue;
+    }
+    if (i + 1 < ops.size() && real(ops[i]) && real(ops[i + 1]) && ops[i].tb != ops[i + 1].tb) {
       BOp h;
       memset(&h, 0, sizeof h);
       h.kf = h.kb = BK_RPAIR;
