@@ -290,8 +290,15 @@ struct Trajectory {
     } else {
       if (joint_bit(q) < 0) QS_TRY(read_joint(ahead()));
       const int b = joint_bit(q);
-      double p[2] = {0.0, 0.0};
-      for (size_t k = 0; k < joint.size(); ++k) p[(k >> b) & 1] += joint[k];
+      // four sums per outcome: one would wait for every addition before the next
+      double s0[4] = {0, 0, 0, 0}, s1[4] = {0, 0, 0, 0};
+      const size_t h = (size_t)1 << b, half = joint.size() / 2;
+      for (size_t k = 0; k < half; ++k) {
+        const size_t j = k + (k & ~(h - 1));  // bit b clear
+        s0[k & 3] += joint[j];
+        s1[k & 3] += joint[j + h];
+      }
+      const double p[2] = {(s0[0] + s0[1]) + (s0[2] + s0[3]), (s1[0] + s1[1]) + (s1[2] + s1[3])};
       for (int j = 0; j < ks.m; ++j) {
         const Mat2& K = ks.K[j];
         w[j] = (K.m[0].re * K.m[0].re + K.m[2].re * K.m[2].re) * p[0] +
