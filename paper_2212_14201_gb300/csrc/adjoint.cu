@@ -265,7 +265,7 @@ struct AdjPassArgs {
   const BOp* ops;   // ops of this pass (device), in execution order
   const QC* mats;   // 4 entries per op (device)
   const QC* dgm;    // 16 entries per diagonal group (device)
-  const QL* rpm;    // 6 entries per real pair (device)
+  const QP* rpm;    // 2 entries per real pair (device)
   double* part;     // [slot][ADJ_GRID_STRIDE]
   int slot_base;
 };
@@ -316,7 +316,7 @@ __global__ void __launch_bounds__(BT_THREADS, 3) k_adj_pass(longlong2* __restric
         const BOp* mem = a.ops + k + 1;
         int64_t gu, gv;
         bt_rpair_back(tP, tL, TS, 1u << mem[0].tb, 1u << mem[1].tb, mem[0].slot >= 0 || mem[1].slot >= 0,
-                      a.rpm + 6 * op.gate, &gu, &gv);
+                      a.rpm + 2 * op.gate, &gu, &gv);
         if (mem[0].slot >= 0) bt_warp_accumulate(gu + gv, wacc, ps.nslots, mem[0].slot);
         if (mem[1].slot >= 0) bt_warp_accumulate(gu - gv, wacc, ps.nslots, mem[1].slot);
         __syncthreads();
@@ -378,7 +378,7 @@ static int backward_fused(qs_state* s, double2* lam, const qs_gate* gates, size_
   std::vector<QC> mats;
   std::vector<QC> dgm;    // 16 Gauss-form entries per diagonal group
   std::vector<int> dgheads, dgsrc, rpheads;
-  std::vector<QL> rpm;    // 6 limb pairs per real pair
+  std::vector<QP> rpm;    // 2 coefficients per real pair
   std::vector<BPass> passes;
   int slot_base = 0;
   std::vector<int> slot_bases;
@@ -471,10 +471,10 @@ static int backward_fused(qs_state* s, double2* lam, const qs_gate* gates, size_
         ra[e] = opm[rpheads[pi] + 1].m[e].re;
         rb[e] = opm[rpheads[pi] + 2].m[e].re;
       }
-      QL c[6];
+      QP c[2];
       int flags;  // rotations: 0
-      q60_pair_coef(ra, rb, c, &flags);
-      rpm.insert(rpm.end(), c, c + 6);
+      q60_pair_gauss_coef(ra, rb, c, &flags);
+      rpm.insert(rpm.end(), c, c + 2);
     }
     bp.op_end = (int)ops.size();
     bp.nslots = slot;
@@ -487,7 +487,7 @@ static int backward_fused(qs_state* s, double2* lam, const qs_gate* gates, size_
   // memory of this call)
   auto up16 = [](size_t b) { return (b + 15) & ~(size_t)15; };
   const size_t ob = up16(sizeof(BOp) * ops.size()), mb = up16(sizeof(QC) * mats.size()),
-               db = up16(sizeof(QC) * dgm.size()), rb = up16(sizeof(QL) * rpm.size()), total = ob + mb + db + rb;
+               db = up16(sizeof(QC) * dgm.size()), rb = up16(sizeof(QP) * rpm.size()), total = ob + mb + db + rb;
   ScratchBuf big;
   char* dev = (char*)s->ws;
   if (total > s->ws_bytes) {
@@ -499,12 +499,12 @@ static int backward_fused(qs_state* s, double2* lam, const qs_gate* gates, size_
   if (!ops.empty()) memcpy(host, ops.data(), sizeof(BOp) * ops.size());
   if (!mats.empty()) memcpy(host + ob, mats.data(), sizeof(QC) * mats.size());
   if (!dgm.empty()) memcpy(host + ob + mb, dgm.data(), sizeof(QC) * dgm.size());
-  if (!rpm.empty()) memcpy(host + ob + mb + db, rpm.data(), sizeof(QL) * rpm.size());
+  if (!rpm.empty()) memcpy(host + ob + mb + db, rpm.data(), sizeof(QP) * rpm.size());
   cudaError_t e = total ? cudaMemcpyAsync(dev, host, total, cudaMemcpyHostToDevice, s->stream) : cudaSuccess;
   const BOp* d_ops = (const BOp*)dev;
   const QC* d_mats = (const QC*)(dev + ob);
   const QC* d_dgm = (const QC*)(dev + ob + mb);
-  const QL* d_rpm = (const QL*)(dev + ob + mb + db);
+  const QP* d_rpm = (const QP*)(dev + ob + mb + db);
   int rc = e == cudaSuccess ? QS_OK : cuda_fail(e, "adjoint op tables");
   static bool attr = false;
   if (rc == QS_OK && !attr) {

@@ -82,8 +82,8 @@ struct BatchArgs {
   QC* dgf;    // 16 per diagonal group (Gauss form), forward
   QC* dgb;    // 16 per diagonal group, adjoint
   const int* rphead;  // per real pair: global index of its head op
-  QL* rpf;    // 6 limb pairs per real pair, forward
-  QL* rpb;    // 6 limb pairs per real pair, adjoint
+  QP* rpf;    // 2 coefficients per real pair, forward
+  QP* rpb;    // 2 coefficients per real pair, adjoint
   int* counter;
 };
 
@@ -176,7 +176,7 @@ __device__ void bt_run_pass(const BatchArgs& d, const BPass& ps, longlong2* psi,
         const BOp& op = rec.ops[k];
         if (op.kf == BK_MEMBER || (base & op.ext) != op.ext) continue;
         if (op.kf == BK_DGROUP) bt_apply_dgroup(tP, TS, rec.ops + k + 1, op.nmem, rec.dg + 16 * op.gate);
-        else if (op.kf == BK_RPAIR) bt_rpair(tP, TS, 1u << rec.ops[k + 1].tb, 1u << rec.ops[k + 2].tb, rec.rp + 6 * op.gate);
+        else if (op.kf == BK_RPAIR) bt_rpair(tP, TS, 1u << rec.ops[k + 1].tb, 1u << rec.ops[k + 2].tb, rec.rp + 2 * op.gate);
         else if (op.kf == BK_PERM) bt_perm(tP, nullptr, TS, rec.ops + k + 1, op.nmem, false, base);
         else bt_apply(tP, TS, op, op.kf, op.c0f, op.c1f, matf + 4 * op.gate, base);
         __syncthreads();
@@ -199,7 +199,7 @@ __device__ void bt_run_pass(const BatchArgs& d, const BPass& ps, longlong2* psi,
           const BOp* mem = rec.ops + k + 1;
           int64_t gu, gv;
           bt_rpair_back(tP, tL, TS, 1u << mem[0].tb, 1u << mem[1].tb, mem[0].slot >= 0 || mem[1].slot >= 0,
-                        rec.rp + 6 * op.gate, &gu, &gv);
+                        rec.rp + 2 * op.gate, &gu, &gv);
           if (mem[0].slot >= 0) bt_warp_accumulate(gu + gv, acc, ps.nslots, mem[0].slot);
           if (mem[1].slot >= 0) bt_warp_accumulate(gu - gv, acc, ps.nslots, mem[1].slot);
           __syncthreads();
@@ -322,14 +322,9 @@ __device__ void bt_eval_set(const BatchArgs& d, int set_id, int rank, int nr, lo
     }
     for (int adj = 0; adj < 2; ++adj) {
       const double sa = adj ? -s[0] : s[0], sb = adj ? -s[1] : s[1];
-      const double v[4] = {0.5 * (c[0] * c[1] - sa * sb), 0.5 * (sa * c[1] + c[0] * sb),
-                           0.5 * (c[0] * c[1] + sa * sb), 0.5 * (sa * c[1] - c[0] * sb)};
-      QL* o = (adj ? d.rpb : d.rpf) + 6 * (size_t)(st.rp_begin + pi);
-      for (int h = 0; h < 2; ++h) {
-        o[3 * h] = q60_split_coef(q60_from_double(v[2 * h]));
-        o[3 * h + 1] = q60_split_coef(q60_from_double(v[2 * h + 1]));
-        o[3 * h + 2] = q60_split_coef(q60_from_double(-v[2 * h + 1]));
-      }
+      QP* o = (adj ? d.rpb : d.rpf) + 2 * (size_t)(st.rp_begin + pi);
+      o[0] = qp_coef(q60_from_double(0.5 * (c[0] * c[1] - sa * sb)), q60_from_double(0.5 * (sa * c[1] + c[0] * sb)));
+      o[1] = qp_coef(q60_from_double(0.5 * (c[0] * c[1] + sa * sb)), q60_from_double(0.5 * (sa * c[1] - c[0] * sb)));
     }
   }
   for (int j = t0; j < st.nparams; j += ts) d.grads[st.param_begin + j] = 0.0;
@@ -727,9 +722,9 @@ extern "C" int qs_batch_create(size_t nsets, const int* n_per_set, const qs_gate
   if (rc == QS_OK && chk(dev_alloc(b, std::max<size_t>(1, dgheads.size()) * 16 * sizeof(QC), &p0dg))) a.dgf = (QC*)p0dg;
   if (rc == QS_OK && chk(dev_alloc(b, std::max<size_t>(1, dgheads.size()) * 16 * sizeof(QC), &p0dg))) a.dgb = (QC*)p0dg;
   if (rc == QS_OK) chk(upload(b, rpheads, &a.rphead));
-  const size_t rp_bytes = std::max<size_t>(1, rpheads.size()) * 6 * sizeof(QL);
-  if (rc == QS_OK && chk(dev_alloc(b, rp_bytes, &p0dg))) a.rpf = (QL*)p0dg;
-  if (rc == QS_OK && chk(dev_alloc(b, rp_bytes, &p0dg))) a.rpb = (QL*)p0dg;
+  const size_t rp_bytes = std::max<size_t>(1, rpheads.size()) * 2 * sizeof(QP);
+  if (rc == QS_OK && chk(dev_alloc(b, rp_bytes, &p0dg))) a.rpf = (QP*)p0dg;
+  if (rc == QS_OK && chk(dev_alloc(b, rp_bytes, &p0dg))) a.rpb = (QP*)p0dg;
   void* p = nullptr;
   const size_t np = std::max<size_t>(1, b->total_params);
   if (rc == QS_OK && chk(dev_alloc(b, np * sizeof(double), &p))) { a.params = (const double*)p; b->d_params = (double*)p; }

@@ -252,14 +252,16 @@ QS_HD QC qc_make(double re, double im) {
 
 // Gauss (three-multiplication) form of an entry c + i d, for the product
 // (a + i b)(c + i d) = [c (a + b) - b (c + d)] + i [c (a + b) + a (d - c)]:
-// re = c, im = d - c, nim = c + d, each from the Q60-rounded c and d, so the
+// re = c, im = d - c, nim = -(c + d), each from the Q60-rounded c and d, so the
 // represented matrix is exactly the one qc_make() gives.  |c +- d| <= sqrt(2)|u|.
+// Both outputs start from the accumulator of c (a + b): nine wide multiply-adds and
+// no addition of accumulators.
 QS_HD QC qc_make_gauss(double re, double im) {
   const int64_t c = q60_from_double(re), d = q60_from_double(im);
   QC q;
   q.re = q60_split_coef(c);
   q.im = q60_split_coef(d - c);
-  q.nim = q60_split_coef(c + d);
+  q.nim = q60_split_coef(-(c + d));
   return q;
 }
 
@@ -269,26 +271,28 @@ QS_HD QC qc_make_gauss(double re, double im) {
 // Six limb products (18 wide multiply-adds) instead of eight.
 QS_HD void q60_gauss_row(const QC& u0, const QC& u1, QL r0, QL i0, QL s0, QL r1, QL i1, QL s1, int64_t* re,
                          int64_t* im) {
-  QAcc k1 = qacc_new(), k2{0, 0}, k3{0, 0};
-  qacc_add(k1, u0.re, s0);
-  qacc_add(k1, u1.re, s1);
-  qacc_add(k2, u0.im, r0);
-  qacc_add(k2, u1.im, r1);
-  qacc_add(k3, u0.nim, i0);
-  qacc_add(k3, u1.nim, i1);
-  *re = qacc_round(QAcc{k1.hi - k3.hi, k1.mid - k3.mid});
-  *im = qacc_round(QAcc{k1.hi + k2.hi, k1.mid + k2.mid});
+  QAcc x = qacc_new();
+  qacc_add(x, u0.re, s0);
+  qacc_add(x, u1.re, s1);
+  QAcc y = x;
+  qacc_add(x, u0.nim, i0);
+  qacc_add(x, u1.nim, i1);
+  qacc_add(y, u0.im, r0);
+  qacc_add(y, u1.im, r1);
+  *re = qacc_round(x);
+  *im = qacc_round(y);
 }
 
 // One complex product u * a in Gauss form (u from qc_make_gauss), a = r + i i,
 // s = r + i (split): three limb products.
 QS_HD void q60_gauss_mul(const QC& u, QL r, QL i, QL s, int64_t* re, int64_t* im) {
-  QAcc k1 = qacc_new(), k2{0, 0}, k3{0, 0};
-  qacc_add(k1, u.re, s);
-  qacc_add(k2, u.im, r);
-  qacc_add(k3, u.nim, i);
-  *re = qacc_round(QAcc{k1.hi - k3.hi, k1.mid - k3.mid});
-  *im = qacc_round(QAcc{k1.hi + k2.hi, k1.mid + k2.mid});
+  QAcc x = qacc_new();
+  qacc_add(x, u.re, s);
+  QAcc y = x;
+  qacc_add(x, u.nim, i);
+  qacc_add(y, u.im, r);
+  *re = qacc_round(x);
+  *im = qacc_round(y);
 }
 
 }  // namespace qs

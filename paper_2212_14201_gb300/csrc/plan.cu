@@ -1542,31 +1542,31 @@ static int build_tile_args(int n, int prec, const PlanPass& ps, const qs_gate* g
       const size_t r = e - i;
       if (r >= 5 && r % 4 != 0) lead = r % 4 == 2 ? 2 : 3;
     }
-    if (lead == 0 && pairs && quads && !f32 && i + 3 < rops.size() && g->nops + 3 <= TILE_MAX_OPS && in_tile_real(op) &&
+    if (lead == 0 && pairs && quads && !f32 && i + 3 < rops.size() && g->nops + 2 <= TILE_MAX_OPS && in_tile_real(op) &&
         in_tile_real(rops[i + 1]) && in_tile_real(rops[i + 2]) && in_tile_real(rops[i + 3])) {
       const uint32_t tm = (1u << local[op.target]) | (1u << local[rops[i + 1].target]) |
                           (1u << local[rops[i + 2].target]) | (1u << local[rops[i + 3].target]);
       if (__builtin_popcount(tm) == 4) {
         // four real rotations on different tile qubits: one op on one component of
-        // 16 amplitudes at a time (three slots); a table before it stays its own op
+        // 16 amplitudes at a time (two slots); a table before it stays its own op
         TileOp* t = &g->ops[g->nops];
-        memset(t, 0, 3 * sizeof(TileOp));
+        memset(t, 0, 2 * sizeof(TileOp));
         t[0].kind = TOP_REAL4;
         t[0].tb = (int8_t)local[op.target];
         t[0].code0 = (int8_t)local[rops[i + 1].target];
         t[0].code1 = -1;
-        t[1].kind = t[2].kind = TOP_CONT;
+        t[1].kind = TOP_CONT;
         double mr[4][4];
         for (int q = 0; q < 4; ++q)
           for (int e = 0; e < 4; ++e) mr[q][e] = rops[i + q].m.m[e].re;
-        Q3 P[24];
+        QW G[24];
         int flags = 0;
-        q60_quad4_coef(mr[0], mr[1], mr[2], mr[3], P, &flags);
-        for (int e = 0; e < 24; ++e) reinterpret_cast<Q3*>(t[e / 8].q)[e % 8] = P[e];
+        q60_quad4_gauss_coef(mr[0], mr[1], mr[2], mr[3], G, &flags);
+        for (int e = 0; e < 24; ++e) reinterpret_cast<QW*>(t[e / 12].q)[e % 12] = G[e];
         t[0].lcmask = (uint32_t)flags | ((uint32_t)local[rops[i + 2].target] << 8) |
                       ((uint32_t)local[rops[i + 3].target] << 16);
-        int_ops += N * 12.0;  // 32 real products per 16 values of a component: 12 limb products per amplitude
-        g->nops += 3;
+        int_ops += N * 12.0;  // as four real products a complex product (the planner's unit)
+        g->nops += 2;
         i += 3;
         continue;
       }
@@ -1574,7 +1574,7 @@ static int build_tile_args(int n, int prec, const PlanPass& ps, const qs_gate* g
     if (lead != 2 && pairs && triples && !f32 && i + 2 < rops.size() && in_tile_real(op) && in_tile_real(rops[i + 1]) &&
         in_tile_real(rops[i + 2]) && rops[i + 1].target != op.target && rops[i + 2].target != op.target &&
         rops[i + 2].target != rops[i + 1].target) {
-      // three real rotations on different tile qubits: one op on octets (two slots)
+      // three real rotations on different tile qubits: one op on octets
       int tab = -1;
       if (g_fuse_tables && i > 0 && rops[i - 1].cls == kTableMark && g->nops > 0 &&
           g->ops[g->nops - 1].kind == TOP_DTABLE && g->ops[g->nops - 1].lcmask < 128) {
@@ -1582,31 +1582,22 @@ static int build_tile_args(int n, int prec, const PlanPass& ps, const qs_gate* g
         tab = (int)g->ops[g->nops].lcmask;
       }
       TileOp& t0 = g->ops[g->nops];
-      TileOp& t1 = g->ops[g->nops + 1];
       memset(&t0, 0, sizeof t0);
-      memset(&t1, 0, sizeof t1);
       t0.kind = TOP_REAL3;
       t0.tb = (int8_t)local[op.target];
       t0.code0 = (int8_t)local[rops[i + 1].target];
       t0.code1 = (int8_t)tab;
-      t1.kind = TOP_CONT;
       double m0[4], m1[4], m2[4];
       for (int e = 0; e < 4; ++e) {
         m0[e] = op.m.m[e].re;
         m1[e] = rops[i + 1].m.m[e].re;
         m2[e] = rops[i + 2].m.m[e].re;
       }
-      QL c[8];
       int flags = 0;
-      q60_triple_coef(m0, m1, m2, c, &flags);
-      Q3 P[4][3];
-      q60_triple_q3(c, P);
-      Q3* d0 = reinterpret_cast<Q3*>(t0.q);
-      Q3* d1 = reinterpret_cast<Q3*>(t1.q);
-      for (int e = 0; e < 12; ++e) (e < 8 ? d0[e] : d1[e - 8]) = P[e / 3][e % 3];
+      q60_triple_gauss_coef(m0, m1, m2, reinterpret_cast<QW*>(t0.q), &flags);
       t0.lcmask = (uint32_t)flags | ((uint32_t)local[rops[i + 2].target] << 8);
-      int_ops += N * 12.0;  // 16 real products per octet and component: 12 limb products per amplitude
-      g->nops += 2;
+      int_ops += N * 12.0;  // as four real products a complex product
+      g->nops += 1;
       i += 2;
       continue;
     }
@@ -1631,8 +1622,6 @@ static int build_tile_args(int n, int prec, const PlanPass& ps, const qs_gate* g
       t0.code0 = (int8_t)local[rops[i + 1].target];
       t0.code1 = (int8_t)tab;
       t1.kind = TOP_CONT;
-      QL* e0 = reinterpret_cast<QL*>(t0.q);
-      QL* e1 = reinterpret_cast<QL*>(t1.q);
       float* f0 = reinterpret_cast<float*>(t0.f);
       float* f1 = reinterpret_cast<float*>(t1.f);
       if (f32) {
@@ -1644,17 +1633,16 @@ static int build_tile_args(int n, int prec, const PlanPass& ps, const qs_gate* g
           }
         flops += N * 16.0;  // 4 real multiply-adds per output component, 2 components, per 4 amplitudes x 4 outputs
       } else {
-        // two complex products on the quad (q60pair.cuh): 6 limb pairs, reflection flags in lcmask
+        // two complex products on the quad (q60pair.cuh), reflection flags in lcmask
         double m0[4], m1[4];
         for (int e = 0; e < 4; ++e) {
           m0[e] = ra.m[e].re;
           m1[e] = rb.m[e].re;
         }
         int flags = 0;
-        q60_pair_coef(m0, m1, e0, &flags);
+        q60_pair_gauss_coef(m0, m1, reinterpret_cast<QP*>(t0.q), &flags);
         t0.lcmask = (uint32_t)flags;
-        (void)e1;
-        int_ops += N * 12.0;  // 8 real products per quad and component: 12 limb products per amplitude
+        int_ops += N * 12.0;  // as four real products a complex product
       }
       g->nops += 2;
       ++i;
@@ -1668,7 +1656,7 @@ static int build_tile_args(int n, int prec, const PlanPass& ps, const qs_gate* g
       to.ext_cmask = 0;
       to.code0 = to.code1 = U_GENERAL;
       if (f32) flops += N * 6.0;  // one complex product per amplitude
-      else int_ops += N * 12.0;   // one complex product (four real ones, 12 limb products) per amplitude
+      else int_ops += N * 12.0;   // one complex product (counted as four real ones) per amplitude
       ++g->nops;
       continue;
     }
@@ -1679,14 +1667,15 @@ static int build_tile_args(int n, int prec, const PlanPass& ps, const qs_gate* g
     TileOp& to = g->ops[g->nops];
     if (prec == 64)
       for (int e = 0; e < 4; ++e) to.f[e] = make_float2((float)mat.m[e].re, (float)mat.m[e].im);
-    else if (fixed && op.cls == OP_GENERAL)  // three limb products per complex product
-      for (int e = 0; e < 4; ++e) to.q[e] = qc_make_gauss(mat.m[e].re, mat.m[e].im);
+    else if (fixed && op.cls == OP_REAL)  // c + i s, or a reflection's after the flip of its bit-1 half
+      to.q[0] = qc_make_gauss(mat.m[0].re, mat.m[2].re);
     else if (fixed)
-      for (int e = 0; e < 4; ++e) to.q[e] = qc_make(mat.m[e].re, mat.m[e].im);
+      for (int e = 0; e < 4; ++e) to.q[e] = qc_make_gauss(mat.m[e].re, mat.m[e].im);
     else
       for (int e = 0; e < 4; ++e) to.m[e] = make_double2(mat.m[e].re, mat.m[e].im);
     to.code0 = (int8_t)op.code0;
     to.code1 = (int8_t)op.code1;
+    if (op.cls == OP_REAL) to.code1 = mat.m[0].re * mat.m[3].re - mat.m[1].re * mat.m[2].re < 0.0;
     uint32_t lcm = 0;
     uint64_t ext = 0;
     for (int b = 0; b < n; ++b)
@@ -1731,8 +1720,9 @@ static int build_tile_args(int n, int prec, const PlanPass& ps, const qs_gate* g
     const TileOp& o = g->ops[k];
     if (o.kind == TOP_DTABLE && (o.lcmask >= ptables.size() || o.tb != m || ptables[o.lcmask].m != m))
       rc = fail(QS_ERR_INVALID_ARG, "internal: malformed phase-table op");
-    if ((o.kind == TOP_REAL2 || o.kind == TOP_REAL3) && (k + 1 >= g->nops || g->ops[k + 1].kind != TOP_CONT ||
-                                (o.code1 >= 0 && (size_t)o.code1 >= ptables.size())))
+    if ((o.kind == TOP_REAL2 || o.kind == TOP_REAL3) && o.code1 >= 0 && (size_t)o.code1 >= ptables.size())
+      rc = fail(QS_ERR_INVALID_ARG, "internal: malformed rotation-group op");
+    if (o.kind == TOP_REAL2 && (k + 1 >= g->nops || g->ops[k + 1].kind != TOP_CONT))
       rc = fail(QS_ERR_INVALID_ARG, "internal: malformed rotation-pair op");
   }
   for (int t = 0; t < TILE_MAX_SIGNED_TABLES; ++t) g->signs[t].n = 0;

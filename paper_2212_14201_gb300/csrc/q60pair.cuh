@@ -75,21 +75,6 @@ QS_HD void q60_pair_comp(int64_t& x00, int64_t& x01, int64_t& x10, int64_t& x11,
   x11 = Vr - Ur;
 }
 
-#ifdef __CUDACC__
-template <int FL>
-__device__ __forceinline__ void q60_pair_quad_t(longlong2& q0, longlong2& q1, longlong2& q2, longlong2& q3,
-                                                const QL* __restrict__ c) {
-  int64_t r0 = q0.x, r1 = q1.x, r2 = q2.x, r3 = q3.x;
-  int64_t i0 = q0.y, i1 = q1.y, i2 = q2.y, i3 = q3.y;
-  q60_pair_comp<FL>(r0, r1, r2, r3, c);
-  q60_pair_comp<FL>(i0, i1, i2, i3, c);
-  q0 = make_longlong2(r0, i0);
-  q1 = make_longlong2(r1, i1);
-  q2 = make_longlong2(r2, i2);
-  q3 = make_longlong2(r3, i3);
-}
-
-#endif
 
 // Three real rotations on tile bits a, b, c, applied to an amplitude octet
 // (index bit(a) + 2 bit(b) + 4 bit(c)) as four complex products.
@@ -168,28 +153,6 @@ QS_HD void q60_triple_q3(const QL* c, Q3 (&P)[4][3]) {
   }
 }
 
-#ifdef __CUDACC__
-// The octet v[0..7]; P: the Q3 coefficients; flags bit k: rotation k (a, b, c) is
-// a reflection, whose sign flip of its bit-1 half comes first.
-__device__ __forceinline__ void q60_triple_octet(longlong2 (&v)[8], const Q3 (&P)[4][3], int flags) {
-  if (flags) {
-#pragma unroll
-    for (int k = 1; k < 8; ++k)
-      if (__popc(k & flags) & 1) v[k] = make_longlong2(-v[k].x, -v[k].y);
-  }
-  int64_t r[8], im[8];
-#pragma unroll
-  for (int k = 0; k < 8; ++k) {
-    r[k] = v[k].x;
-    im[k] = v[k].y;
-  }
-  q60_triple_comp(r, P);
-  q60_triple_comp(im, P);
-#pragma unroll
-  for (int k = 0; k < 8; ++k) v[k] = make_longlong2(r[k], im[k]);
-}
-#endif
-
 // Four real rotations on tile bits a, b, c, d, applied to ONE component of 16
 // amplitudes x[k] (k = bit(a) + 2 bit(b) + 4 bit(c) + 8 bit(d)) as eight complex
 // products.  The pairs along a are complex numbers z_j = x[2j] + i x[2j+1]
@@ -261,6 +224,148 @@ QS_HD void q60_quad4_comp(int64_t (&x)[16], const Q3* P0, const Q3* P1, const Q3
   }
 }
 
+// ---- the same groups with three real products a complex product ------------------------
+// y' = w y as re = c (a + b) - b (c + d), im = c (a + b) + a (d - c) (y = a + i b,
+// w = c + i d): both outputs continue the accumulator of c (a + b), so a complex
+// product takes nine wide multiply-adds instead of twelve.  The multiply-add pipe bounds
+// these kernels (four cycles a wide multiply-add; 62-76 % busy with twelve).
+//
+// Groups of three and four: 32-bit limbs with signed low limbs, v = h 2^32 + l, the
+// coefficients in units of 2^-64 (|c|, |d|, |c +- d| < 1/2), so that a product's
+// units are 2^-60 at once and its rounding takes the upper word of the middle
+// accumulator.  The dropped low x low product is at most 1/4 unit, of either sign.
+// Bounds for norm <= 1.25, in units of 2^60: the middle accumulator of an output is at
+// most 6.7 in a group of four (|w| <= 1/8, |y| <= 3.54, |a + b| <= 5.0) and 7.9 in a
+// group of three (|w| <= 1/4, |y| <= 2.5, |a + b| <= 3.54): below 2^63.
+struct QW {
+  int32_t h, l;
+};
+QS_HD QW qw_split(int64_t v) { return QW{(int32_t)(v >> 32) + (int32_t)((uint32_t)v >> 31), (int32_t)v}; }
+QS_HD void qw_add(QAcc& A, QW p, QW y) {
+  A.hi = madw(p.h, y.h, A.hi);
+  A.mid = madw(p.h, y.l, A.mid);
+  A.mid = madw(p.l, y.h, A.mid);
+}
+QS_HD int64_t qw_round(const QAcc& A) { return A.hi + (int64_t)(int32_t)(A.mid >> 32); }
+
+// (a, b) <- w (a + i b); g[0..2] = c, d - c, -(c + d).
+QS_HD void qw_cmul(const QW* g, int64_t& a, int64_t& b) {
+  const QW s = qw_split(a + b), r = qw_split(a), i = qw_split(b);
+  QAcc x{0, 1ll << 31};
+  qw_add(x, g[0], s);
+  QAcc y = x;
+  qw_add(x, g[2], i);
+  qw_add(y, g[1], r);
+  a = qw_round(x);
+  b = qw_round(y);
+}
+
+// Coefficients of w = c + i d given in units of 2^-64.
+inline void qw_coef(int64_t c, int64_t d, QW g[3]) {
+  g[0] = qw_split(c);
+  g[1] = qw_split(d - c);
+  g[2] = qw_split(-(c + d));
+}
+
+// q60_triple_comp with G[3 k ..] = qw_coef of coefficient k.
+QS_HD void q60_triple_gauss(int64_t (&x)[8], const QW* G) {
+  int64_t ur[2], ui[2], vr[2], vi[2];
+#pragma unroll
+  for (int c = 0; c < 2; ++c) {
+    const int64_t z0r = x[4 * c], z0i = x[4 * c + 1], z1r = x[4 * c + 2], z1i = x[4 * c + 3];
+    ur[c] = z0r - z1i;
+    ui[c] = z0i + z1r;
+    vr[c] = z0r + z1i;
+    vi[c] = z0i - z1r;
+  }
+  int64_t R[8] = {ur[0] - ui[1], ui[0] + ur[1], ur[0] + ui[1], ui[0] - ur[1],
+                  vr[0] - vi[1], vi[0] + vr[1], vr[0] + vi[1], vi[0] - vr[1]};
+#pragma unroll
+  for (int k = 0; k < 4; ++k) qw_cmul(G + 3 * k, R[2 * k], R[2 * k + 1]);
+  const int64_t u0r = R[0] + R[2], u0i = R[1] + R[3], u1r = R[1] - R[3], u1i = R[2] - R[0];
+  const int64_t v0r = R[4] + R[6], v0i = R[5] + R[7], v1r = R[5] - R[7], v1i = R[6] - R[4];
+  x[0] = u0r + v0r;
+  x[1] = u0i + v0i;
+  x[2] = u0i - v0i;
+  x[3] = v0r - u0r;
+  x[4] = u1r + v1r;
+  x[5] = u1i + v1i;
+  x[6] = u1i - v1i;
+  x[7] = v1r - u1r;
+}
+
+// q60_quad4_comp with the 24 coefficients (3 k + 0..2: qw_coef of channel k) in two
+// runs of 12 (two consecutive op slots).
+QS_HD void q60_quad4_gauss(int64_t (&x)[16], const QW* G0, const QW* G1) {
+  int64_t zr[8], zi[8];
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    zr[j] = x[2 * j];
+    zi[j] = x[2 * j + 1];
+  }
+#pragma unroll
+  for (int bit = 1; bit < 8; bit <<= 1)
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+      if (!(j & bit)) {
+        const int64_t lr = zr[j], li = zi[j], hr = zr[j | bit], hi = zi[j | bit];
+        zr[j] = lr - hi;  // lo + i hi
+        zi[j] = li + hr;
+        zr[j | bit] = lr + hi;  // lo - i hi
+        zi[j | bit] = li - hr;
+      }
+#pragma unroll
+  for (int k = 0; k < 8; ++k) qw_cmul(k < 4 ? G0 + 3 * k : G1 + 3 * (k - 4), zr[k], zi[k]);
+#pragma unroll
+  for (int bit = 4; bit >= 1; bit >>= 1)
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+      if (!(j & bit)) {
+        const int64_t ar = zr[j], ai = zi[j], br = zr[j | bit], bi = zi[j | bit];
+        zr[j] = ar + br;  // lo = A + B
+        zi[j] = ai + bi;
+        zr[j | bit] = ai - bi;  // hi = -i (A - B)
+        zi[j | bit] = br - ar;
+      }
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    x[2 * j] = zr[j];
+    x[2 * j + 1] = zi[j];
+  }
+}
+
+// Pairs: |w| <= 1/2 does not fit the 32-bit form.  a and b split as the amplitudes
+// (30-bit limbs, |y| <= 1.77), their sum (<= 2.5) at 31 bits with c as Q3 limbs.
+// Middle accumulator: at most 3.9 in units of 2^60.
+struct QP {
+  Q3 c;
+  QL d, n;  // d - c, -(c + d)
+  int32_t pad;
+};
+QS_HD QP qp_coef(int64_t c, int64_t d) {
+  return QP{q3_of(q60_split_coef(c)), q60_split_coef(d - c), q60_split_coef(-(c + d)), 0};
+}
+QS_HD void qp_cmul(const QP& g, int64_t& a, int64_t& b) {
+  const int64_t s = a + b;
+  QAcc x = qacc_new();
+  q3_add(x, g.c, (int32_t)(s >> 31), (int32_t)(s & 0x7FFFFFFF));
+  QAcc y = x;
+  qacc_add(x, g.n, q60_split(b));
+  qacc_add(y, g.d, q60_split(a));
+  a = qacc_round(x);
+  b = qacc_round(y);
+}
+// One component of a quad through two rotations; g[0] = P, g[1] = Q.
+QS_HD void q60_pair_gauss(int64_t& x00, int64_t& x01, int64_t& x10, int64_t& x11, const QP* g) {
+  int64_t ur = x00 - x11, ui = x01 + x10, vr = x00 + x11, vi = x01 - x10;
+  qp_cmul(g[0], ur, ui);
+  qp_cmul(g[1], vr, vi);
+  x00 = ur + vr;
+  x01 = ui + vi;
+  x10 = ui - vi;
+  x11 = vr - ur;
+}
+
 // Host: rotation angle (c, s) of a real orthogonal 2x2 (row-major) and whether it
 // is a reflection R Z.
 inline int q60_orth_angle(const double* m, double* c, double* s) {
@@ -318,6 +423,44 @@ inline void q60_quad4_coef(const double* ra, const double* rb, const double* rc,
     P[3 * k + 1] = q3_of(im);
     P[3 * k + 2] = q3_neg(P[3 * k + 1]);
   }
+}
+
+// Host: the coefficients of the three-product groups and their reflection flags.
+inline void q60_triple_gauss_coef(const double* ra, const double* rb, const double* rc, QW G[12], int* flags) {
+  double c[3], s[3];
+  const double* r[3] = {ra, rb, rc};
+  *flags = 0;
+  for (int q = 0; q < 3; ++q) *flags |= q60_orth_angle(r[q], &c[q], &s[q]) << q;
+  for (int k = 0; k < 4; ++k) {  // U+, U-, V+, V-
+    const double sb = (k & 2) ? -s[1] : s[1], sc = (k & 1) ? -s[2] : s[2];
+    const double abr = c[0] * c[1] - s[0] * sb, abi = s[0] * c[1] + c[0] * sb;
+    const double re = abr * c[2] - abi * sc, im = abi * c[2] + abr * sc;
+    qw_coef(q60_from_double(4.0 * re), q60_from_double(4.0 * im), G + 3 * k);  // w / 4 in units of 2^-64
+  }
+}
+inline void q60_quad4_gauss_coef(const double* ra, const double* rb, const double* rc, const double* rd, QW G[24],
+                                 int* flags) {
+  double c[4], s[4];
+  const double* r[4] = {ra, rb, rc, rd};
+  *flags = 0;
+  for (int q = 0; q < 4; ++q) *flags |= q60_orth_angle(r[q], &c[q], &s[q]) << q;
+  for (int k = 0; k < 8; ++k) {
+    double wr = c[0], wi = s[0];
+    for (int q = 1; q < 4; ++q) {
+      const double sq = ((k >> (q - 1)) & 1) ? -s[q] : s[q];
+      const double tr = wr * c[q] - wi * sq, ti = wi * c[q] + wr * sq;
+      wr = tr;
+      wi = ti;
+    }
+    qw_coef(q60_from_double(2.0 * wr), q60_from_double(2.0 * wi), G + 3 * k);  // w / 8 in units of 2^-64
+  }
+}
+inline void q60_pair_gauss_coef(const double* ra, const double* rb, QP g[2], int* flags) {
+  double ca, sa, cb, sb;
+  const int fa = q60_orth_angle(ra, &ca, &sa), fb = q60_orth_angle(rb, &cb, &sb);
+  *flags = fa | (fb << 1);
+  g[0] = qp_coef(q60_from_double(0.5 * (ca * cb - sa * sb)), q60_from_double(0.5 * (sa * cb + ca * sb)));
+  g[1] = qp_coef(q60_from_double(0.5 * (ca * cb + sa * sb)), q60_from_double(0.5 * (sa * cb - ca * sb)));
 }
 
 // Host: the six limb pairs and the flags of R_b (x) R_a (a, b real orthogonal

@@ -29,7 +29,7 @@ constexpr int BT_OFFS = 1 << (BT_M - 3);  // high-bit offset table: tiles hold q
 // (nothing to run on their own) and keep their generator slots.
 // BK_RPAIR: two uncontrolled real rotations on distinct tile qubits a (first member)
 // and b, run as two complex products on one component of the quads (j, j|a, j|b,
-// j|a|b) at a time (q60pair.cuh; 6 limb pairs per pair, gate = pair index); in the
+// j|a|b) at a time (q60pair.cuh; 2 coefficients per pair, gate = pair index); in the
 // backward sweep the op also takes both members' generator terms from the basis
 // that the products run in.
 // BK_PERM: a run of X and CNOT gates without a gradient, run as one permutation of
@@ -102,34 +102,25 @@ __device__ __forceinline__ int64_t bt_pair_gen(int gen, QL l0x, QL l0y, QL l1x, 
   return qaccf_result(pos) - qaccf_result(neg);
 }
 
-// The pair's two complex products on basis values u, v (see q60_pair_comp), back to
+// The pair's two complex products on basis values u, v (see q60_pair_gauss), back to
 // the quad at x[0], x[o01], x[o10], x[o11].
-__device__ __forceinline__ void bt_pair_products(const QL* c, int64_t ur, int64_t ui, int64_t vr, int64_t vi,
+__device__ __forceinline__ void bt_pair_products(const QP* g, int64_t ur, int64_t ui, int64_t vr, int64_t vi,
                                                  int64_t* x, uint32_t o01, uint32_t o10, uint32_t o11) {
-  const QL a = q60_split(ur), b = q60_split(ui), d = q60_split(vr), e = q60_split(vi);
-  QAcc A = qacc_new(), B = qacc_new(), D = qacc_new(), E = qacc_new();
-  qacc_add(A, c[0], a);
-  qacc_add(A, c[2], b);
-  qacc_add(B, c[1], a);
-  qacc_add(B, c[0], b);
-  qacc_add(D, c[3], d);
-  qacc_add(D, c[5], e);
-  qacc_add(E, c[4], d);
-  qacc_add(E, c[3], e);
-  const int64_t Ur = qacc_round(A), Ui = qacc_round(B), Vr = qacc_round(D), Vi = qacc_round(E);
-  x[0] = Ur + Vr;
-  x[o01] = Ui + Vi;
-  x[o10] = Ui - Vi;
-  x[o11] = Vr - Ur;
+  qp_cmul(g[0], ur, ui);
+  qp_cmul(g[1], vr, vi);
+  x[0] = ur + vr;
+  x[o01] = ui + vi;
+  x[o10] = ui - vi;
+  x[o11] = vr - ur;
 }
 
-// Real pair forward on one component a thread (12 wide multiply-adds a quad and
+// Real pair forward on one component a thread (18 wide multiply-adds a quad and
 // component for both rotations; as the real 4x4 matrix it took 48, as two single
 // rotations 48 and two sweeps).
 static __device__ __noinline__ void bt_rpair(longlong2* tile, uint32_t TS, uint32_t ta, uint32_t tbb,
-                                             const QL* __restrict__ cg) {
+                                             const QP* __restrict__ cg) {
   const uint32_t lo = min(ta, tbb), hi = max(ta, tbb);
-  const QL c[6] = {cg[0], cg[1], cg[2], cg[3], cg[4], cg[5]};
+  const QP c[2] = {cg[0], cg[1]};
   int64_t* comp = reinterpret_cast<int64_t*>(tile) + (threadIdx.x & 1);
   for (uint32_t i = threadIdx.x >> 1; i < (TS >> 2); i += BT_THREADS / 2) {
     uint32_t j = i + (i & ~(lo - 1));
@@ -148,11 +139,11 @@ static __device__ __noinline__ void bt_rpair(longlong2* tile, uint32_t TS, uint3
 // *out_v receive the two sums over the tile (kept to all four limb products: they are
 // summed over the state; |sum| <= 2 ||psi|| ||lambda|| <= 3.2, below 2^62).
 static __device__ __noinline__ void bt_rpair_back(longlong2* P, longlong2* Lt, uint32_t TS, uint32_t ta,
-                                                  uint32_t tbb, bool gens, const QL* __restrict__ cg, int64_t* out_u,
+                                                  uint32_t tbb, bool gens, const QP* __restrict__ cg, int64_t* out_u,
                                                   int64_t* out_v) {
   int64_t su = 0, sv = 0;
   const uint32_t lo = min(ta, tbb), hi = max(ta, tbb);
-  const QL c[6] = {cg[0], cg[1], cg[2], cg[3], cg[4], cg[5]};
+  const QP c[2] = {cg[0], cg[1]};
   const uint32_t o01 = 2 * ta, o10 = 2 * tbb, o11 = 2 * (ta | tbb);
   int64_t* cp = reinterpret_cast<int64_t*>(P) + (threadIdx.x & 1);
   int64_t* cl = reinterpret_cast<int64_t*>(Lt) + (threadIdx.x & 1);
@@ -528,12 +519,12 @@ constexpr int BT_ST_OPS = 192, BT_ST_DG = 20, BT_ST_RP = 48;
 struct BStage {
   BOp ops[BT_ST_OPS];
   QC dg[16 * BT_ST_DG];
-  QL rp[6 * BT_ST_RP];
+  QP rp[2 * BT_ST_RP];
 };
 struct BRecords {  // indexed as the global arrays
   const BOp* ops;
   const QC* dg;
-  const QL* rp;
+  const QP* rp;
 };
 template <class T>
 __device__ __forceinline__ const T* bt_stage(T* dst, const T* src, int begin, int end, int per, int cap) {
@@ -548,11 +539,11 @@ __device__ __forceinline__ const T* bt_stage(T* dst, const T* src, int begin, in
 // (A barrier must follow before the records are read, and one must precede when the
 // stage holds another pass's.)
 __device__ __forceinline__ BRecords bt_records(BStage* st, const BPass& ps, const BOp* ops, const QC* dg,
-                                               const QL* rp) {
+                                               const QP* rp) {
   BRecords r;
   r.ops = bt_stage(st->ops, ops, ps.op_begin, ps.op_end, 1, BT_ST_OPS);
   r.dg = bt_stage(st->dg, dg, ps.dg_begin, ps.dg_end, 16, BT_ST_DG);
-  r.rp = bt_stage(st->rp, rp, ps.rp_begin, ps.rp_end, 6, BT_ST_RP);
+  r.rp = bt_stage(st->rp, rp, ps.rp_begin, ps.rp_end, 2, BT_ST_RP);
   return r;
 }
 

@@ -57,18 +57,18 @@ __device__ __forceinline__ uint32_t table_sign_mask(const TileArgs& g, int t, ui
 
 // ---- FP64 engine -------------------------------------------------------------------
 // a * T (Q60), T = c + i d from a phase table entry {c.h, c.l, d.h, d.l} (16 bytes),
-// negated when neg: four limb products (direct form: fewer integer-pipe
-// instructions than the three-product Gauss form, and 16 instead of 24 bytes a
-// table entry from L2).
+// negated when neg: three products (nine wide multiply-adds; the multiply-add pipe
+// bounds the pass), the limbs of d - c, -(c + d) and of the amplitude's sum as limb
+// sums (|low limb| < 2^31; middle accumulator at most 5.5 in units of 2^60).
 __device__ __forceinline__ longlong2 table_mul(const int4 e, longlong2 a, bool neg) {
   const int32_t m = neg ? -1 : 0;
-  const QL c{(e.x ^ m) - m, (e.y ^ m) - m}, d{(e.z ^ m) - m, (e.w ^ m) - m}, nd{-d.h, -d.l};
+  const QL c{(e.x ^ m) - m, (e.y ^ m) - m}, d{(e.z ^ m) - m, (e.w ^ m) - m};
   const QL ar = q60_split(a.x), ai = q60_split(a.y);
-  QAcc re = qacc_new(), im = qacc_new();
-  qacc_add(re, c, ar);
-  qacc_add(re, nd, ai);
-  qacc_add(im, d, ar);
-  qacc_add(im, c, ai);
+  QAcc re = qacc_new();
+  qacc_add(re, c, ql_add(ar, ai));
+  QAcc im = re;
+  qacc_add(re, QL{-c.h - d.h, -c.l - d.l}, ai);
+  qacc_add(im, ql_sub(d, c), ar);
   return make_longlong2(qacc_round(re), qacc_round(im));
 }
 
@@ -129,32 +129,23 @@ struct EngQ60 {
   static __device__ __forceinline__ T mul(T a, int code, const TileOp& op, int e) {
     if (code != U_GENERAL) return unit(a, code);
     const QC& u = op.q[e];
-    const QL ar = q60_split(a.x), ai = q60_split(a.y);
-    QAcc re = qacc_new(), im = qacc_new();
-    qacc_add(re, u.re, ar);
-    qacc_add(re, u.nim, ai);
-    qacc_add(im, u.re, ai);
-    qacc_add(im, u.im, ar);
-    return make_longlong2(qacc_round(re), qacc_round(im));
+    int64_t re, im;
+    q60_gauss_mul(u, q60_split(a.x), q60_split(a.y), q60_split(a.x + a.y), &re, &im);
+    return make_longlong2(re, im);
   }
+  // x0 + i x1 of each component times c + i s (a reflection flips x1 first)
   static __device__ __forceinline__ void real2(const TileOp& op, T a0, T a1, T& b0, T& b1) {
-    const QL r0 = q60_split(a0.x), i0 = q60_split(a0.y), r1 = q60_split(a1.x), i1 = q60_split(a1.y);
-    QAcc x = qacc_new(), y = qacc_new(), z = qacc_new(), w = qacc_new();
-    qacc_add(x, op.q[0].re, r0);
-    qacc_add(x, op.q[1].re, r1);
-    qacc_add(y, op.q[0].re, i0);
-    qacc_add(y, op.q[1].re, i1);
-    qacc_add(z, op.q[2].re, r0);
-    qacc_add(z, op.q[3].re, r1);
-    qacc_add(w, op.q[2].re, i0);
-    qacc_add(w, op.q[3].re, i1);
-    b0 = make_longlong2(qacc_round(x), qacc_round(y));
-    b1 = make_longlong2(qacc_round(z), qacc_round(w));
+    if (op.code1) a1 = make_longlong2(-a1.x, -a1.y);
+    const QC& u = op.q[0];
+    int64_t x0, x1, y0, y1;
+    q60_gauss_mul(u, q60_split(a0.x), q60_split(a1.x), q60_split(a0.x + a1.x), &x0, &x1);
+    q60_gauss_mul(u, q60_split(a0.y), q60_split(a1.y), q60_split(a0.y + a1.y), &y0, &y1);
+    b0 = make_longlong2(x0, y0);
+    b1 = make_longlong2(x1, y1);
   }
   static __device__ __forceinline__ void general2(const TileOp& op, T a0, T a1, T& b0, T& b1) {
     const QL r0 = q60_split(a0.x), i0 = q60_split(a0.y), r1 = q60_split(a1.x), i1 = q60_split(a1.y);
-    // Gauss form: K1 = sum c (a + b), K2 = sum a (d - c), K3 = sum b (c + d);
-    // re = K1 - K3, im = K1 + K2 (three limb products per complex product)
+    // Gauss form: three limb products per complex product
     const QL s0 = q60_split(a0.x + a0.y), s1 = q60_split(a1.x + a1.y);
     int64_t re, im;
     q60_gauss_row(op.q[0], op.q[1], r0, i0, s0, r1, i1, s1, &re, &im);
@@ -269,13 +260,13 @@ __device__ __forceinline__ void pair_loop(typename E::T* tile, uint32_t cnt, uin
 }
 
 // Two real rotations on tile bits a and b on the quads (j, j|a, j|b, j|a|b), as
-// two complex products per quad and component (q60pair.cuh): 48 wide
+// two complex products per quad and component (q60pair.cuh): 36 wide
 // multiply-adds per quad where the 4x4 matrix takes 96.  With a phase table
 // (tab != nullptr, the table op just before the pair): every amplitude of the
 // quad is first multiplied by its table entry, which saves the table op's own
 // shared-memory round trip, index arithmetic and barrier.
 template <int THREADS>
-__device__ __forceinline__ void quad_real(longlong2* tile, uint32_t TS, uint32_t ta, uint32_t tbb, const QL* m0,
+__device__ __forceinline__ void quad_real(longlong2* tile, uint32_t TS, uint32_t ta, uint32_t tbb, const QP* m0,
                                           int flags, const int4* tab, uint32_t S) {
   const uint32_t lo = min(ta, tbb), hi = max(ta, tbb);
   const uint32_t pa = tsw(ta), pb = tsw(tbb);
@@ -303,7 +294,16 @@ __device__ __forceinline__ void quad_real(longlong2* tile, uint32_t TS, uint32_t
       for (int c = 1; c < 4; ++c)
         if (__popc(c & flags) & 1) v[c] = make_longlong2(-v[c].x, -v[c].y);
     }
-    q60_pair_quad_t<0>(v[0], v[1], v[2], v[3], m0);
+    int64_t r[4], im[4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      r[c] = v[c].x;
+      im[c] = v[c].y;
+    }
+    q60_pair_gauss(r[0], r[1], r[2], r[3], m0);
+    q60_pair_gauss(im[0], im[1], im[2], im[3], m0);
+#pragma unroll
+    for (int c = 0; c < 4; ++c) v[c] = make_longlong2(r[c], im[c]);
 #pragma unroll
     for (int c = 0; c < 4; ++c) tile[pp[c]] = v[c];
   }
@@ -315,7 +315,7 @@ __device__ __forceinline__ void quad_real(longlong2* tile, uint32_t TS, uint32_t
 // single rotation take 24.  With a phase table, as in quad_real.
 template <int THREADS>
 __device__ __forceinline__ void octet_real(longlong2* tile, uint32_t TS, uint32_t ta, uint32_t tb, uint32_t tc,
-                                           const Q3 (&P)[4][3], int flags, const int4* tab, uint32_t S) {
+                                           const QW* G, int flags, const int4* tab, uint32_t S) {
   const uint32_t p0 = min(ta, min(tb, tc)), p2 = max(ta, max(tb, tc));
   const uint32_t p1 = (ta | tb | tc) & ~(p0 | p2);
   const uint32_t pa = tsw(ta), pb = tsw(tb), pc = tsw(tc);
@@ -340,7 +340,21 @@ __device__ __forceinline__ void octet_real(longlong2* tile, uint32_t TS, uint32_
       v[k] = tile[pp[k]];
       if (tab) v[k] = table_mul(__ldg(tab + jj[k]), v[k], __popc(jj[k] & S) & 1);
     }
-    q60_triple_octet(v, P, flags);
+    if (flags) {  // reflections: the sign flip of their bit-1 half first
+#pragma unroll
+      for (int k = 1; k < 8; ++k)
+        if (__popc(k & flags) & 1) v[k] = make_longlong2(-v[k].x, -v[k].y);
+    }
+    int64_t r[8], im[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      r[k] = v[k].x;
+      im[k] = v[k].y;
+    }
+    q60_triple_gauss(r, G);
+    q60_triple_gauss(im, G);
+#pragma unroll
+    for (int k = 0; k < 8; ++k) v[k] = make_longlong2(r[k], im[k]);
 #pragma unroll
     for (int k = 0; k < 8; ++k) tile[pp[k]] = v[k];
   }
@@ -351,7 +365,7 @@ __device__ __forceinline__ void octet_real(longlong2* tile, uint32_t TS, uint32_
 // two lanes of a pair read the two halves of the same 16-byte amplitudes.
 template <int THREADS>
 __device__ __forceinline__ void quad4_real(longlong2* tile, uint32_t TS, uint32_t ta, uint32_t tb, uint32_t tc,
-                                           uint32_t td, const Q3* P0, const Q3* P1, const Q3* P2, int flags) {
+                                           uint32_t td, const QW* G0, const QW* G1, int flags) {
   const uint32_t all = ta | tb | tc | td;
   uint32_t p[4], rest = all;
 #pragma unroll
@@ -387,7 +401,7 @@ __device__ __forceinline__ void quad4_real(longlong2* tile, uint32_t TS, uint32_
       for (int k = 1; k < 16; ++k)
         if (__popc(k & flags) & 1) x[k] = -x[k];
     }
-    q60_quad4_comp(x, P0, P1, P2);
+    q60_quad4_gauss(x, G0, G1);
 #pragma unroll
     for (int k = 0; k < 16; ++k) comp[2 * pp[k]] = x[k];
   }
@@ -700,40 +714,33 @@ __global__ void __launch_bounds__(THREADS, THREADS == 256 ? E::kMinBlocks : 1) k
           continue;
         }
         if (op.kind == TOP_REAL4) {
-          // 24 Q3 coefficients: 8 in q[] of this slot and of each of the next two
+          // 24 coefficients: 12 in q[] of this slot and 12 in the next slot's
           quad4_real<THREADS>(tile, TS, 1u << op.tb, 1u << op.code0, 1u << ((op.lcmask >> 8) & 31),
-                              1u << ((op.lcmask >> 16) & 31), reinterpret_cast<const Q3*>(op.q),
-                              reinterpret_cast<const Q3*>(g.ops[k + 1].q), reinterpret_cast<const Q3*>(g.ops[k + 2].q),
-                              (int)(op.lcmask & 15));
-          k += 2;  // the continuation slots
+                              1u << ((op.lcmask >> 16) & 31), reinterpret_cast<const QW*>(op.q),
+                              reinterpret_cast<const QW*>(g.ops[k + 1].q), (int)(op.lcmask & 15));
+          ++k;  // the continuation slot
           __syncthreads();
           continue;
         }
         if (op.kind == TOP_REAL3) {
           const int4* tab = op.code1 >= 0 ? reinterpret_cast<const int4*>(g.tables) + (size_t)op.code1 * TS : nullptr;
-          // 12 Q3 coefficients: 8 in this slot's q[] (96 bytes), 4 in the next slot's
-          const Q3* pq0 = reinterpret_cast<const Q3*>(op.q);
-          const Q3* pq1 = reinterpret_cast<const Q3*>(g.ops[k + 1].q);
-          Q3 P[4][3];
-#pragma unroll
-          for (int e = 0; e < 12; ++e) P[e / 3][e % 3] = e < 8 ? pq0[e] : pq1[e - 8];
+          const QW* G = reinterpret_cast<const QW*>(op.q);  // 12 coefficients
           if (tab)
-            octet_real<THREADS>(tile, TS, 1u << op.tb, 1u << op.code0, 1u << (op.lcmask >> 8), P,
+            octet_real<THREADS>(tile, TS, 1u << op.tb, 1u << op.code0, 1u << (op.lcmask >> 8), G,
                                 (int)(op.lcmask & 7), tab, table_sign_mask(g, op.code1, base));
           else
-            octet_real<THREADS>(tile, TS, 1u << op.tb, 1u << op.code0, 1u << (op.lcmask >> 8), P,
+            octet_real<THREADS>(tile, TS, 1u << op.tb, 1u << op.code0, 1u << (op.lcmask >> 8), G,
                                 (int)(op.lcmask & 7), nullptr, 0u);
-          ++k;  // the continuation slot
           __syncthreads();
           continue;
         }
         if (op.kind == TOP_REAL2) {
           const int4* tab = op.code1 >= 0 ? reinterpret_cast<const int4*>(g.tables) + (size_t)op.code1 * TS : nullptr;
           if (tab)
-            quad_real<THREADS>(tile, TS, 1u << op.tb, 1u << op.code0, reinterpret_cast<const QL*>(op.q),
+            quad_real<THREADS>(tile, TS, 1u << op.tb, 1u << op.code0, reinterpret_cast<const QP*>(op.q),
                                (int)op.lcmask, tab, table_sign_mask(g, op.code1, base));
           else
-            quad_real<THREADS>(tile, TS, 1u << op.tb, 1u << op.code0, reinterpret_cast<const QL*>(op.q),
+            quad_real<THREADS>(tile, TS, 1u << op.tb, 1u << op.code0, reinterpret_cast<const QP*>(op.q),
                                (int)op.lcmask, nullptr, 0u);
           ++k;  // the continuation slot
           __syncthreads();

@@ -33,19 +33,18 @@ enum TileOpKind : int8_t {
                    // (table index in lcmask; TileArgs::tables)
   TOP_REAL2 = 11,  // two real rotations on tile bits tb and code0 on amplitude quads (quad
                    // index 2*bit(code0) + bit(tb)): Q60, two complex products (q60pair.cuh,
-                   // 6 limb pairs in q[], reflection flags in lcmask); FP32, the real 4x4
+                   // their coefficients in q[], reflection flags in lcmask); FP32, the real 4x4
                    // (16 floats in f[] of this slot and the next); code1 >= 0: phase
                    // table code1 applied first (the op before the pair)
   TOP_CONT = 12,   // continuation slot of the op before it (never run on its own)
   TOP_REAL3 = 13,  // Q60 only: three real rotations on tile bits tb, code0 and lcmask >> 8 on
                    // amplitude octets (index bit(tb) + 2 bit(code0) + 4 bit(lcmask >> 8)) as
-                   // four complex products (q60pair.cuh); the 12 Q3 coefficients (4 x re, im,
-                   // -im): 8 in q[] of this slot, 4 in the next; reflection flags in
-                   // lcmask & 7; code1 >= 0: phase table code1 applied first
+                   // four complex products (q60pair.cuh); their 12 coefficients fill q[];
+                   // reflection flags in lcmask & 7; code1 >= 0: phase table code1 applied first
   TOP_REAL4 = 14,  // four real rotations on tile bits tb, code0, (lcmask >> 8) & 31 and
                    // (lcmask >> 16) & 31.  Q60: one amplitude component of 16 at a time, as
-                   // eight complex products (q60_quad4_comp); the 24 Q3 coefficients fill q[]
-                   // of this slot and the next two; reflection flags in lcmask & 15.  FP32:
+                   // eight complex products (q60_quad4_gauss); the 24 coefficients fill q[] of
+                   // this slot and the next; reflection flags in lcmask & 15.  FP32:
                    // 16 amplitudes in registers, the four row-major matrices as 16 floats in
                    // q[] of this one slot; code1 >= 0: phase table code1 applied first
 };
@@ -53,7 +52,8 @@ enum TileOpKind : int8_t {
 struct TileOp {
   union {
     double2 m[4];      // FP64 engine: matrix (for SCALAR: m[0] = d0, m[3] = d1)
-    QC q[4];           // Q60 engine: the same entries as limbs (GENERAL ops: Gauss form)
+    QC q[4];           // Q60 engine: the same entries as limbs in Gauss form (REAL ops: q[0] = c + i s
+                       // of the rotation, code1 = 1 for a reflection)
     float2 f[4];       // FP32 engine (complex64 states): the entries rounded to float
   };
   uint64_t ext_cmask;  // control qubits outside the tile (global bit positions)
