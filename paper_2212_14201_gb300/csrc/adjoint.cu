@@ -297,6 +297,7 @@ __global__ void __launch_bounds__(BT_THREADS, 3) k_adj_pass(longlong2* __restric
     __syncthreads();
     bt_load(tP, psi, base, offs, L, TS);
     bt_load(tL, lam, base, offs, L, TS);
+    bt_load_wait();
     __syncthreads();
     for (int k = ps.op_begin; k < ps.op_end; ++k) {
       const BOp& op = a.ops[k];

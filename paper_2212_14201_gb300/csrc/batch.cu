@@ -170,6 +170,7 @@ __device__ void bt_run_pass(const BatchArgs& d, const BPass& ps, longlong2* psi,
     __syncthreads();
     bt_load(tP, psi, base, offs, L, TS);
     if (backward) bt_load(tL, lam, base, offs, L, TS);
+    bt_load_wait();
     __syncthreads();
     if (!backward) {
       for (int k = ps.op_begin; k < ps.op_end; ++k) {

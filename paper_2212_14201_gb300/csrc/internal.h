@@ -70,6 +70,17 @@ __device__ __forceinline__ double2 ld_amp(const float2* a, uint64_t i) {
   const float2 v = a[i];
   return make_double2((double)v.x, (double)v.y);
 }
+// 16-byte copies from global to shared memory that take no register and do not wait;
+// cp_async_wait_all waits for this thread's.
+#ifdef __CUDACC__
+__device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
+  const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(sa), "l"(gmem) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait_all() {
+  asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
+}
+#endif
 inline size_t amp_bytes(const qs_state* s) { return s->prec == 64 ? sizeof(float2) : sizeof(double2); }
 // Calls f with the state's amplitude pointer typed by its precision.
 template <class F>

@@ -547,13 +547,15 @@ __device__ __forceinline__ BRecords bt_records(BStage* st, const BPass& ps, cons
   return r;
 }
 
-// Tile loads and stores.  (Eight loads in flight per thread were slower: their
-// registers spill.)
+// Tile loads and stores.  Loads are asynchronous copies (the tiles hold the same Q60
+// integers as memory): all of a thread's are in flight at once and take no registers;
+// bt_load_wait comes before the barrier.
 __device__ __forceinline__ void bt_load(longlong2* tile, const longlong2* src, uint64_t base, const uint64_t* offs,
                                         int L, uint32_t TS) {
   const uint32_t lowmask = (1u << L) - 1;
-  for (uint32_t j = threadIdx.x; j < TS; j += BT_THREADS) tile[j] = src[base + offs[j >> L] + (j & lowmask)];
+  for (uint32_t j = threadIdx.x; j < TS; j += BT_THREADS) cp_async16(tile + j, src + base + offs[j >> L] + (j & lowmask));
 }
+__device__ __forceinline__ void bt_load_wait() { cp_async_wait_all(); }
 __device__ __forceinline__ void bt_store(const longlong2* tile, longlong2* dst, uint64_t base, const uint64_t* offs,
                                          int L, uint32_t TS) {
   constexpr int E = (1 << BT_M) / BT_THREADS;

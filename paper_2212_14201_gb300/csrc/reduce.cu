@@ -575,18 +575,10 @@ __device__ __forceinline__ uint64_t insert0(uint64_t c, int b) {
   return ((c >> b) << (b + 1)) | (c & ((1ull << b) - 1));
 }
 
-__device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
-  const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(sa), "l"(gmem) : "memory");
-}
 __device__ __forceinline__ void cp_async8(void* smem, const void* gmem) {
   const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
   asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(sa), "l"(gmem) : "memory");
 }
-__device__ __forceinline__ void cp_async_wait_all() {
-  asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
-}
-
 __device__ __forceinline__ Sp sp_h(int4 u) { return {u.x, u.y}; }
 // acc += v when bit 0 of c is clear: a predicated 128-bit add (carry chain)
 __device__ __forceinline__ void add128_if_even(u128& acc, u128 v, uint32_t c) {

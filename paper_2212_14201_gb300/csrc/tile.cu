@@ -652,9 +652,11 @@ __global__ void __launch_bounds__(THREADS, THREADS == 256 ? E::kMinBlocks : 1) k
                                    [](const longlong2& v) { return v; }, tab, Sg);
         else
           load_tile_table<THREADS>(tile, a, base, offs, L, lowmask, TS, tsq, conv, tab, Sg);
-      } else if (g.io & 1) {
-        load_tile<THREADS>(tile, reinterpret_cast<const longlong2*>(a), base, offs, L, lowmask, TS, tsq,
-                           [](const longlong2& v) { return v; });
+      } else if (g.io & 1) {  // Q60 in memory as in the tile: asynchronous copies
+        const longlong2* src = reinterpret_cast<const longlong2*>(a);
+        for (uint32_t j = threadIdx.x; j < TS; j += THREADS)
+          cp_async16(tile + (j ^ tsq), src + base + offs[j >> L] + (j & lowmask));
+        cp_async_wait_all();
       } else {
         load_tile<THREADS>(tile, a, base, offs, L, lowmask, TS, tsq, conv);
       }
