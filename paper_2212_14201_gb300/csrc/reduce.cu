@@ -887,17 +887,23 @@ __global__ void __launch_bounds__(256, 2) k_pauli_z(const A* __restrict__ a, con
   }
 }
 
-// sums[2 k] = the CTA partials of one slot added (modulo 2^128), CTA k of this kernel
-// for the slot at slot[k] of a CTA's `stride` partials.
+// sums[2 k] = the CTA partials of slot k added (modulo 2^128), CTA k of this kernel: all
+// slots of up to PF_MAX in one launch (one per pass was a third of a small state's time).
+constexpr int PF_MAX = 256;
 struct PFinish {
-  int8_t slot[PZ_MAX];
+  struct Slot {
+    uint32_t off;       // its first partial, in words of the partials' area
+    uint16_t nblocks;   // CTAs
+    uint16_t stride;    // slots per CTA
+  } s[PF_MAX];
 };
-__global__ void __launch_bounds__(256) k_pauli_exact_finish(const uint64_t* __restrict__ part, int nblocks, int stride,
-                                                            const PFinish f, uint64_t* __restrict__ sums) {
+__global__ void __launch_bounds__(256) k_pauli_exact_finish(const uint64_t* __restrict__ part,
+                                                            const __grid_constant__ PFinish f,
+                                                            uint64_t* __restrict__ sums) {
   __shared__ uint64_t sh[8][2];
-  const int k = f.slot[blockIdx.x];
+  const PFinish::Slot q = f.s[blockIdx.x];
   u128 t = 0;
-  for (int b = threadIdx.x; b < nblocks; b += 256) t += ld_u128(part + ((size_t)b * stride + k) * 2);
+  for (int b = threadIdx.x; b < q.nblocks; b += 256) t += ld_u128(part + q.off + (size_t)b * q.stride * 2);
   t = block_sum_u128(t, sh);
   if (threadIdx.x == 0) {
     sums[2 * blockIdx.x] = (uint64_t)t;
@@ -1197,10 +1203,13 @@ static int pauli_exact(qs_state* s, const qs_pauli* terms, size_t nterms, double
     const size_t nslots = slots.size();
     std::vector<int> gidx(nslots, -1);
     uint64_t* part = (uint64_t*)s->ws;
-    const size_t part_words = (size_t)1216 * PZ_MAX * 2;
-    uint64_t* sums = part + part_words;
-    if ((part_words + 2 * nslots) * sizeof(uint64_t) > s->ws_bytes)
+    // the workspace: slot sums, then the partials of the passes since the last finish
+    uint64_t* sums = part;
+    part += 2 * nslots;
+    const size_t pass_words = (size_t)1216 * PZ_MAX * 2;  // more than any pass writes
+    if ((pass_words + 2 * nslots) * sizeof(uint64_t) > s->ws_bytes)
       return fail(QS_ERR_UNSUPPORTED, "Pauli slot sums exceed the workspace");
+    const size_t part_words = std::min<size_t>(s->ws_bytes / sizeof(uint64_t) - 2 * nslots, 0xFFFFFFFFu);
     static std::once_flag smem_once;
     std::call_once(smem_once, [] {
       cudaFuncSetAttribute(k_pauli_tile<double2>, cudaFuncAttributeMaxDynamicSharedMemorySize, 16 << PT_TMAX);
@@ -1208,46 +1217,58 @@ static int pauli_exact(qs_state* s, const qs_pauli* terms, size_t nterms, double
       cudaFuncSetAttribute(k_pauli_x<double2>, cudaFuncAttributeMaxDynamicSharedMemorySize, 16 << PT_TMAX);
       cudaFuncSetAttribute(k_pauli_x<float2>, cudaFuncAttributeMaxDynamicSharedMemorySize, 16 << PT_TMAX);
     });
-    int next = 0;
-    // adds the partials of `count` slots (at f.slot[] of a CTA's) into sums[next ..]
-    auto finish = [&](int nblocks, int stride, const PFinish& f, int count) {
-      k_pauli_exact_finish<<<count, 256, 0, s->stream>>>(part, nblocks, stride, f, sums + 2 * (size_t)next);
-      next += count;
+    int next = 0, done = 0;  // slots launched, and finished
+    size_t used = 0;         // words of partials since the last finish
+    PFinish f;
+    auto finish = [&] {
+      if (next == done) return (int)QS_OK;
+      note_launch(1);
+      k_pauli_exact_finish<<<next - done, 256, 0, s->stream>>>(part, f, sums + 2 * (size_t)done);
+      done = next;
+      used = 0;
       return launch_check("pauli_exact_finish");
     };
-    // From 16 qubits on, field slots and |a|^2 slots have kernels of their own (below
-    // that, a state has too few tiles to fill the GPU with them).
-    const bool own = n >= 16;
+    // room for a pass of up to PZ_MAX slots
+    auto room = [&] {
+      return next - done + PZ_MAX > PF_MAX || used + pass_words > part_words ? finish() : (int)QS_OK;
+    };
+    // records slot `at` of a pass whose CTAs write `stride` slots from the current place
+    auto record = [&](int k, int at, int nblocks, int stride) {
+      f.s[next - done] = {(uint32_t)(used + 2 * (size_t)at), (uint16_t)nblocks, (uint16_t)stride};
+      gidx[k] = next++;
+    };
+    // Field slots and |a|^2 slots have kernels of their own wherever a tile of 12
+    // coordinates exists (13-site chain 92 -> 54 us, 25 sites 2.9 -> 1.4 ms).
+    const bool own = n >= 12;
     if (own) {
       std::vector<int> zs;
       for (const auto& P : passes)
         for (int k : P.sl)
           if (!slots[k].xm) zs.push_back(k);
       for (size_t z0 = 0; z0 < zs.size(); z0 += PZ_MAX) {
+        QS_TRY(room());
         PZArgs g{};
-        PFinish f{};
         g.ntiles = 1ull << (n - 11);
         g.nt = (int)std::min<size_t>(PZ_MAX, zs.size() - z0);
+        const int nblocks = (int)std::min<uint64_t>(2 * 152, g.ntiles);
         for (int k = 0; k < g.nt; ++k) {
           g.zm[k] = slots[zs[z0 + k]].zm;
-          gidx[zs[z0 + k]] = next + k;
-          f.slot[k] = (int8_t)k;
+          record(zs[z0 + k], k, nblocks, PZ_MAX);
         }
-        const int nblocks = (int)std::min<uint64_t>(2 * 152, g.ntiles);
         KTimer kt(s, QS_K_REDUCE, n, g.nt, 0, 0, (double)(1ull << n), 8.0 * g.nt * (double)(1ull << n));
-        note_launch(2);
+        note_launch(1);
         with_amps(s, [&](auto* a) {
           using T = std::remove_cv_t<std::remove_pointer_t<decltype(a)>>;
-          k_pauli_z<T><<<nblocks, 256, 0, s->stream>>>(a, g, part);
+          k_pauli_z<T><<<nblocks, 256, 0, s->stream>>>(a, g, part + used);
           return QS_OK;
         });
         QS_TRY(launch_check("pauli_z"));
-        QS_TRY(finish(nblocks, PZ_MAX, f, g.nt));
+        used += (size_t)nblocks * PZ_MAX * 2;
       }
     }
     for (const auto& P : passes) {
+      QS_TRY(room());
       PXArgs gx{};
-      PFinish fx{};
       int nx = 0;
       PTile g{};
       g.T = (int)P.bm.size();
@@ -1256,7 +1277,7 @@ static int pauli_exact(qs_state* s, const qs_pauli* terms, size_t nterms, double
         g.bm[q] = gx.bm[q] = P.bm[q];
         g.lead[q] = gx.lead[q] = pp_lead(P.bm[q]);
       }
-      PFinish f{};
+      const int xblocks = (int)std::min<uint64_t>(2 * 152, gx.ntiles);
       std::vector<int> left;  // slots for k_pauli_tile
       for (int k : P.sl) {
         const PauliSlot& sl = slots[k];
@@ -1264,31 +1285,31 @@ static int pauli_exact(qs_state* s, const qs_pauli* terms, size_t nterms, double
         uint32_t xc = 0;
         if (sl.xm) pp_reduce(P.bm, sl.xm, &xc);
         if (own && !sl.zm && !sl.im && (xc & (xc - 1)) == 0) {
-          gidx[k] = next + nx;
-          fx.slot[nx++] = (int8_t)(31 - __builtin_clz(xc));
+          record(k, 31 - __builtin_clz(xc), xblocks, PT_TMAX);
+          ++nx;
           gx.want |= xc;
         } else {
           left.push_back(k);
         }
       }
       if (nx) {
-        const int nblocks = (int)std::min<uint64_t>(2 * 152, gx.ntiles);
         KTimer kt(s, QS_K_REDUCE, n, nx, 0, 0, (double)(1ull << n), 8.0 * nx * (double)(1ull << n));
-        note_launch(2);
+        note_launch(1);
         with_amps(s, [&](auto* a) {
           using T = std::remove_cv_t<std::remove_pointer_t<decltype(a)>>;
-          k_pauli_x<T><<<nblocks, 256, (size_t)16 << PT_TMAX, s->stream>>>(a, gx, part);
+          k_pauli_x<T><<<xblocks, 256, (size_t)16 << PT_TMAX, s->stream>>>(a, gx, part + used);
           return QS_OK;
         });
         QS_TRY(launch_check("pauli_x"));
-        QS_TRY(finish(nblocks, PT_TMAX, fx, nx));
+        used += (size_t)xblocks * PT_TMAX * 2;
       }
       if (left.empty()) continue;
+      QS_TRY(room());
       g.nt = (int)left.size();
+      const int nblocks = (int)std::min<uint64_t>(3 * 152, g.ntiles);  // three CTAs per SM
       for (int q = 0; q < g.nt; ++q) {
         const PauliSlot& sl = slots[left[q]];
-        gidx[left[q]] = next + q;
-        f.slot[q] = (int8_t)q;
+        record(left[q], q, nblocks, PS_MAX);
         g.zm[q] = sl.zm;
         g.im[q] = (uint8_t)sl.im;
         uint32_t zc = 0;
@@ -1305,17 +1326,17 @@ static int pauli_exact(qs_state* s, const qs_pauli* terms, size_t nterms, double
           g.top[q] = 31 - __builtin_clz(xc);
         }
       }
-      const int nblocks = (int)std::min<uint64_t>(3 * 152, g.ntiles);  // three CTAs per SM
       KTimer kt(s, QS_K_REDUCE, n, g.nt, 0, 0, (double)(1ull << n), 8.0 * g.nt * (double)(1ull << n));
-      note_launch(2);
+      note_launch(1);
       with_amps(s, [&](auto* a) {
         using T = std::remove_cv_t<std::remove_pointer_t<decltype(a)>>;
-        k_pauli_tile<T><<<nblocks, 256, (size_t)16 << g.T, s->stream>>>(a, g, part);
+        k_pauli_tile<T><<<nblocks, 256, (size_t)16 << g.T, s->stream>>>(a, g, part + used);
         return QS_OK;
       });
       QS_TRY(launch_check("pauli_tile"));
-      QS_TRY(finish(nblocks, PS_MAX, f, g.nt));
+      used += (size_t)nblocks * PS_MAX * 2;
     }
+    QS_TRY(finish());
     std::vector<uint64_t> hs(2 * nslots);
     if (nslots) QS_TRY(read_back(s, (const double*)sums, 2 * nslots, (double*)hs.data()));
     auto sum_of = [&](int k) {
