@@ -29,9 +29,23 @@ namespace qs {
 // 3..5 allows; 18 of the 299 such bit sets keep a 2-way conflict).
 __device__ __forceinline__ uint32_t tsw_bits(uint32_t j) { return (0x3958f8u >> (3u * ((j >> 3) & 7u))) & 7u; }
 __device__ __forceinline__ uint32_t tsw(uint32_t j) { return j ^ tsw_bits(j); }
-// In a loop over i = threadIdx.x + k * THREADS (THREADS >= 64) whose element index
-// j inserts zero bits into i, bits 3..5 of j come from the low bits of i, i.e. from
+// In a loop over i = threadIdx.x + k * THREADS (THREADS >= 256) whose element index
+// j inserts zero bits into i, bits 3..7 of j come from the low bits of i, i.e. from
 // threadIdx.x alone: the swizzle is one XOR with a per-thread constant.
+// Elements of 8 bytes (complex64) have 16 to a row of banks: their swizzle folds bits
+// 4..7 into bits 0..3 with the vectors 5, 10, 3, 8, so that the groups of four bits
+// that runs of rotations are cut into ({0,3,6,9}, {1,4,7,10}, {2,5,8,11}), any three
+// or all of the low bits and most pairs keep the 16 lanes of a half-warp apart (with
+// the map above every one of those groups had a two-way conflict).
+template <int BYTES>
+__device__ __forceinline__ uint32_t tsw_bits_of(uint32_t j) {
+  if (BYTES == 8) return (uint32_t)(0x41EB72D8C963FA50ull >> (4u * ((j >> 4) & 15u))) & 15u;
+  return tsw_bits(j);
+}
+template <int BYTES>
+__device__ __forceinline__ uint32_t tsw_of(uint32_t j) {
+  return j ^ tsw_bits_of<BYTES>(j);
+}
 
 // Insert zero bits at the set positions of `fixed` (ascending), then OR `set`.
 __device__ __forceinline__ uint32_t tile_expand(uint32_t i, uint32_t fixed, uint32_t set) {
@@ -235,8 +249,9 @@ template <class E, int KIND, int THREADS>
 __device__ __forceinline__ void pair_loop(typename E::T* tile, uint32_t cnt, uint32_t fixed, uint32_t lcm, uint32_t tb,
                                           const TileOp& op) {
   using T = typename E::T;
-  const uint32_t tbp = tsw(tb);
-  const uint32_t csw = tsw_bits(lcm ? tile_expand(threadIdx.x, fixed, lcm) : threadIdx.x + (threadIdx.x & ~(tb - 1)));
+  constexpr int B = sizeof(T);
+  const uint32_t tbp = tsw_of<B>(tb);
+  const uint32_t csw = tsw_bits_of<B>(lcm ? tile_expand(threadIdx.x, fixed, lcm) : threadIdx.x + (threadIdx.x & ~(tb - 1)));
 #pragma unroll 2
   for (uint32_t i = threadIdx.x; i < cnt; i += THREADS) {
     // without in-tile controls the insertion of one zero bit is a mask and an add
@@ -414,11 +429,11 @@ template <int THREADS>
 __device__ __forceinline__ void quad_real_f32(float2* tile, uint32_t TS, uint32_t ta, uint32_t tbb, const float* m0,
                                               const float* m1, const float2* tab, uint32_t S) {
   const uint32_t lo = min(ta, tbb), hi = max(ta, tbb);
-  const uint32_t pa = tsw(ta), pb = tsw(tbb);
+  const uint32_t pa = tsw_of<8>(ta), pb = tsw_of<8>(tbb);
   uint32_t csw;
   {
     uint32_t j = threadIdx.x + (threadIdx.x & ~(lo - 1));
-    csw = tsw_bits(j + (j & ~(hi - 1)));
+    csw = tsw_bits_of<8>(j + (j & ~(hi - 1)));
   }
   const uint32_t cnt = TS >> 2;
 #pragma unroll 2
@@ -471,13 +486,13 @@ __device__ __forceinline__ void quad4_f32(float2* tile, uint32_t TS, uint32_t ta
     p[e] = rest & (0u - rest);
     rest ^= p[e];
   }
-  const uint32_t pa = tsw(ta), pb = tsw(tb), pc = tsw(tc), pd = tsw(td);
+  const uint32_t pa = tsw_of<8>(ta), pb = tsw_of<8>(tb), pc = tsw_of<8>(tc), pd = tsw_of<8>(td);
   uint32_t csw;
   {
     uint32_t j = threadIdx.x;
 #pragma unroll
     for (int e = 0; e < 4; ++e) j = j + (j & ~(p[e] - 1));
-    csw = tsw_bits(j);
+    csw = tsw_bits_of<8>(j);
   }
   const uint32_t cnt = TS >> 4;
   for (uint32_t g = threadIdx.x; g < cnt; g += THREADS) {
@@ -636,7 +651,7 @@ __global__ void __launch_bounds__(THREADS, THREADS == 256 ? E::kMinBlocks : 1) k
     offs[h] = o;
   }
   const uint32_t lowmask = (1u << L) - 1;
-  const uint32_t tsq = tsw_bits(threadIdx.x);  // swizzle of the sequential loops over j
+  const uint32_t tsq = tsw_bits_of<sizeof(T)>(threadIdx.x);  // swizzle of the sequential loops over j
   for (uint64_t r = blockIdx.x; r < g.ntiles; r += gridDim.x) {
     uint64_t base = 0;
     for (int b = 0; b < g.nout; ++b) base |= ((r >> b) & 1ull) << g.outpos[b];
@@ -756,7 +771,7 @@ __global__ void __launch_bounds__(THREADS, THREADS == 256 ? E::kMinBlocks : 1) k
         const int e = one ? 3 : 0;
         const uint32_t cnt = TS >> __popc(lcm);
         for (uint32_t i = threadIdx.x; i < cnt; i += THREADS) {
-          const uint32_t j = tsw(tile_expand(i, lcm, lcm));
+          const uint32_t j = tsw_of<sizeof(T)>(tile_expand(i, lcm, lcm));
           tile[j] = E::mul(tile[j], code, op, e);
         }
       } else {
@@ -765,7 +780,7 @@ __global__ void __launch_bounds__(THREADS, THREADS == 256 ? E::kMinBlocks : 1) k
         const uint32_t cnt = TS >> __popc(fixed);
         if (op.kind == TOP_PHASE1) {
           for (uint32_t i = threadIdx.x; i < cnt; i += THREADS) {
-            const uint32_t j = tsw(tile_expand(i, fixed, lcm) | tb);
+            const uint32_t j = tsw_of<sizeof(T)>(tile_expand(i, fixed, lcm) | tb);
             tile[j] = E::mul(tile[j], op.code1, op, 3);
           }
         } else if (op.kind == TOP_GENERAL) {
