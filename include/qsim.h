@@ -677,7 +677,7 @@ int qs_batch_info(const qs_batch* b, int* grid, int* threads, size_t* smem_bytes
 int qs_batch_cluster(const qs_batch* b, int* ctas);
 
 /* Cluster size of batches created after the call: 1, 2, 4 or 8 CTAs, or 0
- * (default) to choose per batch the size whose longest-processing-time schedule
+ * (default) to choose per batch the size (up to 16) whose longest-processing-time schedule
  * of the work items over the resident clusters has the shortest estimated
  * makespan (set cost ~ 2^n x gates).  Not thread-safe against a concurrent
  * qs_batch_create.  Errors: INVALID_ARG. */

@@ -4,7 +4,7 @@
 // quantum-classical algorithm" and "Variational quantum circuit"; the batching
 // itself is this library's design, not the paper's).
 //
-// The kernel runs in clusters of c CTAs (c = 1, 2, 4 or 8, chosen per batch).
+// The kernel runs in clusters of c CTAs (c = 1, 2, 4, 8 or 16, chosen per batch).
 // Each cluster repeatedly takes the next work item from a device counter (items
 // pre-sorted by decreasing cost): one large set (at least c tiles of 2^11
 // amplitudes per pass), whose tiles the c CTAs share with hardware cluster
@@ -13,10 +13,10 @@
 //   1. gate matrices of the set from its parameters (forward and adjoint);
 //   2. forward sweep psi = U_G ... U_1 |0> as greedy tile passes (<= 11 tile
 //      qubits, Q60 arithmetic in shared memory);
-//   3. lambda = (H / S) psi and E = S Re<psi|lambda> (FP64 gather);
+//   3. lambda = (H / S) psi and E = S Re<psi|lambda> (Q60 gather, exact sum);
 //   4. backward sweep over the passes in reverse: for every op in reverse, the
 //      generator inner product Im<lambda|G|psi> over the tile (Q60 products,
-//      FP64 accumulation, fixed reduction order), then U^dag on both tiles.
+//      exact integer sums), then U^dag on both tiles.
 // The host side of a run (parameters in, energies and gradients out) is
 // captured once in a CUDA graph and replayed.
 #include <math.h>

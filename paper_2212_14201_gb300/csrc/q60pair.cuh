@@ -1,6 +1,10 @@
-// Two real one-qubit rotations on tile bits a and b, applied to an amplitude
-// quad as two complex products (Q60 engine).
+// Real one-qubit rotations on two, three or four tile bits, applied to amplitude
+// groups as complex products (Q60 engine).  First the forms with four real products a
+// complex product (q60_pair_comp, q60_triple_comp, q60_quad4_comp: the derivations,
+// pinned by the host tests), then the forms with three that the kernels run
+// (q60_pair_gauss, q60_triple_gauss, q60_quad4_gauss).
 //
+// Two rotations on bits a and b of a quad:
 // On one real component, the quad (x00, x01, x10, x11) (index bit(a) + 2 bit(b))
 // is two complex numbers z_b = x_b0 + i x_b1.  A rotation R_a = [[c, -s], [s, c]]
 // multiplies each z_b by w_a = c + i s; R_b mixes z_0 and z_1 with real

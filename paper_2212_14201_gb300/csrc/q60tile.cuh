@@ -18,7 +18,7 @@ namespace qs {
 
 constexpr int BT_THREADS = 256;
 constexpr int BT_M = 11;          // tile qubits: psi and lambda tiles of 2^11 x 16 B
-constexpr int BT_MAX_OPS = 128;   // ops (and gradient slots) per pass: keeps 3 CTAs per SM
+constexpr int BT_MAX_OPS = 128;   // gates (and gradient slots) per pass
 constexpr int BT_MAX_N = 24;
 constexpr int BT_OFFS = 1 << (BT_M - 3);  // high-bit offset table: tiles hold qubits 0..2 (or all of n < 3)
 
