@@ -578,6 +578,7 @@ def bench_learned_plan(q, torch, stream):
         plans = {"greedy": q.qs_plan_create(n, g, q.PLAN_GREEDY, 5), "learned": q.qs_plan_create_learned(n, g, model),
                  "plain": None}
         for name, p in plans.items():
+            q.qs_timing_enable(h, p is None)  # without a plan: a kernel per gate only while launches are logged
             q.qs_set_zero(h)
             q.qs_apply(h, g, None, p)
             q.qs_set_zero(h)
@@ -590,6 +591,8 @@ def bench_learned_plan(q, torch, stream):
             st = q.qs_plan_get_stats(p) if p else {}
             out[name] = {"ms": ms, "amp_updates_per_s": len(g) * float(1 << n) / (ms * 1e-3),
                          "passes": st.get("n_passes"), "tile_qubits": st.get("tile_qubits")}
+        q.qs_timing_fetch(h)
+        q.qs_timing_enable(h, False)
         out["norm2"] = float(q.qs_probs(h, [])[0])
         out["learned_gain_vs_greedy"] = out["greedy"]["ms"] / out["learned"]["ms"]
         out["learned_gain_vs_plain"] = out["plain"]["ms"] / out["learned"]["ms"]
@@ -789,7 +792,7 @@ def run_ours(args, world, rank, local, pg):
                 "d2h_bytes_per_step": SHOTS * 8 + 8, "matches_device_run": bool(ok_e2e),
                 "plan_ms": plan_ms,
                 "plan_note": "the greedy plan is built once before the timed steps (host, plan_ms) and reused; "
-                             "each step's op lists and phase tables are rebuilt on the host from the gate list"},
+                             "each step's op lists are rebuilt on the host from the gate list, its phase tables on the device"},
         "gpu_launches": int(launches),
         "clocks": clocks,
         "batched_vqe": extra.get("batched_vqe"),
