@@ -643,10 +643,7 @@ extern "C" int qs_adjoint_grad(qs_state* s, const qs_gate* gates, size_t ng, con
       (rc = choose_fixed(s, &fixed)) == QS_OK) {
     const bool keep = fixed && g_adj_fused;
     rc = qs_apply_plan(s, gates, ng, params, plan, fixed, keep ? &held : nullptr);
-    if (rc == QS_OK && keep && !held) {
-      rc = launch_q60_hold(s);
-      held = rc == QS_OK;
-    }
+    if (rc == QS_OK && keep && !held) rc = launch_q60_hold(s, &held);
   }
   if (plan) qs_plan_free(plan);
   if (rc == QS_OK) rc = apply_hamiltonian(s, s->amps, lam, terms, nterms, S, held);
@@ -716,10 +713,13 @@ extern "C" int qs_adjoint_grad(qs_state* s, const qs_gate* gates, size_t ng, con
     if (e != cudaSuccess) rc = cuda_fail(e, "adjoint readback");
   }
   if (held) {  // the state is complex128 again, also after an error
-    const int rc2 = launch_q60_release(s);
+    const int rc2 = launch_q60_release(s, &held);
     if (rc == QS_OK) rc = rc2;
   }
-  if (rc != QS_OK) return rc;
+  if (rc != QS_OK) {
+    s->bound = 0;
+    return rc;
+  }
   *energy = host[nslots] * S;
   for (size_t j = 0; j < np; ++j) grad[j] = 0.0;
   for (size_t j = 0; j < nslots; ++j) grad[slot_param[j]] += host[j] * S;

@@ -87,8 +87,9 @@ int cuda_fail(cudaError_t e, const char* what) {
 
 void clear_error() { g_err.clear(); }
 
-int launch_check(const char* what) {
+int launch_check(const char* what, bool* queued) {
   cudaError_t e = cudaGetLastError();
+  if (queued) *queued = e == cudaSuccess;
   if (e != cudaSuccess) return cuda_fail(e, what);
   if (fault_fire(QS_FAULT_LAUNCH)) return cuda_fail(cudaErrorLaunchFailure, what);
   return QS_OK;

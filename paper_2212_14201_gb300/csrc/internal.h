@@ -108,7 +108,9 @@ void clear_error();
   } while (0)
 
 int check_state(const qs_state* s);
-int launch_check(const char* what);  // cudaGetLastError after a launch
+// cudaGetLastError after a launch; *queued: whether the kernel was queued (an injected
+// failure comes after that).
+int launch_check(const char* what, bool* queued = nullptr);
 
 // ---- host-side fault injection (qs_fault_set, QS_FAULT) --------------------------
 // True when the armed fault of `kind` (QS_FAULT_ALLOC or QS_FAULT_LAUNCH) fires at
@@ -173,9 +175,10 @@ int unit_code(const C2& z);
 // Whether the next gate kernels of this state run in Q60 fixed point (may
 // synchronise once to bound an unknown state's magnitude).
 int choose_fixed(qs_state* s, bool* fixed);
-// Buffer conversions in place: complex128 to Q60 integer pairs, and back.
-int launch_q60_hold(qs_state* s);
-int launch_q60_release(qs_state* s);
+// Buffer conversions in place: complex128 to Q60 integer pairs, and back.  *held: what
+// the buffer holds once the queued kernels have run, also after an error.
+int launch_q60_hold(qs_state* s, bool* held);
+int launch_q60_release(qs_state* s, bool* held);
 int launch_op1(qs_state* s, const Op1& op, bool fixed);  // complex64 states: FP32 arithmetic
 int launch_dense(qs_state* s, const int* targets, int k, uint64_t cmask, const C2* mat);
 
@@ -240,6 +243,7 @@ int ensure_pinned(qs_state* s, size_t bytes);
 // The passes that qs_apply runs for a gate list without a plan.
 int plan_implicit(int n, int prec, const qs_gate* gates, size_t ng, qs_plan** out);
 // qs_apply with a plan.  held != nullptr: the amplitudes may stay Q60 integers after a
-// last tile pass (*held says so); else they are complex128 when the call returns.
+// last tile pass (*held says so); else, and after an error, they are complex128 when
+// the call returns.
 int qs_apply_plan(qs_state* s, const qs_gate* gates, size_t ng, const double* params, const qs_plan* plan,
                   bool fixed, bool* held = nullptr);

@@ -1744,8 +1744,8 @@ static int build_tile_args(int n, int prec, const PlanPass& ps, const qs_gate* g
   return rc;
 }
 
-// io: TileArgs::io (Q60 engine only); *launched: whether a kernel ran (a pass
-// whose ops all cancel launches nothing).
+// io: TileArgs::io (Q60 engine only); *launched: whether the pass's kernel was queued,
+// also when the call fails (a pass whose ops all cancel launches nothing).
 static int run_tile_pass(qs_state* s, const PlanPass& ps, const qs_gate* gates, const double* params, bool fixed,
                          int io, bool* launched, bool direct) {
   *launched = false;
@@ -1756,8 +1756,7 @@ static int run_tile_pass(qs_state* s, const PlanPass& ps, const qs_gate* gates, 
   int rc = build_tile_args(s->n, s->prec, ps, gates, params, fixed, io, g, ptables, &flops, &int_ops, direct);
   if (rc == QS_OK && !ptables.empty()) rc = build_tables(s, ptables, &g->tables, s->prec == 64);
   if (rc == QS_OK && (g->nops > 0 || (g->io >> 8) != 0)) {
-    rc = launch_tile(s, *g, fixed ? 0.0 : flops, fixed ? int_ops : 0.0, (int)ps.gates.size(), fixed);
-    *launched = rc == QS_OK;
+    rc = launch_tile(s, *g, fixed ? 0.0 : flops, fixed ? int_ops : 0.0, (int)ps.gates.size(), fixed, launched);
   }
   delete g;
   return rc;
@@ -1802,22 +1801,18 @@ extern "C" int qs_plan_pass_kernel_ops(const qs_plan* p, size_t pass, const qs_g
   return tile_pass_profile(p->n, p->passes[pass], gates, params, counts, int_ops_per_amp);
 }
 
-int qs_apply_plan(qs_state* s, const qs_gate* gates, size_t ng, const double* params, const qs_plan* plan,
-                  bool fixed, bool* held_out) {
-  if (plan->n != s->n || plan->ng != ng || plan->fingerprint != fingerprint(gates, ng))
-    return fail(QS_ERR_INVALID_ARG, "plan does not match the program");
-  // Between consecutive Q60 tile passes the buffer keeps the Q60 integers (the
-  // same 16 bytes per amplitude): no conversion to complex128 and back, and no
-  // rounding to double in between.  It is complex128 again when the call returns.
+// The passes of a plan.  Between consecutive Q60 tile passes the buffer keeps the Q60
+// integers (the same 16 bytes per amplitude): no conversion to complex128 and back, and
+// no rounding to double in between.  *held: whether it holds them now, also after an
+// error; last_held: it may hold them at the end.
+static int run_passes(qs_state* s, const qs_gate* gates, const double* params, const qs_plan* plan, bool fixed,
+                      bool last_held, bool* held_out) {
   const bool q60 = fixed && s->prec == 128;
-  bool held = false;
+  bool& held = *held_out;
   for (size_t i = 0; i < plan->passes.size(); ++i) {
     const PlanPass& ps = plan->passes[i];
     if (ps.kind == PASS_GATE) {
-      if (held) {
-        QS_TRY(launch_q60_release(s));
-        held = false;
-      }
+      if (held) QS_TRY(launch_q60_release(s, &held));
       const qs_gate& g = gates[ps.gates[0]];
       int t;
       uint64_t cm;
@@ -1827,14 +1822,28 @@ int qs_apply_plan(qs_state* s, const qs_gate* gates, size_t ng, const double* pa
       QS_TRY(launch_op1(s, classify(t, cm, m), fixed));
     } else {
       const bool last = i + 1 == plan->passes.size();
-      const bool next_tile = q60 && (last ? held_out != nullptr : plan->passes[i + 1].kind == PASS_TILE);
+      const bool next_tile = q60 && (last ? last_held : plan->passes[i + 1].kind == PASS_TILE);
       bool launched = false;
-      QS_TRY(run_tile_pass(s, ps, gates, params, fixed, (held ? 1 : 0) | (next_tile ? 2 : 0), &launched,
-                           plan->direct));
+      const int rc = run_tile_pass(s, ps, gates, params, fixed, (held ? 1 : 0) | (next_tile ? 2 : 0), &launched,
+                                   plan->direct);
       if (launched) held = next_tile;
+      if (rc != QS_OK) return rc;
     }
   }
-  if (held_out) *held_out = held;
-  else if (held) QS_TRY(launch_q60_release(s));
   return QS_OK;
+}
+
+int qs_apply_plan(qs_state* s, const qs_gate* gates, size_t ng, const double* params, const qs_plan* plan,
+                  bool fixed, bool* held_out) {
+  if (plan->n != s->n || plan->ng != ng || plan->fingerprint != fingerprint(gates, ng))
+    return fail(QS_ERR_INVALID_ARG, "plan does not match the program");
+  bool held = false;
+  int rc = run_passes(s, gates, params, plan, fixed, held_out != nullptr, &held);
+  if (held && (rc != QS_OK || !held_out)) {  // integers would be read as doubles
+    const int rc2 = launch_q60_release(s, &held);
+    if (rc == QS_OK) rc = rc2;
+  }
+  if (rc != QS_OK) s->bound = 0;  // a kernel may be missing: the next call looks at the norm again
+  if (held_out) *held_out = held;
+  return rc;
 }

@@ -896,7 +896,7 @@ __global__ void k_q60_hold(double2* __restrict__ a, size_t N) {
 }
 
 template <class E, int THREADS>
-static int launch_engine_t(qs_state* s, const TileArgs& g, size_t smem) {
+static int launch_engine_t(qs_state* s, const TileArgs& g, size_t smem, bool* queued) {
   static bool attr_set = false;
   static int sms = 0;
   if (!attr_set) {
@@ -908,7 +908,7 @@ static int launch_engine_t(qs_state* s, const TileArgs& g, size_t smem) {
   QS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_tile<E, THREADS>, THREADS, smem));
   const uint64_t grid = std::min<uint64_t>(g.ntiles, (uint64_t)std::max(1, sms) * std::max(1, per_sm));
   k_tile<E, THREADS><<<(unsigned)grid, THREADS, smem, s->stream>>>(reinterpret_cast<typename E::G*>(s->amps), g);
-  return launch_check("tile kernel");
+  return launch_check("tile kernel", queued);
 }
 
 // 256 threads per CTA (measured at n=30, 12-qubit tiles: 512 threads with 2 CTAs
@@ -916,37 +916,44 @@ static int launch_engine_t(qs_state* s, const TileArgs& g, size_t smem) {
 // runs 512 threads, and so does a pass of at most one tile of 11 qubits or more per
 // SM, where a CTA has the SM to itself.
 template <class E>
-static int launch_engine(qs_state* s, const TileArgs& g) {
+static int launch_engine(qs_state* s, const TileArgs& g, bool* queued) {
   const size_t H = (size_t)1 << g.nhigh;
   const size_t smem = ((H * sizeof(uint64_t) + 15) & ~(size_t)15) + (sizeof(typename E::T) << g.m);
-  if (g.m >= 13 || (g.m >= 11 && g.ntiles <= 152)) return launch_engine_t<E, 512>(s, g, smem);
-  return launch_engine_t<E, 256>(s, g, smem);
+  if (g.m >= 13 || (g.m >= 11 && g.ntiles <= 152)) return launch_engine_t<E, 512>(s, g, smem, queued);
+  return launch_engine_t<E, 256>(s, g, smem, queued);
 }
 
-int launch_q60_release(qs_state* s) {
+int launch_q60_release(qs_state* s, bool* held) {
   const size_t N = (size_t)1 << s->n;
   const int blocks = (int)std::min<size_t>((N + 255) / 256, 152 * 16);
   KTimer kt(s, QS_K_OTHER, 0, 0, 0, 0, (double)N, 0.0);
   k_q60_release<<<blocks, 256, 0, s->stream>>>(s->amps, N);
-  return launch_check("q60 release");
+  bool queued = false;
+  const int rc = launch_check("q60 release", &queued);
+  if (queued) *held = false;
+  return rc;
 }
 
-int launch_q60_hold(qs_state* s) {
+int launch_q60_hold(qs_state* s, bool* held) {
   const size_t N = (size_t)1 << s->n;
   KTimer kt(s, QS_K_OTHER, 0, 0, 0, 0, (double)N, 0.0);
   k_q60_hold<<<(int)std::min<size_t>((N + 255) / 256, 152 * 16), 256, 0, s->stream>>>(s->amps, N);
-  return launch_check("q60 hold");
+  bool queued = false;
+  const int rc = launch_check("q60 hold", &queued);
+  if (queued) *held = true;
+  return rc;
 }
 
-int launch_tile(qs_state* s, const TileArgs& g, double flops, double int_ops, int ngates, bool fixed) {
+int launch_tile(qs_state* s, const TileArgs& g, double flops, double int_ops, int ngates, bool fixed,
+                bool* queued) {
   size_t H = (size_t)1 << g.nhigh;
   size_t smem = ((H * sizeof(uint64_t) + 15) & ~(size_t)15) + ((size_t)16 << g.m);
   uint64_t qmask = 0;
   for (int b = 0; b < g.m - g.nhigh; ++b) qmask |= 1ull << b;
   for (int b = 0; b < g.nhigh; ++b) qmask |= 1ull << g.qhigh[b];
   KTimer kt(s, QS_K_TILE, g.m, ngates, qmask, 0, (double)(1ull << g.n), flops, int_ops);
-  if (s->prec == 64) return launch_engine<EngF32>(s, g);
-  return fixed ? launch_engine<EngQ60>(s, g) : launch_engine<EngF64>(s, g);
+  if (s->prec == 64) return launch_engine<EngF32>(s, g, queued);
+  return fixed ? launch_engine<EngQ60>(s, g, queued) : launch_engine<EngF64>(s, g, queued);
 }
 
 }  // namespace qs

@@ -97,6 +97,8 @@ static_assert(4 * TILE_MAX_M + 5 * TILE_MAX_OPS <= TABLE_ARGS_WORDS, "one table 
 // Multiplies the tables out at `out` (Q60 limb pairs of Re and Im, or float2).
 int launch_tables(qs_state* s, const TableArgs& args, void* out);
 
-int launch_tile(qs_state* s, const TileArgs& args, double flops, double int_ops, int ngates, bool fixed);
+// *queued: whether the kernel was queued (also when its launch check failed).
+int launch_tile(qs_state* s, const TileArgs& args, double flops, double int_ops, int ngates, bool fixed,
+                bool* queued);
 
 }  // namespace qs
