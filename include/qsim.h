@@ -204,8 +204,11 @@ int qs_state_modified(qs_state* s);
  * param_idx >= 0) supplies theta for parametrised records; param_idx must be
  * < the caller's params length (not checkable: the caller guarantees it).
  * plan == NULL: the gates run in passes that the call plans for itself, or one
- * kernel per gate (plain mode) where the timing log is on, arithmetic is FP64 or
- * there is one gate only.  Otherwise the plan must have
+ * kernel per gate (plain mode) where the timing log is on, arithmetic is FP64, or
+ * there is one gate only.  Either way an amplitude is rounded only by gates that
+ * multiply it: a list of X, Y, Z, S, CNOT, CZ and the like (unit factors) moves
+ * the bits that it finds, and one whose other gates are all controlled or act on
+ * half the amplitudes (T, P, CR) runs per gate.  Otherwise the plan must have
  * been created from exactly this gate list and qubit count; its passes are run
  * (fused mode) with matrices computed from `params` at this call.
  * Every record is validated before any work is queued: a bad record returns

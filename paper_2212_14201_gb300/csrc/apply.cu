@@ -463,6 +463,31 @@ int launch_dense(qs_state* s, const int* targets, int k, uint64_t cmask, const C
 
 using namespace qs;
 
+// What a gate list rounds when it runs gate by gate in Q60 arithmetic: no amplitude
+// (only unit factors, which move bits), some amplitudes (phases and controlled gates
+// alone), or all of them (an uncontrolled gate with arithmetic in both halves).
+enum ListRounds { ROUNDS_NONE, ROUNDS_SOME, ROUNDS_ALL };
+static int list_rounds(const qs_gate* gates, size_t ng, int n, const double* params, ListRounds* out) {
+  *out = ROUNDS_NONE;
+  for (size_t k = 0; k < ng; ++k) {
+    int t;
+    uint64_t cm;
+    Mat2 m;
+    QS_TRY(gate_qubits(gates[k], n, &t, &cm));
+    QS_TRY(gate_matrix(gates[k], params, &m));
+    const Op1 op = classify(t, cm, m);
+    if (op.cls == OP_IDENTITY || !needs_arith(op)) continue;
+    *out = ROUNDS_SOME;
+    const bool both = op.cls == OP_REAL || op.cls == OP_GENERAL ||
+                      (op.cls != OP_PHASE1 && op.code0 == U_GENERAL && op.code1 == U_GENERAL);
+    if (both && cm == 0) {
+      *out = ROUNDS_ALL;
+      return QS_OK;
+    }
+  }
+  return QS_OK;
+}
+
 extern "C" int qs_apply(qs_state* s, const qs_gate* gates, size_t ng, const double* params, const qs_plan* plan) {
   clear_error();
   QS_TRY(check_state(s));
@@ -474,10 +499,16 @@ extern "C" int qs_apply(qs_state* s, const qs_gate* gates, size_t ng, const doub
   // for 600): a kernel per gate is a launch of 4 us each on small states and a sweep
   // of HBM each on large ones.  Per gate stay FP64 arithmetic and a state whose
   // timing log is on (its user asks for the gates one by one).
-  if (ng > 1 && !s->timing && (fixed || s->prec == 64)) {
+  // A Q60 pass rounds every amplitude to 2^-60, a kernel per gate only those that the
+  // gate multiplies.  So a list without arithmetic runs its passes in the FP64 engine,
+  // where unit factors move bits, and one whose arithmetic reaches some amplitudes only
+  // runs per gate: the others stay as they are.
+  ListRounds rounds = ROUNDS_ALL;
+  if (fixed && ng > 1) QS_TRY(list_rounds(gates, ng, s->n, params, &rounds));
+  if (ng > 1 && !s->timing && (fixed || s->prec == 64) && rounds != ROUNDS_SOME) {
     qs_plan* p = nullptr;
     if (plan_implicit(s->n, s->prec, gates, ng, &p) == QS_OK) {
-      const int rc = qs_apply_plan(s, gates, ng, params, p, fixed);
+      const int rc = qs_apply_plan(s, gates, ng, params, p, fixed && rounds == ROUNDS_ALL);
       qs_plan_free(p);
       return rc;
     }
