@@ -372,8 +372,8 @@ static int backward_fused(qs_state* s, double2* lam, const qs_gate* gates, size_
   }
   const int m = std::min(n, BT_M);
   const uint64_t low = (1ull << std::min(n, 3)) - 1;
-  std::vector<uint32_t> remaining(ng), pass, rest;
-  for (size_t i = 0; i < ng; ++i) remaining[i] = (uint32_t)i;
+  GateQueue remaining = gate_queue(tgt, cms), rest;
+  std::vector<uint32_t> pass;
   std::vector<BOp> ops;
   std::vector<Mat2> opm;  // each op's matrix (double), parallel to ops
   std::vector<QC> mats;
@@ -482,7 +482,7 @@ static int backward_fused(qs_state* s, double2* lam, const qs_gate* gates, size_
     passes.push_back(bp);
     slot_bases.push_back(slot_base);
     slot_base += slot;
-    remaining.swap(rest);
+    std::swap(remaining, rest);
   }
   // one upload from pinned memory into the workspace (or, if that is too small, into
   // memory of this call)

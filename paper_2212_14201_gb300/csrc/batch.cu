@@ -628,8 +628,8 @@ extern "C" int qs_batch_create(size_t nsets, const int* n_per_set, const qs_gate
     const int dg_first = (int)dgheads.size(), rp_first = (int)rpheads.size();
     const int m = std::min(n, BT_M);
     const uint64_t low = (1ull << std::min(n, 3)) - 1;
-    std::vector<uint32_t> remaining(ng), pass, rest;
-    for (size_t k = 0; k < ng; ++k) remaining[k] = (uint32_t)k;
+    GateQueue remaining = gate_queue(tgt, cms), rest;
+    std::vector<uint32_t> pass;
     st.pass_begin = (int)passes.size();
     while (!remaining.empty()) {
       uint64_t Q = greedy_pass(gates + g0, tgt, cms, remaining, m, low, BT_MAX_OPS, pass, rest);
@@ -688,7 +688,7 @@ extern "C" int qs_batch_create(size_t nsets, const int* n_per_set, const qs_gate
       bp.rp_end = (int)rpheads.size();
       bp.nslots = slot;
       passes.push_back(bp);
-      remaining.swap(rest);
+      std::swap(remaining, rest);
     }
     st.npasses = (int)passes.size() - st.pass_begin;
     st.dg_begin = dg_first;

@@ -186,21 +186,33 @@ int launch_dense(qs_state* s, const int* targets, int k, uint64_t cmask, const C
 bool structurally_diagonal(int type);
 
 // ---- planning ------------------------------------------------------------------
-// One greedy fusion pass over `remaining` (indices in program order): `pass`
-// receives the gates that run in a tile of at most m qubits containing `low`,
-// `rest` the others (still in order); returns the tile's qubit mask.
+// The gates of a program that no pass has taken yet, in program order: `left` (indices
+// that passes looked at and left), then next .. end - 1, which none has looked at.
+struct GateQueue {
+  std::vector<uint32_t> left;
+  uint32_t next = 0, end = 0;
+  uint64_t used = 0;  // qubits of the whole program
+  bool empty() const { return left.empty() && next == end; }
+};
+GateQueue gate_queue(const std::vector<int>& tgt, const std::vector<uint64_t>& cms);
+// One greedy fusion pass over the queue `in`: `pass` receives the gates that run in a
+// tile of at most m qubits containing `low`, `rest` the others (still in order; not
+// `in` itself); returns the tile's qubit mask.  The scan ends where the pass is full,
+// where every qubit waits for a gate already left, or after PASS_SCAN_LEFT gates left,
+// so that planning a program takes time in proportion to its gates.
+constexpr int PASS_SCAN_LEFT = 2048;
 uint64_t greedy_pass(const qs_gate* gates, const std::vector<int>& tgt, const std::vector<uint64_t>& cms,
-                     const std::vector<uint32_t>& remaining, int m, uint64_t low, int max_ops,
-                     std::vector<uint32_t>& pass, std::vector<uint32_t>& rest);
+                     const GateQueue& in, int m, uint64_t low, int max_ops, std::vector<uint32_t>& pass,
+                     GateQueue& rest);
 // The same scan starting from the qubit set `init` (it grows while it has fewer
 // than m qubits, never by a qubit of `forbid`).
 uint64_t greedy_pass_from(const qs_gate* gates, const std::vector<int>& tgt, const std::vector<uint64_t>& cms,
-                          const std::vector<uint32_t>& remaining, int m, uint64_t init, int max_ops,
-                          std::vector<uint32_t>& pass, std::vector<uint32_t>& rest, uint64_t forbid = 0);
+                          const GateQueue& in, int m, uint64_t init, int max_ops, std::vector<uint32_t>& pass,
+                          GateQueue& rest, uint64_t forbid = 0);
 // A starting qubit set for a pass: `low`, the first runnable gate's target and
 // the most frequent targets among the next `window` runnable gates (m qubits).
 uint64_t seed_qubits(const qs_gate* gates, const std::vector<int>& tgt, const std::vector<uint64_t>& cms,
-                     const std::vector<uint32_t>& remaining, int m, uint64_t low, int window);
+                     const GateQueue& in, int m, uint64_t low, int window);
 
 // Inputs of a cost model (0 for NULL).
 int mlp_inputs(const qs_mlp* m);

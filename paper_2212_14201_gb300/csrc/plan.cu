@@ -653,10 +653,17 @@ static void extract_phases(const std::vector<Op1>& ops, const int* local, int n,
   commit(none.data());
 }
 
+GateQueue gate_queue(const std::vector<int>& tgt, const std::vector<uint64_t>& cms) {
+  GateQueue q;
+  q.end = (uint32_t)tgt.size();
+  for (size_t k = 0; k < tgt.size(); ++k) q.used |= cms[k] | (1ull << tgt[k]);
+  return q;
+}
+
 uint64_t greedy_pass(const qs_gate* gates, const std::vector<int>& tgt, const std::vector<uint64_t>& cms,
-                     const std::vector<uint32_t>& remaining, int m, uint64_t low, int max_ops,
-                     std::vector<uint32_t>& pass, std::vector<uint32_t>& rest) {
-  return greedy_pass_from(gates, tgt, cms, remaining, m, low, max_ops, pass, rest);
+                     const GateQueue& in, int m, uint64_t low, int max_ops, std::vector<uint32_t>& pass,
+                     GateQueue& rest) {
+  return greedy_pass_from(gates, tgt, cms, in, m, low, max_ops, pass, rest);
 }
 
 // Qubits to start a pass with, from the remaining gates' targets: the target of
@@ -665,13 +672,15 @@ uint64_t greedy_pass(const qs_gate* gates, const std::vector<int>& tgt, const st
 // ties), up to m qubits with `low`.  A pass that starts from them keeps the
 // qubits most gates act on, where the greedy scan takes targets in program order.
 uint64_t seed_qubits(const qs_gate* gates, const std::vector<int>& tgt, const std::vector<uint64_t>& cms,
-                     const std::vector<uint32_t>& remaining, int m, uint64_t low, int window) {
+                     const GateQueue& in, int m, uint64_t low, int window) {
   uint64_t blockedN = 0, blockedD = 0;
   int count[64] = {0}, first_seen[64];
   for (int b = 0; b < 64; ++b) first_seen[b] = 1 << 30;
   uint64_t Q = low;
-  int seen = 0, order = 0;
-  for (uint32_t k : remaining) {
+  int seen = 0, order = 0, left = 0;
+  const size_t nl = in.left.size(), total = nl + (in.end - in.next);
+  for (size_t i = 0; i < total && left < PASS_SCAN_LEFT && (blockedN & in.used) != in.used; ++i) {
+    const uint32_t k = i < nl ? in.left[i] : in.next + (uint32_t)(i - nl);
     const bool diag = structurally_diagonal(gates[k].type);
     const uint64_t Nm = diag ? 0 : (1ull << tgt[k]);
     const uint64_t Dm = (diag ? (1ull << tgt[k]) : 0) | cms[k];
@@ -679,6 +688,7 @@ uint64_t seed_qubits(const qs_gate* gates, const std::vector<int>& tgt, const st
     if (blocked) {
       blockedN |= Nm;
       blockedD |= Dm;
+      ++left;
       continue;
     }
     if (!Nm) continue;
@@ -701,24 +711,30 @@ uint64_t seed_qubits(const qs_gate* gates, const std::vector<int>& tgt, const st
 }
 
 uint64_t greedy_pass_from(const qs_gate* gates, const std::vector<int>& tgt, const std::vector<uint64_t>& cms,
-                          const std::vector<uint32_t>& remaining, int m, uint64_t init, int max_ops,
-                          std::vector<uint32_t>& pass, std::vector<uint32_t>& rest, uint64_t forbid) {
+                          const GateQueue& in, int m, uint64_t init, int max_ops, std::vector<uint32_t>& pass,
+                          GateQueue& rest, uint64_t forbid) {
   uint64_t Q = init;
   uint64_t blockedN = 0, blockedD = 0;
   pass.clear();
-  rest.clear();
+  rest.left.clear();
+  rest.end = in.end;
+  rest.used = in.used;
   int nops = 0;
-  for (uint32_t k : remaining) {
+  const size_t nl = in.left.size(), total = nl + (in.end - in.next);
+  size_t i = 0;
+  // (past a full pass, or once every used qubit is blocked, each gate would be left)
+  for (; i < total && nops < max_ops && (blockedN & in.used) != in.used && rest.left.size() < PASS_SCAN_LEFT; ++i) {
+    const uint32_t k = i < nl ? in.left[i] : in.next + (uint32_t)(i - nl);
     const bool diag = structurally_diagonal(gates[k].type);
     const uint64_t Nm = diag ? 0 : (1ull << tgt[k]);
     const uint64_t Dm = (diag ? (1ull << tgt[k]) : 0) | cms[k];
-    bool conflict = (Nm & (blockedN | blockedD)) || (Dm & blockedN) || nops >= max_ops;
+    bool conflict = (Nm & (blockedN | blockedD)) || (Dm & blockedN);
     if (!conflict && Nm && !(Q & Nm)) {
       if (__builtin_popcountll(Q) < m && !(Nm & forbid)) Q |= Nm;
       else conflict = true;
     }
     if (conflict) {
-      rest.push_back(k);
+      rest.left.push_back(k);
       blockedN |= Nm;
       blockedD |= Dm;
     } else {
@@ -726,12 +742,14 @@ uint64_t greedy_pass_from(const qs_gate* gates, const std::vector<int>& tgt, con
       ++nops;
     }
   }
+  if (i < nl) rest.left.insert(rest.left.end(), in.left.begin() + (ptrdiff_t)i, in.left.end());
+  rest.next = in.next + (uint32_t)(i < nl ? 0 : i - nl);
   return Q;
 }
 
 }  // namespace qs
 
-// One tile pass over `remaining` at width m, padded to the full width:
+// One tile pass over the queue `in` at width m, padded to the full width:
 //   strategy 0  greedy: targets taken in program order;
 //   strategy 1  seeded: the scan starts from seed_qubits;
 //   strategy 2  lookahead: the greedy pass, or a variant of it that never takes
@@ -758,37 +776,38 @@ static void pad_pass(PlanPass& ps, const std::vector<int>& tgt, const std::vecto
 
 // Gates the greedy pass at width m would absorb from `rest`.
 static size_t greedy_absorbed(const qs_gate* gates, const std::vector<int>& tgt, const std::vector<uint64_t>& cms,
-                              const std::vector<uint32_t>& rest, int n, int m) {
+                              const GateQueue& rest, int n, int m) {
   if (rest.empty()) return 0;
-  std::vector<uint32_t> p2, r2;
+  std::vector<uint32_t> p2;
+  GateQueue r2;
   greedy_pass_from(gates, tgt, cms, rest, m, low_qubits(n), kPassMaxGates, p2, r2);
   return p2.size();
 }
 
 static PlanPass make_pass(const qs_gate* gates, const std::vector<int>& tgt, const std::vector<uint64_t>& cms,
-                          const std::vector<uint32_t>& remaining, int n, int m, int strategy,
-                          std::vector<uint32_t>& rest, uint64_t forbid = 0, uint64_t* grown = nullptr) {
+                          const GateQueue& in, int n, int m, int strategy, GateQueue& rest, uint64_t forbid = 0,
+                          uint64_t* grown = nullptr) {
   const uint64_t low = low_qubits(n);
   PlanPass ps;
   ps.kind = PASS_TILE;
   if (strategy == 2) {
     uint64_t g0 = 0;
-    ps = make_pass(gates, tgt, cms, remaining, n, m, 0, rest, 0, &g0);
+    ps = make_pass(gates, tgt, cms, in, n, m, 0, rest, 0, &g0);
     size_t best = ps.gates.size() + greedy_absorbed(gates, tgt, cms, rest, n, m);
-    std::vector<uint32_t> r;
+    GateQueue r;
     for (uint64_t c = g0; c; c &= c - 1) {
-      PlanPass v = make_pass(gates, tgt, cms, remaining, n, m, 0, r, c & (~c + 1));
+      PlanPass v = make_pass(gates, tgt, cms, in, n, m, 0, r, c & (~c + 1));
       const size_t a = v.gates.size() + greedy_absorbed(gates, tgt, cms, r, n, m);
       if (a > best) {
         best = a;
         ps = std::move(v);
-        rest.swap(r);
+        std::swap(rest, r);
       }
     }
     return ps;
   }
-  const uint64_t init = strategy == 1 ? seed_qubits(gates, tgt, cms, remaining, m, low, 4 * m) : low;
-  ps.qmask = greedy_pass_from(gates, tgt, cms, remaining, m, init, kPassMaxGates, ps.gates, rest, forbid);
+  const uint64_t init = strategy == 1 ? seed_qubits(gates, tgt, cms, in, m, low, 4 * m) : low;
+  ps.qmask = greedy_pass_from(gates, tgt, cms, in, m, init, kPassMaxGates, ps.gates, rest, forbid);
   if (grown) *grown = ps.qmask & ~low;
   pad_pass(ps, tgt, cms, n, m);
   return ps;
@@ -838,8 +857,7 @@ static int plan_build(int n, const qs_gate* gates, size_t ng, int mode, int kmax
     return QS_OK;
   }
 
-  std::vector<uint32_t> remaining(ng), rest;
-  for (size_t k = 0; k < ng; ++k) remaining[k] = (uint32_t)k;
+  GateQueue remaining = gate_queue(tgt, cms), rest;
   while (!remaining.empty()) {
     PlanPass ps = make_pass(gates, tgt, cms, remaining, n, p->m, strategy, rest);
     // Cost: a tile pass sweeps the whole state once and is bound by its limb
@@ -867,7 +885,7 @@ static int plan_build(int n, const qs_gate* gates, size_t ng, int mode, int kmax
       p->est_seconds += tile_cost;
       ++p->n_tile;
     }
-    remaining.swap(rest);
+    std::swap(remaining, rest);
   }
   *out = p;
   return QS_OK;
@@ -1064,11 +1082,10 @@ static int plan_build_learned(int n, const qs_gate* gates, size_t ng, const Pass
   lp->ng = ng;
   lp->fingerprint = fingerprint(gates, ng);
   lp->m = 0;
-  std::vector<uint32_t> remaining(ng);
-  for (size_t k = 0; k < ng; ++k) remaining[k] = (uint32_t)k;
+  GateQueue remaining = gate_queue(tgt, cms);
   struct Cand {
     PlanPass ps;
-    std::vector<uint32_t> rest;
+    GateQueue rest;
     PlanPass next;  // the greedy pass that would follow (no gates at the end)
   };
   std::vector<Cand> cands;
@@ -1079,7 +1096,7 @@ static int plan_build_learned(int n, const qs_gate* gates, size_t ng, const Pass
     for (const Cand& o : cands)
       if (o.ps.qmask == c.ps.qmask && o.ps.gates == c.ps.gates) return;
     if (!c.rest.empty()) {
-      std::vector<uint32_t> r2;
+      GateQueue r2;
       c.next = make_pass(gates, tgt, cms, c.rest, n, std::min(n, TILE_DEFAULT_M), 0, r2);
     }
     cands.push_back(std::move(c));
@@ -1160,7 +1177,7 @@ static int plan_build_learned(int n, const qs_gate* gates, size_t ng, const Pass
         lp->passes.push_back(std::move(g1));
       }
     }
-    remaining.swap(c.rest);
+    std::swap(remaining, c.rest);
   }
   if (lp->m == 0) lp->m = std::min(n, TILE_DEFAULT_M);
   double greedy_total = 0.0;
