@@ -459,6 +459,25 @@ int launch_dense(qs_state* s, const int* targets, int k, uint64_t cmask, const C
   }
 }
 
+static int run_per_gate(qs_state* s, const qs_gate* gates, size_t ng, const double* params, bool fixed) {
+  for (size_t k = 0; k < ng; ++k) {
+    int t;
+    uint64_t cm;
+    Mat2 m;
+    QS_TRY(gate_qubits(gates[k], s->n, &t, &cm));
+    QS_TRY(gate_matrix(gates[k], params, &m));
+    QS_TRY(launch_op1(s, classify(t, cm, m), fixed));
+  }
+  return QS_OK;
+}
+
+int apply_per_gate(qs_state* s, const qs_gate* gates, size_t ng, const double* params) {
+  QS_TRY(validate_gates(gates, ng, s->n, params));
+  bool fixed = false;
+  QS_TRY(choose_fixed(s, &fixed));
+  return run_per_gate(s, gates, ng, params, fixed);
+}
+
 }  // namespace qs
 
 using namespace qs;
@@ -514,15 +533,7 @@ extern "C" int qs_apply(qs_state* s, const qs_gate* gates, size_t ng, const doub
     }
     clear_error();  // no host memory for a plan
   }
-  for (size_t k = 0; k < ng; ++k) {
-    int t;
-    uint64_t cm;
-    Mat2 m;
-    QS_TRY(gate_qubits(gates[k], s->n, &t, &cm));
-    QS_TRY(gate_matrix(gates[k], params, &m));
-    QS_TRY(launch_op1(s, classify(t, cm, m), fixed));
-  }
-  return QS_OK;
+  return run_per_gate(s, gates, ng, params, fixed);
 }
 
 extern "C" int qs_apply_matrix(qs_state* s, const int* targets, int k, uint64_t ctrl_mask, const double* mat) {

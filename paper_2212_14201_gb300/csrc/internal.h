@@ -180,6 +180,9 @@ int choose_fixed(qs_state* s, bool* fixed);
 int launch_q60_hold(qs_state* s, bool* held);
 int launch_q60_release(qs_state* s, bool* held);
 int launch_op1(qs_state* s, const Op1& op, bool fixed);  // complex64 states: FP32 arithmetic
+// A gate list with one kernel per gate, as qs_apply through a QS_PLAN_PLAIN plan (what
+// callers with a fuse switch run with it off).
+int apply_per_gate(qs_state* s, const qs_gate* gates, size_t ng, const double* params);
 int launch_dense(qs_state* s, const int* targets, int k, uint64_t cmask, const C2* mat);
 
 // Whether records of this type are diagonal whatever their parameters.

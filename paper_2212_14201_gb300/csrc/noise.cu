@@ -275,7 +275,7 @@ struct Trajectory {
       if (rc == QS_OK) rc = qs_apply(s, pending.data(), pending.size(), nullptr, p);
       if (p) qs_plan_free(p);
     } else {
-      rc = qs_apply(s, pending.data(), pending.size(), nullptr, nullptr);
+      rc = apply_per_gate(s, pending.data(), pending.size(), nullptr);
     }
     pending.clear();
     return rc;

@@ -116,7 +116,7 @@ struct PaBlock {
           if (!it.plan) QS_TRY(qs_plan_create(nq, it.gates.data(), it.gates.size(), QS_PLAN_GREEDY, 5, &it.plan));
           QS_TRY(qs_apply(s, it.gates.data(), it.gates.size(), params, it.plan));
         } else {
-          QS_TRY(qs_apply(s, it.gates.data(), it.gates.size(), params, nullptr));
+          QS_TRY(apply_per_gate(s, it.gates.data(), it.gates.size(), params));
         }
       } else if (it.kind == 1) {
         if (bits[it.cut]) QS_TRY(qs_apply(s, &it.gate, 1, params, nullptr));

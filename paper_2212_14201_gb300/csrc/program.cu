@@ -9,8 +9,8 @@
 //   part scaled by 1 / sqrt(p_outcome).
 // Inside a program, measurement k (0-based, in execution order) draws
 // u_k = u01(SplitMix64 output k of the stream seeded `seed`), the sampler's
-// generator.  The interpreter runs on the host; every gate run is a qs_apply
-// (plain per-gate kernels, or one cached greedy fusion plan per gate run).
+// generator.  The interpreter runs on the host; a gate run is one kernel per gate,
+// or a qs_apply with the greedy fusion plan cached for it.
 #include <math.h>
 
 #include <algorithm>
@@ -137,7 +137,7 @@ struct Runner {
     const size_t ng = (size_t)(in.gate_end - in.gate_begin);
     if (ng == 0) return QS_OK;
     const qs_gate* g = gates + in.gate_begin;
-    if (!fuse) return qs_apply(s, g, ng, params, nullptr);
+    if (!fuse) return apply_per_gate(s, g, ng, params);
     if (!plans[at]) QS_TRY(qs_plan_create(s->n, g, ng, QS_PLAN_GREEDY, 5, &plans[at]));
     return qs_apply(s, g, ng, params, plans[at]);
   }
