@@ -432,7 +432,7 @@ def bench_reductions(q, torch, stream, hbm_peak: float, reps: int = 3, n: int = 
         q.qs_plan_free(p)
         q.qs_timing_enable(h, True)
         q.qs_expect_pauli(h, terms)
-        pauli_passes = sum(1 for r in q.qs_timing_fetch(h) if r["kind"] == q._lib.K_REDUCE)
+        pauli_passes = sum(1 for r in q.qs_timing_fetch(h) if r["kind"] == q._lib.K_REDUCE and r["items"])
         q.qs_timing_enable(h, False)
         out["pauli_passes"] = pauli_passes
         dev = torch.empty(64, dtype=torch.float64, device="cuda")

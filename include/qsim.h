@@ -688,8 +688,11 @@ int qs_set_batch_cluster(int ctas);
 int qs_batch_free(qs_batch* b);
 
 /* ---- instrumentation ---------------------------------------------------------------
- * Per-kernel timing log of one state: when enabled, every kernel the library
- * queues for the state is bracketed by CUDA events on the state's stream.
+ * Timing log of one state: when enabled, every kernel the library queues for the
+ * state lies between two CUDA events on the state's stream.  One record covers one
+ * step: a gate, a tile pass with the phase tables built for it, a reduction with its
+ * finishing kernel, a sampling.  While the log is on, qs_apply without a plan runs
+ * one kernel per gate; to log the passes, give it a plan.
  * qs_timing_fetch synchronises the stream, converts the pending pairs to
  * milliseconds, returns up to `cap` records (host memory, in launch order),
  * stores the number available in *count and clears the log.  The log is the

@@ -704,6 +704,7 @@ extern "C" int qs_adjoint_grad(qs_state* s, const qs_gate* gates, size_t ng, con
   }
   std::vector<double> host(nslots + 1);
   if (rc == QS_OK) {
+    KTimer kt(s, QS_K_ADJOINT, 0, (int)nslots + 1, 0, 0, 0.0, 0.0);
     k_slot_sums<<<(unsigned)(nslots + 1), 256, 0, s->stream>>>(part, nblocks, sums);
     rc = launch_check("slot sums");
   }

@@ -1011,6 +1011,7 @@ static int marginal_device(qs_state* s, const int* qubits, int nq, double* dout,
       return QS_OK;
     });
     QS_TRY(launch_check("norm2"));
+    note_launch(1);
     k_marginal_finish<<<1, 256, 0, s->stream>>>(part, nblocks, 1, dout);
     return launch_check("norm2 finish");
   }
@@ -1032,6 +1033,7 @@ static int marginal_device(qs_state* s, const int* qubits, int nq, double* dout,
       return QS_OK;
     });
     QS_TRY(launch_check("marginal_tiny"));
+    note_launch(1);
     const int H = 1 << nq;
     k_marginal_finish<<<H, 256, 0, s->stream>>>(part, nblocks, H, dout);
     return launch_check("marginal_finish");
@@ -1172,6 +1174,7 @@ extern "C" int qs_expect_z_all(const qs_state* cs, double* out) {
     return QS_OK;
   });
   QS_TRY(launch_check("expect_z"));
+  note_launch(1);
   k_expect_z_finish<<<n, 256, 0, s->stream>>>(part, nblocks, r, dres);
   QS_TRY(launch_check("expect_z_finish"));
   return read_back(s, dres, n, out);
@@ -1222,7 +1225,7 @@ static int pauli_exact(qs_state* s, const qs_pauli* terms, size_t nterms, double
     PFinish f;
     auto finish = [&] {
       if (next == done) return (int)QS_OK;
-      note_launch(1);
+      KTimer kt(s, QS_K_REDUCE, n, next - done, 0, 0, 0.0, 0.0);  // reads partials, no amplitudes
       k_pauli_exact_finish<<<next - done, 256, 0, s->stream>>>(part, f, sums + 2 * (size_t)done);
       done = next;
       used = 0;
@@ -1256,7 +1259,6 @@ static int pauli_exact(qs_state* s, const qs_pauli* terms, size_t nterms, double
           record(zs[z0 + k], k, nblocks, PZ_MAX);
         }
         KTimer kt(s, QS_K_REDUCE, n, g.nt, 0, 0, (double)(1ull << n), 8.0 * g.nt * (double)(1ull << n));
-        note_launch(1);
         with_amps(s, [&](auto* a) {
           using T = std::remove_cv_t<std::remove_pointer_t<decltype(a)>>;
           k_pauli_z<T><<<nblocks, 256, 0, s->stream>>>(a, g, part + used);
@@ -1294,7 +1296,6 @@ static int pauli_exact(qs_state* s, const qs_pauli* terms, size_t nterms, double
       }
       if (nx) {
         KTimer kt(s, QS_K_REDUCE, n, nx, 0, 0, (double)(1ull << n), 8.0 * nx * (double)(1ull << n));
-        note_launch(1);
         with_amps(s, [&](auto* a) {
           using T = std::remove_cv_t<std::remove_pointer_t<decltype(a)>>;
           k_pauli_x<T><<<xblocks, 256, (size_t)16 << PT_TMAX, s->stream>>>(a, gx, part + used);
@@ -1327,7 +1328,6 @@ static int pauli_exact(qs_state* s, const qs_pauli* terms, size_t nterms, double
         }
       }
       KTimer kt(s, QS_K_REDUCE, n, g.nt, 0, 0, (double)(1ull << n), 8.0 * g.nt * (double)(1ull << n));
-      note_launch(1);
       with_amps(s, [&](auto* a) {
         using T = std::remove_cv_t<std::remove_pointer_t<decltype(a)>>;
         k_pauli_tile<T><<<nblocks, 256, (size_t)16 << g.T, s->stream>>>(a, g, part + used);
@@ -1383,6 +1383,7 @@ extern "C" int qs_expect_pauli(const qs_state* cs, const qs_pauli* terms, size_t
       return QS_OK;
     });
     QS_TRY(launch_check("pauli"));
+    note_launch(1);
     k_pauli_finish<<<1, 32, 0, s->stream>>>(part, nblocks, g.nt, dres);
     QS_TRY(launch_check("pauli_finish"));
     QS_TRY(read_back(s, dres, g.nt, vals.data() + k0));
