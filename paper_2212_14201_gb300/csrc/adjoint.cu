@@ -30,7 +30,7 @@ struct AdjArgs {
   uint64_t cmask;
   int64_t items;
   int t, nfix;
-  int fix[16];
+  int fix[QS_MAX_QUBITS];
   int cls, code0, code1;
   int gen;          // GenKind
   double gsign;     // -1 for a dagger record

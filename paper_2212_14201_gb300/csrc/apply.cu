@@ -24,7 +24,7 @@ struct OpArgs {
   int64_t items;    // work items (pairs, or single amplitudes for PHASE1)
   int t;            // target bit
   int nfix;         // sorted fixed positions (target + controls) to insert
-  int fix[16];
+  int fix[QS_MAX_QUBITS];
   int code0, code1;
 };
 
@@ -100,7 +100,7 @@ struct OpArgs32 {
   int64_t items;
   int t;
   int nfix;
-  int fix[16];
+  int fix[QS_MAX_QUBITS];
   int code0, code1;
 };
 
@@ -161,7 +161,7 @@ struct OpArgsFx {
   uint64_t cmask;
   int64_t items;
   int t, nfix;
-  int fix[16];
+  int fix[QS_MAX_QUBITS];
   int code0, code1;
 };
 
@@ -282,7 +282,6 @@ static int launch_op1_c64(qs_state* s, const Op1& op) {
   g.code1 = op.code1;
   const uint64_t fixbits = op.cmask | (1ull << op.target);
   const int nf = __builtin_popcountll(fixbits);
-  if (nf > 16) return fail(QS_ERR_UNSUPPORTED, "more than 15 controls");
   g.nfix = 0;
   for (int b = 0; b < 64; ++b)
     if ((fixbits >> b) & 1) g.fix[g.nfix++] = b;
@@ -319,7 +318,6 @@ int launch_op1(qs_state* s, const Op1& op, bool fixed) {
     g.code1 = op.code1;
     uint64_t fx = op.cmask | (1ull << op.target);
     int nf = __builtin_popcountll(fx);
-    if (nf > 16) return fail(QS_ERR_UNSUPPORTED, "more than 15 controls");
     g.nfix = 0;
     for (int b = 0; b < 64; ++b)
       if ((fx >> b) & 1) g.fix[g.nfix++] = b;
@@ -351,7 +349,6 @@ int launch_op1(qs_state* s, const Op1& op, bool fixed) {
   g.code1 = op.code1;
   uint64_t fixbits = op.cmask | (1ull << op.target);
   int nf = __builtin_popcountll(fixbits);
-  if (nf > 16) return fail(QS_ERR_UNSUPPORTED, "more than 15 controls");
   g.nfix = 0;
   for (int b = 0; b < 64; ++b)
     if ((fixbits >> b) & 1) g.fix[g.nfix++] = b;
