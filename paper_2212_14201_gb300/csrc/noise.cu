@@ -388,19 +388,27 @@ extern "C" int qs_run_noisy(qs_state* s, const qs_gate* gates, size_t ng, const 
     return (R.gate_type < 0 || R.gate_type == g.type) && (R.q0 < 0 || R.q0 == g.q0) &&
            (R.q1 < 0 || R.q1 == (two_qubit(g.type) ? g.q1 : -1));
   };
-  // q, then the qubits that channels with weights touch from gate k on, until
-  // the table is full or a gate changes the populations of one of them
+  // q, then the qubits that channels with weights touch in the next gates, until the
+  // table is full or a gate changes the populations of one of them.  A qubit whose
+  // populations change before its channel is left out: its entry would be of no use, and
+  // that gate would end the table (a rotation with a channel on every qubit of a layer
+  // then reads one qubit, not eleven, for each).
+  constexpr size_t kAheadGates = 256;  // (looked at again at every table)
+  const uint64_t all = (1ull << s->n) - 1;
   auto ahead = [&](size_t k, int q) {
     std::vector<int> list{q};
-    uint64_t in = 1ull << q;
-    for (size_t j = k; j < ng; ++j) {
+    uint64_t in = 1ull << q, moved = 0;
+    for (size_t j = k; j < ng && j < k + kAheadGates && (in | moved) != all; ++j) {
       int t;
       uint64_t cm;
       if (gate_qubits(gates[j], s->n, &t, &cm) != QS_OK) break;
-      if (j > k && !structurally_diagonal(gates[j].type) && ((in >> t) & 1)) break;
+      if (j > k && !structurally_diagonal(gates[j].type)) {
+        if ((in >> t) & 1) break;
+        moved |= 1ull << t;
+      }
       for (size_t r = 0; r < nrules; ++r) {
         if (sets[r].unital || !matches(rules[r], gates[j])) continue;
-        for (uint64_t b = (cm | (1ull << t)) & ~in; b; b &= b - 1) {
+        for (uint64_t b = (cm | (1ull << t)) & ~(in | moved); b; b &= b - 1) {
           if (list.size() == JOINT_MAX) return list;
           list.push_back(__builtin_ctzll(b));
           in |= b & (0 - b);
