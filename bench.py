@@ -576,9 +576,8 @@ def bench_learned_plan(q, torch, stream):
     h = q.qs_alloc(n, stream)
     try:
         plans = {"greedy": q.qs_plan_create(n, g, q.PLAN_GREEDY, 5), "learned": q.qs_plan_create_learned(n, g, model),
-                 "plain": None}
+                 "plain": q.qs_plan_create(n, g, q.PLAN_PLAIN, 1)}  # (no plan at all would run in passes)
         for name, p in plans.items():
-            q.qs_timing_enable(h, p is None)  # without a plan: a kernel per gate only while launches are logged
             q.qs_set_zero(h)
             q.qs_apply(h, g, None, p)
             q.qs_set_zero(h)
@@ -588,11 +587,10 @@ def bench_learned_plan(q, torch, stream):
             e1.record(stream)
             torch.cuda.synchronize()
             ms = e0.elapsed_time(e1)
-            st = q.qs_plan_get_stats(p) if p else {}
+            st = q.qs_plan_get_stats(p)
             out[name] = {"ms": ms, "amp_updates_per_s": len(g) * float(1 << n) / (ms * 1e-3),
-                         "passes": st.get("n_passes"), "tile_qubits": st.get("tile_qubits")}
-        q.qs_timing_fetch(h)
-        q.qs_timing_enable(h, False)
+                         "passes": None if name == "plain" else st["n_passes"],
+                         "tile_qubits": None if name == "plain" else st["tile_qubits"]}
         out["norm2"] = float(q.qs_probs(h, [])[0])
         out["learned_gain_vs_greedy"] = out["greedy"]["ms"] / out["learned"]["ms"]
         out["learned_gain_vs_plain"] = out["plain"]["ms"] / out["learned"]["ms"]
@@ -711,7 +709,8 @@ def run_ours(args, world, rank, local, pg):
     plain_fp64 = None
     if plan is not None and not args.no_plain:
         ksteps = max(1, args.steps - 1)
-        pms, precs, _, _ = timed(None, ksteps, 1)
+        per_gate = q.qs_plan_create(n, gates, q.PLAN_PLAIN, 1)  # (no plan at all would run in passes)
+        pms, precs, _, _ = timed(per_gate, ksteps, 1)
         pb = sum(r["items"] * 32.0 for r in precs if r["kind"] in (1, 2, 3, 4, 5))
         pg_ms = sum(r["ms"] for r in precs if r["kind"] in (1, 2, 3, 4, 5)) / ksteps
         plain = {"value": whole_job_value(world, amp_updates, pms), "ms_per_step": pms,
@@ -719,10 +718,11 @@ def run_ours(args, world, rank, local, pg):
                  "roofline": roofline(precs, hbm_peak)}
         # the same per-gate kernels with IEEE FP64 arithmetic (context: the FP64 pipe bound)
         q.qs_set_arith(h, q.ARITH_FP64)
-        fms, frecs, _, _ = timed(None, 1, 1)
+        fms, frecs, _, _ = timed(per_gate, 1, 1)
         q.qs_set_arith(h, q.ARITH_AUTO)
         plain_fp64 = {"value": whole_job_value(world, amp_updates, fms), "ms_per_step": fms,
                       "roofline": roofline(frecs, hbm_peak)}
+        q.qs_plan_free(per_gate)
 
     # end to end through the public API: host gate list in, norm and samples out to host
     host_samples = np.empty(SHOTS, dtype=np.uint64)
