@@ -1340,7 +1340,7 @@ extern "C" int qs_set_aggregate(int on) {
 }
 
 
-// The launches that build a pass's phase tables, and where: their factors travel as
+// Builds a pass's phase tables in the state's table buffer: their factors travel as
 // kernel parameters and k_phase_tables multiplies them out there (on the host the
 // 2^m entries of 25 tables took 0.6 ms of the 0.61 ms that 300 random gates on 20
 // qubits needed, and an upload had to wait for the pass before it).  They stay in
@@ -1350,8 +1350,7 @@ extern "C" int qs_set_aggregate(int on) {
 static size_t tables_bytes(const std::vector<PhaseTable>& pt, bool f32) {
   return pt.empty() ? 0 : (pt.size() << pt[0].m) * (f32 ? sizeof(float2) : 2 * sizeof(QL));
 }
-static int plan_tables(qs_state* s, const std::vector<PhaseTable>& pt, const QL** dev, bool f32,
-                       std::vector<TableLaunch>* launches) {
+static int build_tables(qs_state* s, const std::vector<PhaseTable>& pt, const QL** dev, bool f32) {
   const int m = pt[0].m;
   const size_t bytes = tables_bytes(pt, f32), per = bytes / pt.size();
   if (s->ws_bytes < bytes && s->tables_bytes < bytes) {
@@ -1365,9 +1364,9 @@ static int plan_tables(qs_state* s, const std::vector<PhaseTable>& pt, const QL*
     s->tables_bytes = bytes;
   }
   char* buf = (char*)(s->ws_bytes < bytes ? s->tables : s->ws);
+  std::unique_ptr<TableArgs> g(new (std::nothrow) TableArgs);
+  if (!g) return fail(QS_ERR_OOM, "host allocation failed");
   for (size_t t = 0; t < pt.size();) {
-    launches->emplace_back();
-    TableArgs* g = &launches->back().args;
     g->m = m;
     g->f32 = f32;
     g->ntab = 0;
@@ -1407,7 +1406,7 @@ static int plan_tables(qs_state* s, const std::vector<PhaseTable>& pt, const QL*
       used += need;
     }
     if (t == first) return fail(QS_ERR_UNSUPPORTED, "phase table of %zu terms", pt[t].terms.size());
-    launches->back().out = buf + first * per;
+    QS_TRY(launch_tables(s, *g, buf + first * per));
   }
   *dev = (const QL*)buf;
   return QS_OK;
@@ -1772,10 +1771,12 @@ static int run_tile_pass(qs_state* s, const PlanPass& ps, const qs_gate* gates, 
   std::vector<PhaseTable> ptables;
   double flops = 0.0, int_ops = 0.0;
   int rc = build_tile_args(s->n, s->prec, ps, gates, params, fixed, io, g, ptables, &flops, &int_ops, direct);
-  std::vector<TableLaunch> tables;
-  if (rc == QS_OK && !ptables.empty()) rc = plan_tables(s, ptables, &g->tables, s->prec == 64, &tables);
   if (rc == QS_OK && (g->nops > 0 || (g->io >> 8) != 0)) {
-    rc = launch_tile(s, *g, tables, fixed ? 0.0 : flops, fixed ? int_ops : 0.0, (int)ps.gates.size(), fixed, launched);
+    // one record of the timing log for the pass: its tables, then its tile kernel
+    KTimer kt(s, QS_K_TILE, g->m, (int)ps.gates.size(), ps.qmask, 0, (double)(1ull << g->n), fixed ? 0.0 : flops,
+              fixed ? int_ops : 0.0);
+    if (!ptables.empty()) rc = build_tables(s, ptables, &g->tables, s->prec == 64);
+    if (rc == QS_OK) rc = launch_tile(s, *g, fixed, launched);
   }
   delete g;
   return rc;

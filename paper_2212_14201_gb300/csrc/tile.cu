@@ -871,10 +871,10 @@ __global__ void __launch_bounds__(256) k_phase_tables(const __grid_constant__ Ta
   }
 }
 
-static int launch_tables(qs_state* s, const TableLaunch& t) {
-  const uint32_t TS = 1u << t.args.m;
+int launch_tables(qs_state* s, const TableArgs& g, void* out) {
+  const uint32_t TS = 1u << g.m;
   note_launch(1);
-  k_phase_tables<<<t.args.ntab * (TS / std::min(TS, TABLE_RUN)), 256, 0, s->stream>>>(t.args, t.out);
+  k_phase_tables<<<g.ntab * (TS / std::min(TS, TABLE_RUN)), 256, 0, s->stream>>>(g, out);
   return launch_check("phase tables");
 }
 
@@ -944,15 +944,7 @@ int launch_q60_hold(qs_state* s, bool* held) {
   return rc;
 }
 
-int launch_tile(qs_state* s, const TileArgs& g, const std::vector<TableLaunch>& tables, double flops,
-                double int_ops, int ngates, bool fixed, bool* queued) {
-  size_t H = (size_t)1 << g.nhigh;
-  size_t smem = ((H * sizeof(uint64_t) + 15) & ~(size_t)15) + ((size_t)16 << g.m);
-  uint64_t qmask = 0;
-  for (int b = 0; b < g.m - g.nhigh; ++b) qmask |= 1ull << b;
-  for (int b = 0; b < g.nhigh; ++b) qmask |= 1ull << g.qhigh[b];
-  KTimer kt(s, QS_K_TILE, g.m, ngates, qmask, 0, (double)(1ull << g.n), flops, int_ops);
-  for (const TableLaunch& t : tables) QS_TRY(launch_tables(s, t));
+int launch_tile(qs_state* s, const TileArgs& g, bool fixed, bool* queued) {
   if (s->prec == 64) return launch_engine<EngF32>(s, g, queued);
   return fixed ? launch_engine<EngQ60>(s, g, queued) : launch_engine<EngF64>(s, g, queued);
 }

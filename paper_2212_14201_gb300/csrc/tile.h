@@ -94,15 +94,11 @@ struct TableArgs {
   double w[TABLE_ARGS_WORDS];
 };
 static_assert(4 * TILE_MAX_M + 5 * TILE_MAX_OPS <= TABLE_ARGS_WORDS, "one table must fit a launch");
-// A launch that multiplies tables out at `out` (Q60 limb pairs of Re and Im, or float2).
-struct TableLaunch {
-  TableArgs args;
-  void* out;
-};
+// Multiplies the tables out at `out` (Q60 limb pairs of Re and Im, or float2).
+int launch_tables(qs_state* s, const TableArgs& args, void* out);
 
-// A pass: its tables, then its tile kernel, under one record of the timing log.
-// *queued: whether the tile kernel was queued (also when its launch check failed).
-int launch_tile(qs_state* s, const TileArgs& args, const std::vector<TableLaunch>& tables, double flops,
-                double int_ops, int ngates, bool fixed, bool* queued);
+// The tile kernel of a pass (the caller's KTimer covers it and the pass's tables).
+// *queued: whether the kernel was queued (also when its launch check failed).
+int launch_tile(qs_state* s, const TileArgs& args, bool fixed, bool* queued);
 
 }  // namespace qs
