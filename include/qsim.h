@@ -205,7 +205,8 @@ int qs_state_modified(qs_state* s);
  * < the caller's params length (not checkable: the caller guarantees it).
  * plan == NULL: the gates run in passes that the call plans for itself, or one
  * kernel per gate (plain mode) where the timing log is on, arithmetic is FP64, or
- * there is one gate only.  Either way an amplitude is rounded only by gates that
+ * there are too few gates for a pass to pay (one; two or three on most states of
+ * less than 24 qubits).  Either way an amplitude is rounded only by gates that
  * multiply it: a list of X, Y, Z, S, CNOT, CZ and the like (unit factors) moves
  * the bits that it finds, and one whose other gates are all controlled or act on
  * half the amplitudes (T, P, CR) runs per gate.  Otherwise the plan must have

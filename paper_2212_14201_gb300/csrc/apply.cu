@@ -504,6 +504,24 @@ static int list_rounds(const qs_gate* gates, size_t ng, int n, const double* par
   return QS_OK;
 }
 
+// The fewest gates of a list without a plan that run as passes.  Two gates take two short
+// launches alone where a pass takes a long one, so below 24 qubits they stay apart (two
+// random gates and a wait, n = 12: 15.6 us per gate, 17.9 as a pass; n = 18: 17.0, 22.5),
+// and so do three from 18 qubits on (21.0, 23.8; n = 22: 49, 54), where a tile has more
+// work, and three diagonal ones of complex64 from 12 on, which a phase table has to be
+// built for (19.6, 25.1).  From 24 qubits on a pass saves a sweep of HBM (two random
+// gates at n = 24: 143 us per gate, 124 as a pass), but not for two diagonal gates, whose
+// kernels have less arithmetic than a pass (103, 129; complex64 54, 60, from 25 qubits on
+// 111, 106).  Queued one after the other the shortest lists lose up to 2 us to this below
+// 18 qubits (n = 12: 6.1 us as a pass, 8.0 per gate).
+static size_t fewest_pass_gates(const qs_state* s, const qs_gate* gates, size_t ng) {
+  if (ng > 3) return ng;
+  bool diag = true;
+  for (size_t k = 0; k < ng; ++k) diag = diag && structurally_diagonal(gates[k].type);
+  if (s->n >= 24) return diag && (s->prec == 128 || s->n == 24) ? 3 : 2;
+  return s->n >= (s->prec == 128 ? 18 : diag ? 12 : 24) ? 4 : 3;
+}
+
 extern "C" int qs_apply(qs_state* s, const qs_gate* gates, size_t ng, const double* params, const qs_plan* plan) {
   clear_error();
   QS_TRY(check_state(s));
@@ -511,17 +529,18 @@ extern "C" int qs_apply(qs_state* s, const qs_gate* gates, size_t ng, const doub
   bool fixed = false;
   QS_TRY(choose_fixed(s, &fixed));
   if (plan) return qs_apply_plan(s, gates, ng, params, plan, fixed);
-  // Two gates or more run as greedy tile passes planned here (3 us for 20 gates, 30
-  // for 600, 8 ms for 100 000 on 20 qubits): a kernel per gate is a launch of 4 us each on small states and a sweep
-  // of HBM each on large ones.  Per gate stay FP64 arithmetic and a state whose
-  // timing log is on (its user asks for the gates one by one).
+  // Lists of several gates run as greedy tile passes planned here (3 us for 20 gates, 30
+  // for 600, 8 ms for 100 000 on 20 qubits): a kernel per gate is a launch of 4 us each on
+  // small states and a sweep of HBM each on large ones.  Per gate stay FP64 arithmetic and
+  // a state whose timing log is on.
   // A Q60 pass rounds every amplitude to 2^-60, a kernel per gate only those that the
   // gate multiplies.  So a list without arithmetic runs its passes in the FP64 engine,
   // where unit factors move bits, and one whose arithmetic reaches some amplitudes only
   // runs per gate: the others stay as they are.
+  const bool passes = !s->timing && (fixed || s->prec == 64) && ng >= fewest_pass_gates(s, gates, ng);
   ListRounds rounds = ROUNDS_ALL;
-  if (fixed && ng > 1) QS_TRY(list_rounds(gates, ng, s->n, params, &rounds));
-  if (ng > 1 && !s->timing && (fixed || s->prec == 64) && rounds != ROUNDS_SOME) {
+  if (fixed && passes) QS_TRY(list_rounds(gates, ng, s->n, params, &rounds));
+  if (passes && rounds != ROUNDS_SOME) {
     qs_plan* p = nullptr;
     if (plan_implicit(s->n, s->prec, gates, ng, &p) == QS_OK) {
       const int rc = qs_apply_plan(s, gates, ng, params, p, fixed && rounds == ROUNDS_ALL);
