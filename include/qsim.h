@@ -129,8 +129,14 @@ int qs_fault_get(int* kind, long long* after, long long* left, long long* fired,
 
 /* Allocate an n-qubit state (1 <= n <= qs_max_qubits()) on the current CUDA
  * device, bound to `stream` (a cudaStream_t; NULL = the legacy default stream),
- * initialised to |0...0>.  The library owns the amplitude buffer and a small
- * reduction workspace; both are released by qs_free.
+ * initialised to |0...0>.  The library owns the amplitude buffer, a reduction
+ * workspace (10 MB; 24 bytes per 1024 amplitudes where that is more) and, from the
+ * first call on that needs it, a buffer for one call's temporaries, which grows to
+ * what calls asked for, up to 256 MiB (sampling: 2^n bytes for 15 to 27 qubits, else
+ * 2^n / 4, and 8 bytes per shot returned to the host; a gradient: 16 x 2^n and 4.9 KB
+ * per parametrised gate; probabilities returned to the host: 8 bytes each).  A call
+ * that needs more than 256 MiB takes it from the stream's memory pool and gives it
+ * back.  All are released by qs_free, and only there.
  * Errors: INVALID_ARG (n out of range), OOM, CUDA. */
 int qs_alloc(int n, void* stream, qs_state** out);
 
@@ -266,7 +272,7 @@ int qs_set_aggregate(int on);
  * plain diagonal gates between them and the controlled diagonal gates among the
  * tile's qubits (CZ, CR, ...) commute into one table op a_j *= T[j], a diagonal
  * over the tile (2^m phases in device memory, one complex product per
- * amplitude), leaving real rotations: 12 instead of 18 limb products per
+ * amplitude), leaving real rotations: 9 instead of 18 limb products per
  * amplitude.  A table is built where the general ops it makes real and the
  * diagonals it absorbs outweigh its own cost.  The tables are built on the device
  * before each pass.  Results agree with the switch off within rounding (table
@@ -280,8 +286,9 @@ int qs_set_phase_tables(int on);
  * z_b the complex number formed along the first qubit: both rotations act on u
  * and v as multiplications), three on amplitude octets as four complex products
  * (the same basis change along each further qubit), four on one component of 16
- * amplitudes as eight: 8, 16 and 32 real products where the rotations apart take
- * 16, 24 and 64.  A phase table op just before a pair or triple runs inside its
+ * amplitudes as eight, three real products each: 6, 12 and 24 per quad, octet and 16
+ * values of a component where the rotations one by one take 12, 36 and 96.  A phase
+ * table op just before a pair or triple runs inside its
  * loop.  Results agree with the switch off within the Q60 rounding.  For
  * measurement: on = 1 (default) groups of four, three and two, 4 groups of three
  * and two, 3 pairs only with tables fused, 2 pairs without table fusion, 0
@@ -483,9 +490,10 @@ int qs_expect_pauli(const qs_state* s, const qs_pauli* terms, size_t nterms, dou
  * is the left-to-right prefix of the block totals); the sample is the smallest x
  * with E_b + (left-to-right partial sum of block b up to x) > u_s, or, when no x
  * qualifies, the largest x with p_x > 0.
- * The search within a block starts from the running sum kept after every 32
- * amplitudes (2^n / 32 doubles of stream-ordered scratch, freed when the call
- * returns), which continues the same left-to-right additions.
+ * The search within a block starts from a running sum kept after every 8
+ * amplitudes (every 32 above 27 qubits and below 15; 2^n / 8 or 2^n / 32 doubles of
+ * the state's temporaries, see qs_alloc), which continues the same left-to-right
+ * additions.
  * out[s] (uint64, device or host memory) receives the basis index of shot s. */
 int qs_sample(const qs_state* s, uint64_t seed, uint64_t shots, uint64_t* out, int on_device);
 
@@ -502,8 +510,9 @@ int qs_sample(const qs_state* s, uint64_t seed, uint64_t shots, uint64_t* out, i
  * RX -> X, RY -> Y, RZ -> Z, P and CR -> -2|1><1| on the target, times the
  * projector on the control qubits; a dagger record flips the sign.
  * The state `s` (n qubits) is used as the psi buffer and is overwritten; a
- * second vector and the partial sums are allocated on the state's stream for the
- * call.  Synchronous (returns results in host memory).
+ * second vector and the partial sums are temporaries of the call (see qs_alloc: up
+ * to 256 MiB of them stay with the state, for 23 qubits and less).  Synchronous
+ * (returns results in host memory).
  * Errors: INVALID_ARG (bad record, param_idx >= np, term outside n),
  * UNSUPPORTED (a parametrised record other than RX, RY, RZ, P, CR), OOM, CUDA. */
 int qs_adjoint_grad(qs_state* s, const qs_gate* gates, size_t ng, const double* params, size_t np,
@@ -604,8 +613,10 @@ typedef struct qs_noise_rule {
  * psi <- K_j psi / sqrt(w_j).  Draw k is (SplitMix64 output k of the stream
  * seeded `seed` >> 11) * 2^-53; *ndraws (nullable) receives the count.
  * Stretches without damping-type channels run as one gate list (fused with a
- * greedy plan if fuse != 0); damping-type channels take one reduction pass for
- * their weights.  Synchronous.  Errors: INVALID_ARG (rule, probability,
+ * greedy plan if fuse != 0).  Damping-type channels take their weights from the
+ * joint populations of the qubits that channels touch next, up to 11 of them, read
+ * in one reduction pass; a gate that is not diagonal on one of these qubits, or a
+ * jump, ends the use of that table.  Synchronous.  Errors: INVALID_ARG (rule, probability,
  * decoherence times), the errors of qs_apply. */
 int qs_run_noisy(qs_state* s, const qs_gate* gates, size_t ng, const double* params,
                  const qs_noise_rule* rules, size_t nrules, double rotation_error, uint64_t seed, int fuse,

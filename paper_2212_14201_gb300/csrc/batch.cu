@@ -370,7 +370,9 @@ __device__ void bt_eval_set(const BatchArgs& d, int set_id, int rank, int nr, lo
 // decreasing estimated cost); the item is either one large set shared by the whole
 // cluster or up to d.csize small sets, one per CTA.
 // Two CTAs per SM: a third would leave 80 registers a thread and next to no L1 for what
-// they spill (128 sets of 10..18 qubits: 40.6 ms with three, 29.6 with two).
+// they spill (128 sets of 10..18 qubits: 40.6 ms with three, 29.6 with two).  With 128
+// registers 180 bytes are spilled and 284 reloaded, beside the indexed local arrays of
+// the diagonal groups (a stack of 432 bytes in all).
 __global__ void __launch_bounds__(BT_THREADS, 2) k_batch(const BatchArgs d) {
   extern __shared__ __align__(16) unsigned char smem[];
   longlong2* tP = reinterpret_cast<longlong2*>(smem);

@@ -100,8 +100,9 @@ int check_state(const qs_state* s) {
   return QS_OK;
 }
 
-// Workspace: per-1024-amplitude block sums and prefixes for the sampler (and per
-// superblock of 1024 blocks), plus per-CTA partial results of the reductions.
+// Workspace, by one call at a time: per-1024-amplitude block sums and prefixes of the
+// sampler (and per superblock of 1024 blocks); per-CTA partial results of a reduction;
+// the phase tables of the tile pass being run; the op tables of a backward sweep.
 size_t workspace_bytes(int n) {
   size_t N = (size_t)1 << n;
   size_t L = N < 1024 ? N : 1024;
@@ -109,8 +110,8 @@ size_t workspace_bytes(int n) {
   size_t nsb = nb < 1024 ? 1 : nb / 1024;
   size_t sampler = (2 * (nb + 1) + 2 * (nsb + 1)) * sizeof(double) + (nb + 1 + 2 * (nsb + 1)) * sizeof(long long) + 256;
   size_t reduce = (size_t)1024 * 72 * sizeof(double) + 256;  // up to 1024 CTAs x (n + 2) values
-  size_t hist = (size_t)304 * 4096 * sizeof(double);          // marginal histograms
-  return std::max(sampler, std::max(reduce, hist)) + 4096;
+  size_t tables = (size_t)152 * 4096 * 16;  // 152 phase tables of 4096 entries; more go to a buffer of their own
+  return std::max(sampler, std::max(reduce, tables)) + 4096;
 }
 
 int take_scratch(qs_state* s, size_t bytes, ScratchBuf* out, bool keep) {

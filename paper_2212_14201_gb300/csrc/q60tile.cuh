@@ -209,7 +209,10 @@ static __device__ __noinline__ void bt_perm(longlong2* P, longlong2* Lt, uint32_
 }
 
 // Backward step of a diagonal group in one sweep: per amplitude the members'
-// generator terms (as bt_gen_dgroup) and then E on psi and on lambda.
+// generator terms and then E on psi and on lambda.  With w = Im(conj(l_j) p_j), once per
+// amplitude, a Z member's term is (-1)^bit w and a P member's -2 [bit] w; the members
+// commute with each other and with each other's generators, so every term may be taken
+// before the group runs.
 static __device__ void bt_back_dgroup(longlong2* P, longlong2* Lt, uint32_t TS, const BOp* mem, int nm,
                                       const QC* __restrict__ E, int64_t* out) {
   int tbs[BT_DG_MAX], gens[BT_DG_MAX];
@@ -242,36 +245,6 @@ static __device__ void bt_back_dgroup(longlong2* P, longlong2* Lt, uint32_t TS, 
     Lt[j] = make_longlong2(re, im);
   }
 }
-
-// Generator partials of every member of a diagonal group on the same tiles, in
-// Q60 units: w_j = Im(conj(l_j) p_j) once per amplitude, then per member Z:
-// (-1)^bit w_j, P: -2 [bit] w_j (the members commute with each other and with
-// each other's generators, so every term may be taken before the group runs).
-// Bounds as in bt_gen_partial.
-static __device__ void bt_gen_dgroup(const longlong2* P, const longlong2* Lt, uint32_t TS, const BOp* mem, int nm,
-                                     int64_t* out) {
-  int tbs[BT_DG_MAX], gens[BT_DG_MAX];
-#pragma unroll
-  for (int m = 0; m < BT_DG_MAX; ++m) {
-    out[m] = 0;
-    tbs[m] = m < nm ? mem[m].tb : 0;
-    gens[m] = m < nm ? mem[m].gen : BG_NONE;
-  }
-  for (uint32_t j = threadIdx.x; j < TS; j += BT_THREADS) {
-    const longlong2 p = P[j], l = Lt[j];
-    QAccF acc{0, 0, 0};
-    qaccf_add(acc, q60_split(l.x), q60_split(p.y));
-    qaccf_add(acc, q60_split(-l.y), q60_split(p.x));
-    const int64_t w = qaccf_result(acc);
-#pragma unroll
-    for (int m = 0; m < BT_DG_MAX; ++m) {
-      const bool one = (j >> tbs[m]) & 1u;
-      if (gens[m] == BG_Z) out[m] += one ? -w : w;
-      else if (gens[m] == BG_P && one) out[m] -= 2 * w;
-    }
-  }
-}
-
 
 __device__ __forceinline__ longlong2 bt_unit(longlong2 a, int code) {
   switch (code) {

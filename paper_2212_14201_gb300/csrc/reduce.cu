@@ -307,7 +307,8 @@ __global__ void __launch_bounds__(256) k_marginal_finish(const double* __restric
   if (threadIdx.x == 0) out[blockIdx.x] = s;
 }
 
-// ---- marginal over many qubits: one thread per output entry -----------------------
+// ---- marginal of fewer than 5 qubits, over 4 of them in another order: one thread per
+// output entry (every other marginal has a kernel above) ------------------------------
 struct MargBigArgs {
   uint64_t H;         // 2^nq outputs
   uint64_t R;         // 2^(n-nq) terms per output
@@ -719,7 +720,8 @@ __global__ void __launch_bounds__(256, 3) k_pauli_tile(const A* __restrict__ a, 
 //   sum h h' <= 1.5625 2^60,  sum h l' + l h' < 2^62.9,  sum l l' <= 2^62
 // and join the 128-bit sum once per coordinate and tile: 8 multiply-adds a pair and
 // little else (k_pauli_tile combines and adds 128 bits for every pair, and reads it
-// from shared memory: 540 us for 12 slots at n = 25).
+// from shared memory: 540 us for 12 slots at n = 25, 286 here).  At 128 registers, two
+// CTAs per SM, 88 bytes spill (56 for complex64).
 struct PXArgs {
   uint64_t ntiles;
   int lead[PT_TMAX];
@@ -1180,10 +1182,10 @@ extern "C" int qs_expect_z_all(const qs_state* cs, double* out) {
   return read_back(s, dres, n, out);
 }
 
-// <sum_k coef_k P_k> with the exact passes of k_pauli_exact.  Slots are keyed by
-// (xm, zm, part); X masks are taken two at a time as a cell basis, every other
-// X mask in their span joins that pass, and |a|^2 slots fill the free places
-// (then passes of their own over cells of bits 0 and 1).
+// <sum_k coef_k P_k> by exact integer sums, 16384 terms at a time.  plan_pauli keys the
+// slots by (xm, zm, part) and gathers them into passes over tiles that span their X
+// masks; from 12 qubits on |a|^2 slots run in k_pauli_z and slots of one coordinate
+// without Z in k_pauli_x, and k_pauli_tile takes the rest.
 static int pauli_exact(qs_state* s, const qs_pauli* terms, size_t nterms, double* out) {
   const int n = s->n;
   const size_t kChunk = 16384;  // terms per plan: at most 2 slots each

@@ -211,7 +211,9 @@ __device__ __forceinline__ float2 entry_sign(float2 e, uint32_t odd) {
 struct EngF32 {
   using T = float2;
   using G = float2;
-  static constexpr int kMinBlocks = 4;  // 32 KiB tiles; four per SM leave the 16-amplitude register groups unspilled
+  // 32 KiB tiles, four per SM: 64 registers, of which the groups of 16 amplitudes with
+  // eight table entries in flight spill 88 bytes.
+  static constexpr int kMinBlocks = 4;
   static __device__ __forceinline__ T load(const float2& a) { return a; }
   static __device__ __forceinline__ float2 store(const T& a) { return a; }
   static __device__ __forceinline__ float2 u(const TileOp& op, int e) { return op.f[e]; }
