@@ -1243,37 +1243,78 @@ static int pauli_exact(qs_state* s, const qs_pauli* terms, size_t nterms, double
       gidx[k] = next++;
     };
     // Field slots and |a|^2 slots have kernels of their own wherever a tile of 12
-    // coordinates exists (13-site chain 92 -> 54 us, 25 sites 2.9 -> 1.4 ms).
+    // coordinates exists (13-site chain 92 -> 54 us, 25 sites 2.9 -> 1.4 ms).  A few of
+    // them stay in k_pauli_tile where it runs for other slots anyway: a launch of their
+    // own reads and decodes the state again, 1.4 to 1.6 ms at n = 28, where a field slot
+    // more costs the tile 0.34 ms, the first |a|^2 slots 0.7 and each further one 0.1
+    // (Z + X + XY: three launches 4.91 ms, one 3.30; seven Z + XY 3.66 and 3.55, eight
+    // 3.69 either way; five X + XY 3.80 and 3.65, six 3.91 and 4.0).  Below 19 qubits a
+    // launch more costs 3 us and a slot next to nothing.  One Z and one X alone go
+    // together from 26 qubits on (2.98 and 2.83 ms, complex64 3.19 and 2.84).
     const bool own = n >= 12;
-    if (own) {
-      std::vector<int> zs;
-      for (const auto& P : passes)
-        for (int k : P.sl)
-          if (!slots[k].xm) zs.push_back(k);
-      for (size_t z0 = 0; z0 < zs.size(); z0 += PZ_MAX) {
-        QS_TRY(room());
-        PZArgs g{};
-        g.ntiles = 1ull << (n - 11);
-        g.nt = (int)std::min<size_t>(PZ_MAX, zs.size() - z0);
-        const int nblocks = (int)std::min<uint64_t>(2 * 152, g.ntiles);
-        for (int k = 0; k < g.nt; ++k) {
-          g.zm[k] = slots[zs[z0 + k]].zm;
-          record(zs[z0 + k], k, nblocks, PZ_MAX);
+    const size_t kFewZ = n < 19 ? PS_MAX : 8, kFewX = n < 19 ? PS_MAX : 5;  // (of |a|^2 slots: in the whole sum)
+    struct Split {
+      std::vector<int> x, left;  // field slots for k_pauli_x; slots for k_pauli_tile, in the pass's order
+      std::vector<uint32_t> xc;  // the coordinate of each of x
+    };
+    std::vector<Split> split(passes.size());
+    std::vector<int> zs;
+    size_t nz_all = 0;
+    for (const PauliSlot& sl : slots) nz_all += !sl.xm;
+    for (size_t i = 0; i < passes.size(); ++i) {
+      const auto& P = passes[i];
+      std::vector<uint32_t> coord(P.sl.size(), 0);  // of its field slots
+      size_t nz = 0, nx = 0;
+      for (size_t q = 0; q < P.sl.size() && own; ++q) {
+        const PauliSlot& sl = slots[P.sl[q]];
+        nz += !sl.xm;
+        if (!sl.xm || sl.zm || sl.im) continue;
+        pp_reduce(P.bm, sl.xm, &coord[q]);
+        if (coord[q] & (coord[q] - 1)) coord[q] = 0;
+        nx += coord[q] != 0;
+      }
+      const bool others = nz + nx < P.sl.size();
+      const bool both = n >= 26 && nz == 2 && nz_all == 2 && nx == 1;
+      const bool own_z = own && !((others && nz_all <= kFewZ) || both);
+      const bool own_x = own && !((others && nx <= kFewX) || both);
+      for (size_t q = 0; q < P.sl.size(); ++q) {
+        const int k = P.sl[q];
+        if (!slots[k].xm && own_z) {
+          zs.push_back(k);  // for k_pauli_z
+        } else if (coord[q] && own_x) {
+          split[i].x.push_back(k);
+          split[i].xc.push_back(coord[q]);
+        } else {
+          split[i].left.push_back(k);
         }
-        KTimer kt(s, QS_K_REDUCE, n, g.nt, 0, 0, (double)(1ull << n), 8.0 * g.nt * (double)(1ull << n));
-        with_amps(s, [&](auto* a) {
-          using T = std::remove_cv_t<std::remove_pointer_t<decltype(a)>>;
-          k_pauli_z<T><<<nblocks, 256, 0, s->stream>>>(a, g, part + used);
-          return QS_OK;
-        });
-        QS_TRY(launch_check("pauli_z"));
-        used += (size_t)nblocks * PZ_MAX * 2;
       }
     }
-    for (const auto& P : passes) {
+    for (size_t z0 = 0; z0 < zs.size(); z0 += PZ_MAX) {
+      QS_TRY(room());
+      PZArgs g{};
+      g.ntiles = 1ull << (n - 11);
+      g.nt = (int)std::min<size_t>(PZ_MAX, zs.size() - z0);
+      const int nblocks = (int)std::min<uint64_t>(2 * 152, g.ntiles);
+      for (int k = 0; k < g.nt; ++k) {
+        g.zm[k] = slots[zs[z0 + k]].zm;
+        record(zs[z0 + k], k, nblocks, PZ_MAX);
+      }
+      KTimer kt(s, QS_K_REDUCE, n, g.nt, 0, 0, (double)(1ull << n), 8.0 * g.nt * (double)(1ull << n));
+      with_amps(s, [&](auto* a) {
+        using T = std::remove_cv_t<std::remove_pointer_t<decltype(a)>>;
+        k_pauli_z<T><<<nblocks, 256, 0, s->stream>>>(a, g, part + used);
+        return QS_OK;
+      });
+      QS_TRY(launch_check("pauli_z"));
+      used += (size_t)nblocks * PZ_MAX * 2;
+    }
+    for (size_t i = 0; i < passes.size(); ++i) {
+      const auto& P = passes[i];
+      const std::vector<int>& left = split[i].left;
+      const int nx = (int)split[i].x.size();
+      if (!nx && left.empty()) continue;
       QS_TRY(room());
       PXArgs gx{};
-      int nx = 0;
       PTile g{};
       g.T = (int)P.bm.size();
       g.ntiles = gx.ntiles = 1ull << (n - g.T);
@@ -1282,19 +1323,9 @@ static int pauli_exact(qs_state* s, const qs_pauli* terms, size_t nterms, double
         g.lead[q] = gx.lead[q] = pp_lead(P.bm[q]);
       }
       const int xblocks = (int)std::min<uint64_t>(2 * 152, gx.ntiles);
-      std::vector<int> left;  // slots for k_pauli_tile
-      for (int k : P.sl) {
-        const PauliSlot& sl = slots[k];
-        if (own && !sl.xm) continue;
-        uint32_t xc = 0;
-        if (sl.xm) pp_reduce(P.bm, sl.xm, &xc);
-        if (own && !sl.zm && !sl.im && (xc & (xc - 1)) == 0) {
-          record(k, 31 - __builtin_clz(xc), xblocks, PT_TMAX);
-          ++nx;
-          gx.want |= xc;
-        } else {
-          left.push_back(k);
-        }
+      for (int q = 0; q < nx; ++q) {
+        record(split[i].x[q], 31 - __builtin_clz(split[i].xc[q]), xblocks, PT_TMAX);
+        gx.want |= split[i].xc[q];
       }
       if (nx) {
         KTimer kt(s, QS_K_REDUCE, n, nx, 0, 0, (double)(1ull << n), 8.0 * nx * (double)(1ull << n));
