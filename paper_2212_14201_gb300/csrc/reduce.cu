@@ -1079,7 +1079,9 @@ namespace qs {
 int marginal_host(qs_state* s, const int* qubits, int nq, double* out, bool allow_exact) {
   const size_t bytes = sizeof(double) << nq;
   ScratchBuf tmp;
-  QS_TRY(take_scratch(s, bytes, &tmp, nq < s->n));  // the whole distribution: half a state
+  // (a whole distribution, half a state, is not kept, but for the small ones that a
+  // trajectory reads as tables: an allocation per call takes 40 us)
+  QS_TRY(take_scratch(s, bytes, &tmp, nq < s->n || nq <= 11));
   QS_TRY(marginal_device(s, qubits, nq, (double*)tmp.p, allow_exact));
   cudaError_t e = cudaMemcpyAsync(out, tmp.p, bytes, cudaMemcpyDeviceToHost, s->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
