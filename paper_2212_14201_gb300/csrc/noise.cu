@@ -38,35 +38,48 @@ namespace qs {
 
 // ---- product of real diagonal factors on a few qubits ----------------------------------
 // a_x *= f[key], key = the listed qubits' bits of x.  Moves the state once for all of
-// them; two FP64 products per amplitude (2^22 amplitudes: 17 us at GB300's FP64 rate,
-// about what their bytes take from L2).
+// them.  complex128: two FP64 products per amplitude (2^22 amplitudes: 17 us at GB300's
+// FP64 rate, about what their bytes take from L2).  complex64: the factor as a pair of
+// floats, two FP32 operations a component and one rounding of the exact product, as a
+// double product rounded to float gives it but for ties (the FP64 pipe, conversions
+// included, made a trajectory with one operator a time 1.25 times as long as FP32
+// kernels do: n = 22, decoherence on every U3, 5.7 ms).
 constexpr int JOINT_MAX = 11;
+struct FloatPair {
+  float hi, lo;
+};
+__host__ __device__ inline double scale_factor(double f, double2*) { return f; }
+__host__ __device__ inline FloatPair scale_factor(double f, float2*) {
+  const float hi = (float)f;
+  return FloatPair{hi, (float)(f - (double)hi)};
+}
+template <class A>
+using ScaleFactor = decltype(scale_factor(0.0, (A*)nullptr));
+// CAP: most qubits of a launch.  One operator at a time has a small variant: the
+// arguments of the large one are 16 KB to copy and launch with.
+template <class A, int CAP>
 struct ScaleArgs {
   uint64_t N;
   int nq;
-  int q[JOINT_MAX];
-  double f[1 << JOINT_MAX];
+  int q[CAP];
+  ScaleFactor<A> f[1 << CAP];
 };
 
-__device__ __forceinline__ void scale_amp(double2* p, double f) {
-  const double2 v = *p;
-  *p = make_double2(v.x * f, v.y * f);
-}
-__device__ __forceinline__ void scale_amp(float2* p, double f) {
-  const float2 v = *p;
-  *p = make_float2((float)(v.x * f), (float)(v.y * f));
+__device__ __forceinline__ double2 scale_amp(double2 v, double f) { return make_double2(v.x * f, v.y * f); }
+__device__ __forceinline__ float2 scale_amp(float2 v, FloatPair f) {
+  return make_float2(fmaf(v.x, f.hi, v.x * f.lo), fmaf(v.y, f.hi, v.y * f.lo));
 }
 
-template <class A>
-__global__ void __launch_bounds__(256) k_scale(A* __restrict__ a, const __grid_constant__ ScaleArgs g) {
-  __shared__ double f[1 << JOINT_MAX];
+template <class A, int CAP>
+__global__ void __launch_bounds__(256) k_scale(A* __restrict__ a, const __grid_constant__ ScaleArgs<A, CAP> g) {
+  __shared__ ScaleFactor<A> f[1 << CAP];
   for (int i = threadIdx.x; i < (1 << g.nq); i += 256) f[i] = g.f[i];
   __syncthreads();
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
   auto factor = [&](uint64_t x) {
     uint32_t key = 0;
 #pragma unroll
-    for (int j = 0; j < JOINT_MAX; ++j)
+    for (int j = 0; j < CAP; ++j)
       if (j < g.nq) key |= (uint32_t)((x >> g.q[j]) & 1) << j;
     return f[key];
   };
@@ -76,12 +89,9 @@ __global__ void __launch_bounds__(256) k_scale(A* __restrict__ a, const __grid_c
 #pragma unroll
     for (int k = 0; k < 4; ++k) v[k] = a[x + k * stride];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      scale_amp(&v[k], factor(x + k * stride));
-      a[x + k * stride] = v[k];
-    }
+    for (int k = 0; k < 4; ++k) a[x + k * stride] = scale_amp(v[k], factor(x + k * stride));
   }
-  for (; x < g.N; x += stride) scale_amp(a + x, factor(x));
+  for (; x < g.N; x += stride) a[x] = scale_amp(a[x], factor(x));
 }
 
 // ---- readout error on sampled indices ----------------------------------------------
@@ -234,24 +244,31 @@ struct Trajectory {
     return QS_OK;
   }
 
-  int apply_scales() {
-    if (scales.empty()) return QS_OK;
-    ScaleArgs g;
+  template <int CAP, class A>
+  void launch_scales(A* a) {
+    ScaleArgs<A, CAP> g;
     g.N = 1ull << s->n;
     g.nq = (int)scales.size();
     for (int j = 0; j < g.nq; ++j) g.q[j] = scales[j].q;
     for (int k = 0; k < (1 << g.nq); ++k) {
       double f = 1.0;
       for (int j = 0; j < g.nq; ++j) f *= (k >> j) & 1 ? scales[j].f1 : scales[j].f0;
-      g.f[k] = f;
+      g.f[k] = scale_factor(f, a);
     }
-    scales.clear();
     const int nblocks = (int)std::min<uint64_t>(152 * 8, (g.N + 255) / 256);
-    KTimer kt(s, QS_K_DIAG, 1, g.nq, 0, 0, (double)g.N, 2.0 * (double)g.N);
+    k_scale<A, CAP><<<nblocks, 256, 0, s->stream>>>(a, g);
+  }
+
+  int apply_scales() {
+    if (scales.empty()) return QS_OK;
+    const double N = (double)(1ull << s->n);
+    KTimer kt(s, QS_K_DIAG, 1, (int)scales.size(), 0, 0, N, 2.0 * N);
     with_amps(s, [&](auto* a) {
-      k_scale<<<nblocks, 256, 0, s->stream>>>(a, g);
+      if (scales.size() <= 2) launch_scales<2>(a);
+      else launch_scales<JOINT_MAX>(a);
       return QS_OK;
     });
+    scales.clear();
     return launch_check("scale");
   }
 
