@@ -61,3 +61,20 @@ def test_layers_of_entanglers_share_a_table(q, orc, entangler):
     else:
         # a CNOT moves its target after the table of the gate before was read
         assert max(got) > 1 and len(got) <= 3 * per_layer
+
+
+def test_large_states_read_seven_qubits(q, orc):
+    """From 20 qubits on a narrow table is read with other qubits and folded."""
+    n = 20
+    g = w.pack([w.gate("RY", k, theta=0.3 + 0.1 * k) for k in range(n)] + [w.gate("CZ", 0, 1), w.gate("H", 1)])
+    rules = w.noise_rules([w.noise_rule("DAMPING", "RY", 0.05), w.noise_rule("PHASE_DAMPING", "CZ", 0.05)])
+    ref, nd = orc.run_noisy(n, g, rules, seed=6)
+    h = q.qs_alloc(n)
+    try:
+        q.qs_timing_enable(h, True)
+        assert q.qs_run_noisy(h, g, rules, seed=6) == nd
+        got = [r["k"] for r in q.qs_timing_fetch(h) if r["kind"] == q._lib.K_REDUCE]
+        assert len(got) >= n and set(got) == {7}
+        assert np.max(np.abs(q.qs_get_state(h) - orc.as_complex(ref))) < TOL
+    finally:
+        q.qs_free(h)
